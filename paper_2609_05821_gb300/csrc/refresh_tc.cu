@@ -2,48 +2,53 @@
 // (selective recompute, Conduit Sec. 3.1 / 4.3):
 //   out[l][i][h] = sum_{j <= p_i} softmax_j(<q[l][i][h], K'[l][h/G][j]> / sqrt(d)) V'[l][h/G][j]
 //
-// Work item: one query tile of 128 rows of one (layer, KV head, request),
-// floor(128/G) consecutive selected rows times the G query heads that share
-// the KV head. Keys stream in tiles of 128 (an MMA-issuing thread, which
-// shares its sub-partition with two softmax warps, is paced per instruction,
-// so wide tiles halve its work). The kernel is persistent: one CTA per SM
-// takes items from an atomic counter, and the query tile of the next item
-// loads into a second buffer while the current item computes. Roles (384
-// threads):
-//   warp 0     TMA loads: the query tile of each item (a 3-D box of 64 dims x
-//              G heads x floor(128/G) rows lands in the tile's row order) into
-//              one of two buffers, then its K tiles (two stages); the lanes
-//              issue the copies of a tile together (one per page half when
-//              paged)
-//   warp 10    the same for the V tiles (two stages), so that a V stage
-//              waiting for its P.V never holds back K and the next query tile
-//   warp 1     one thread issues S(t) = Q K(t)^T into TMEM buffer t % 3
-//   warp 11    one thread issues O += P(t) V(t) with P read from TMEM; two
-//              issuing threads, because one thread issuing both (with a wait
-//              for each P.V before the S that reuses its buffer) took longer
-//              per key tile than the softmax
-//   warps 2-9  softmax, two warps per TMEM lane quarter: each thread owns one
-//              row and one half (64 keys) of every key tile. Per tile it reads
-//              its half of S(t), applies the causal mask j <= p_i, exchanges
-//              the half-row max with its partner through shared memory, keeps
-//              a lazy running max (O and the row sum are rescaled only when
-//              the max grows by 2^8; warp-uniform, since tcgen05.ld/st are
-//              warp-collective), writes its half of P as bf16 pairs over the
-//              upper half of S(t), and at the item's end writes its half of
-//              O / rowsum
-// TMEM: three S buffers at columns [0, 384) (P in the upper 64 of each), O at
-// [384, 512). S(t) reuses the buffer of P(t-3), so it is issued once
-// P(t-3) V(t-3) has completed (per-buffer completion barriers): the S thread
-// runs up to two tiles ahead of the softmax, which finds S(t+1) ready when it
-// finishes P(t) and probes for it without suspending; the next item's first
-// S tiles are computed while the softmax writes the previous item's O. Rows
-// are sorted by position, so an item needs
-// keys up to its last row's position only. Every barrier phase follows from
-// per-CTA sequence numbers (items n, key tiles T) that all roles advance
-// alike. Every wait is bounded by one second; a role that gives up raises an
-// abort flag the others watch, the kernel sets CONDUIT_FLAG_TIMEOUT, drains
-// its copies and MMAs, and frees TMEM.
+// Work item: two query tiles A and B of 128 rows of one (layer, KV head,
+// request), each floor(128/G) consecutive selected rows times the G query
+// heads that share the KV head; B holds the later rows. Keys stream in tiles
+// of 128, and every K and V tile serves both query tiles: an SM takes at most
+// about 39 bytes per clock from L2 by bulk copies (measured, whatever is in
+// flight), so one query tile per 64 KB of K and V cannot run faster than about
+// 1 700 cycles per tile, and two share that. The kernel is persistent: one CTA
+// per SM takes items from an atomic counter. Roles (384 threads):
+//   warp 0      takes and decodes the items (record and row positions in
+//               shared memory, one item ahead) and loads the K tiles
+//   warp 2      loads the V tiles
+//   warps 1, 3  the query tile and the MMAs of A and of B. The whole warp walks
+//               the schedule on uniform values and one lane issues: beside the
+//               softmax warps that keeps an MMA at its 64 tensor cycles, where
+//               one lane of a diverged warp needs 83
+//   warps 4-7   softmax of tile A, warps 8-11 of tile B: each thread owns one
+//               row (TMEM lane) and all 128 keys of a key tile. It reads S(t),
+//               applies the causal mask j <= p_i, keeps a lazy running max (O
+//               and the row sum are rescaled only when the max grows by 2^8;
+//               warp-uniform, since tcgen05.ld/st are warp-collective), writes
+//               P as bf16 pairs over the upper half of S(t), and at the item's
+//               end writes its row of O / rowsum.
+// A turn of an MMA warp is P_x(t) V(t) and then S_x(t+1); the warps take turns
+// strictly, so the two tiles stay half a period apart and one tile's softmax
+// runs beside the other's MMAs (without turns both softmaxes fall into step:
+// 1.1 x slower). MMAs of one thread execute in issue order, so S_x(t+1) may
+// overwrite P_x(t) without a wait, and S_x(t+1) ready implies that P_x(t) V(t)
+// has completed (the softmax may then rescale O_x).
+// TMEM: S_A, S_B at columns [0, 256), O_A, O_B at [256, 512).
+//
+// Measured (GB300, SM clock 2 070 MHz, against one query tile per item with
+// three S buffers): multi-image prompt 1 253 -> 945 us, batched serving 22.6 ->
+// 18.6 ms, long document 15.2 -> 15.0 ms (17.0 -> 16.3 ms back to back, under
+// the power cap). What bounds it: the chain softmax (about 1 150 cycles for 128
+// keys a thread) -> P V -> next S of a tile, about 3 000 cycles per pair of
+// tiles against 2 048 of tensor work. About 10 % of the multi-image gain is that
+// rows a box leaves empty (G not a power of two) no longer take the masking
+// path.
+//
+// Rows are sorted by position, so an item needs keys up to its last row's
+// position only (tile A often fewer than tile B). Every barrier phase follows
+// from per-CTA sequence numbers that all roles advance alike. Every wait is
+// bounded by one second; a role that gives up raises an abort flag the others
+// watch, the kernel sets CONDUIT_FLAG_TIMEOUT, drains its copies and MMAs, and
+// frees TMEM.
 #include <cuda.h>
+#include <limits.h>
 
 #include "internal.cuh"
 #include "tc_common.cuh"
@@ -51,52 +56,60 @@
 namespace conduit {
 namespace {
 
-constexpr int kD = 128;
+constexpr int kMaxD = 128;
 constexpr int kKT = 128;                         // keys per tile
 constexpr int kRows = 128;                       // rows per query tile
-constexpr int kSoftThreads = 256;
-constexpr int kVWarp = 10;                       // after the loader, MMA and eight softmax warps
-constexpr int kPvWarp = 11;                      // the thread issuing O += P V
-constexpr int kThreads = 64 + kSoftThreads + 64;
-constexpr int kKStages = 2;
-constexpr int kVStages = 2;
-constexpr int kQBufs = 2;
-constexpr uint32_t kQHalf = kRows * 128;         // 16 KB: one 64-dim half of the query tile
-constexpr uint32_t kQBytes = 2 * kQHalf;         // 32 KB
-constexpr uint32_t kTileHalf = kKT * 128;        // 16 KB: one 64-dim half of a K or V tile
-constexpr uint32_t kTileBytes = 2 * kTileHalf;   // 32 KB
-constexpr int kRecInts = 9;                      // decoded item record (see Smem::rec)
-constexpr uint32_t kSmem = 1024 + kQBufs * kQBytes + (kKStages + kVStages) * kTileBytes + 256 +
-                           2 * 2 * 128 * 4 + 2 * 128 * 4 + kQBufs * (kRecInts + kRows) * 4;
-constexpr uint32_t kTmemCols = 512;              // three S / P buffers and O
+constexpr int kMmaWarp = 1, kVWarp = 2, kSoftWarp0 = 4;  // warp 0: items and K; warps 1, 3: MMAs
+constexpr int kThreads = 384;
+constexpr uint32_t kHalfBytes = 128 * 128;       // 16 KB: one 64-dim half of a 128-row tile
+constexpr int kRecReaders = 11;                  // two MMA warps, V warp, eight softmax warps
+constexpr uint32_t kTailBytes = 256 + 2 * (16 + 2 * kRows) * 4;
+
+// Head sizes: kHalves 64-dim halves of a row (one 128-byte swizzled row each;
+// a smaller head_dim is padded with zeros by the copies).
+template <int kHalves>
+struct Shape {
+  static constexpr uint32_t kTileBytes = kHalves * kHalfBytes;
+  // K and V tiles in one ring, K(0) V(0) K(1) V(1) ...: tile T may be loaded
+  // once tile T - kAhead is done, and fewer than kDone tiles are undecided
+  static constexpr int kStages = kHalves == 1 ? 9 : 5;
+  static constexpr int kAhead = (kStages - 1) / 2;
+  static constexpr int kDone = 2 * kAhead;
+  static constexpr uint32_t kSmem = (2 + kStages) * kTileBytes + kTailBytes;
+  static_assert(kSmem <= 232448, "shared memory of one CTA");
+  static_assert((kStages + kDone + 6 + 4 + 4 + 2) * 8 + 32 <= 256, "barriers and counters");
+};
+constexpr uint32_t kTmemCols = 512;
 constexpr uint32_t kSCols = 128;                 // one S buffer
-constexpr int kSBufs = 3;                        // S runs up to two key tiles ahead of the softmax
-constexpr uint32_t kPCol = 64;                   // P (bf16 pairs) over the upper half of S
-constexpr uint32_t kOCol = kSBufs * kSCols;      // O
+constexpr uint32_t kPCol = 64;                   // P (bf16 pairs) over the upper half of S ...
+constexpr uint32_t kPLoCol = 0;                  // ... and its rounding errors over the lower one (kSplit)
+constexpr uint32_t kOCol = 2 * kSCols;           // O_A, then O_B
 constexpr float kRescaleLog2 = 8.f;
+constexpr int kPassEarly = 2;                    // MMAs of a turn still to issue when the other stream's may start
 
 struct RefArgs {
   KvDev kv;
   BatchDev b;
   const int32_t* idx;
   const int32_t* idx_off;
-  const __nv_bfloat16* q_rows;
   __nv_bfloat16* out;
   int32_t out32;           // out is 32-byte aligned: rows are written in 32-byte stores
   int32_t n_sel;
   int32_t rows_per_tile;   // selected rows per query tile, floor(128 / G)
-  int32_t n_blocks;        // query tiles per (layer, KV head)
+  int32_t n_blocks;        // items per (layer, KV head)
   int32_t n_items;         // n_blocks * Hkv * L
-  int32_t blocks_major;    // item order: query tile (largest first) outer, or (layer, head) outer
+  int32_t blocks_major;    // item order: block (largest first) outer, or (layer, head) outer
   int32_t* next_item;      // work counter, zero at launch
   float scale_log2;
   int32_t* status;
 };
 
-// A work item: query tile `blk` of (layer l, KV head g), counted from the
-// largest positions, and the request, first selected row and row count.
+// A work item: block `blk` of (layer l, KV head g), counted from the largest
+// positions, and the request, first selected row and row count. A request's
+// blocks are cut from its last row down, so only the block of its smallest
+// positions may hold fewer than two query tiles.
 // Every layer and head of a request has the same selected positions, so the
-// blocks-major order (all (layer, head) pairs of the largest tile first) is
+// blocks-major order (all (layer, head) pairs of the largest block first) is
 // longest-first scheduling; the (layer, head)-major order keeps the CTAs in
 // flight on few K/V prefixes, which L2 then shares when the cache exceeds it.
 struct Item {
@@ -112,16 +125,17 @@ __device__ __forceinline__ Item decode_item(const RefArgs& a, int u) {
   it.l = lg / a.kv.Hkv;
   int blk = a.n_blocks - 1 - x;
   it.r = 0;
-  it.i0 = -1;
+  it.i0 = 0;
   it.cnt = 0;
-  const int span = a.rows_per_tile;
+  const int span = 2 * a.rows_per_tile;
   for (int rr = 0; rr < a.b.R; ++rr) {
     const int k0 = a.idx_off[rr], kr = a.idx_off[rr + 1] - k0;
     const int nb = (kr + span - 1) / span;
     if (blk < nb) {
+      const int end = kr - (nb - 1 - blk) * span, begin = max(0, end - span);
       it.r = rr;
-      it.i0 = k0 + blk * span;
-      it.cnt = min(span, kr - blk * span);
+      it.i0 = k0 + begin;
+      it.cnt = end - begin;
       break;
     }
     blk -= nb;
@@ -129,81 +143,52 @@ __device__ __forceinline__ Item decode_item(const RefArgs& a, int u) {
   return it;
 }
 
-// Key tiles of an item: up to its last row's position.
-__device__ __forceinline__ int item_tiles(const RefArgs& a, const Item& it) {
-  if (it.i0 < 0) return 0;
-  const int N = a.b.tok_off[it.r + 1] - a.b.tok_off[it.r];
-  const int p_max = min(a.idx[it.i0 + it.cnt - 1], N - 1);
-  return p_max < 0 ? 0 : p_max / kKT + 1;
-}
-
 struct Smem {
-  uint8_t* q;        // [kQBufs][2 halves][128 rows][128 B]
-  uint8_t* k;        // [kKStages][2 halves][128 keys][128 B]
-  uint8_t* v;        // [kVStages][2 halves][128 keys][128 B]
-  uint64_t *kfull, *kempty;   // [kKStages]
-  uint64_t *vfull, *vempty;   // [kVStages]
-  uint64_t *sfull, *pfull;    // [kSBufs] per S buffer
-  uint64_t *pvdone;           // [kSBufs] per S buffer: the P.V that read its P has completed
-  uint64_t *qfull, *qempty;   // [kQBufs] query tile (and item index) of one item
-  uint64_t *ofull, *oempty;   // once per item: O complete / O read out
-  uint64_t *mdone;            // [2] per MMA thread: all its MMAs completed
+  uint8_t* q;        // [2 tiles][halves][128 rows][128 B]
+  uint8_t* kv;       // [kStages][halves][128 keys][128 B]: K tile t of the CTA in slot 2t mod kStages, V in 2t + 1
+  uint64_t* full;             // [kStages]
+  uint64_t* done;             // [kDone] tile T of the CTA: K(T) and V(T - 1) have been used
+  uint64_t *sfull, *pfull;    // [2] per query tile: S computed / P written
+  uint64_t *ofull;            // [2] per query tile, once per item that has rows in it: O complete
+  uint64_t* qfull;            // [2] per query tile
+  uint64_t* turn;             // [2] the stream's MMA warp may issue its next turn
+  uint64_t *recfull, *recempty;  // [2] item records
+  uint64_t* mdone;            // [2] per MMA warp: all its MMAs completed
   uint32_t* tmem_slot;
   volatile int* abort;
-  uint32_t* counters;  // [0] K loads, [1] V loads, [2] K consumed, [3] V consumed
-  float* xmax;         // [2 tile parities][2 halves][128 rows] half-row maxima
-  float* xsum;         // [2 halves][128 rows] half-row sums at the end
-  // per query buffer, written by the loader with the query tile: the decoded
-  // item {u (-1: no more work), l, g, r, i0, cnt, key tiles, N_r, t0} and the
-  // positions of its selected rows, so the other roles read no global memory
-  // between items
-  volatile int* rec;   // [kQBufs][kRecInts]
-  volatile int* pos;   // [kQBufs][kRows]
+  uint32_t* counters;  // [0] K tiles, [1] V tiles loaded
+  // per item parity, written by the loader: the decoded item {u (-1: no more
+  // work), l, g, r, i0, rows of A, rows of B, key tiles of A, of B, N_r, t0}
+  // and the positions of its selected rows, so that the other roles read no
+  // global memory between items
+  volatile int* rec;   // [2][16]
+  volatile int* pos;   // [2][2 tiles][kRows]
 };
 
-__device__ __forceinline__ Smem carve(uint8_t* raw) {
-  uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(raw) + 1023) & ~uintptr_t(1023));
+template <int kHalves>
+__device__ __forceinline__ Smem carve(uint8_t* base) {
+  using C = Shape<kHalves>;
   Smem s;
   s.q = base;
-  s.k = s.q + kQBufs * kQBytes;
-  s.v = s.k + kKStages * kTileBytes;
-  uint64_t* bar = reinterpret_cast<uint64_t*>(s.v + kVStages * kTileBytes);
-  s.kfull = bar;
-  s.kempty = s.kfull + kKStages;
-  s.vfull = s.kempty + kKStages;
-  s.vempty = s.vfull + kVStages;
-  s.sfull = s.vempty + kVStages;
-  s.pfull = s.sfull + kSBufs;
-  s.pvdone = s.pfull + kSBufs;
-  s.qfull = s.pvdone + kSBufs;
-  s.qempty = s.qfull + kQBufs;
-  s.ofull = s.qempty + kQBufs;
-  s.oempty = s.ofull + 1;
-  s.mdone = s.oempty + 1;
+  s.kv = s.q + 2 * C::kTileBytes;
+  uint64_t* bar = reinterpret_cast<uint64_t*>(s.kv + C::kStages * C::kTileBytes);
+  s.full = bar;
+  s.done = s.full + C::kStages;
+  s.sfull = s.done + C::kDone;
+  s.pfull = s.sfull + 2;
+  s.ofull = s.pfull + 2;
+  s.qfull = s.ofull + 2;
+  s.turn = s.qfull + 2;
+  s.recfull = s.turn + 2;
+  s.recempty = s.recfull + 2;
+  s.mdone = s.recempty + 2;
   s.tmem_slot = reinterpret_cast<uint32_t*>(s.mdone + 2);
   s.abort = reinterpret_cast<volatile int*>(s.tmem_slot + 1);
   s.counters = reinterpret_cast<uint32_t*>(s.tmem_slot + 2);
-  s.xmax = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(bar) + 256);
-  s.xsum = s.xmax + 2 * 2 * 128;
-  s.rec = reinterpret_cast<volatile int*>(s.xsum + 2 * 128);
-  s.pos = s.rec + kQBufs * kRecInts;
+  s.rec = reinterpret_cast<volatile int*>(reinterpret_cast<uint8_t*>(bar) + 256);
+  s.pos = s.rec + 2 * 16;
   return s;
 }
-
-// Non-blocking test of the phase with the given parity (no suspension): for
-// the softmax's wait on S, which the S thread has usually completed already.
-// Waits that are often not yet complete (the MMA threads') use wait_or_abort
-// alone: a probe in front of them cost more than it saved.
-__device__ __forceinline__ bool mbar_probe(uint64_t* bar, uint32_t parity) {
-  uint32_t done;
-  asm volatile(
-      "{\n.reg .pred p;\nmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}\n"
-      : "=r"(done)
-      : "r"(tc::smem_u32(bar)), "r"(parity)
-      : "memory");
-  return done != 0;
-}
-
 __device__ __forceinline__ bool wait_or_abort(uint64_t* bar, uint32_t parity, volatile int* abort) {
   if (tc::mbar_try_wait(bar, parity)) return true;
   const uint64_t t0 = tc::globaltimer_ns();
@@ -214,6 +199,14 @@ __device__ __forceinline__ bool wait_or_abort(uint64_t* bar, uint32_t parity, vo
   return false;
 }
 
+// The same for a converged warp. The first test is a plain probe by all lanes,
+// which costs about 75 cycles when the phase is complete (a suspending
+// try_wait about 100, one lane's wait shared with the others about 250).
+__device__ __forceinline__ bool wait_warp(uint64_t* bar, uint32_t parity, volatile int* abort) {
+  if (__all_sync(0xffffffffu, tc::mbar_probe(bar, parity))) return true;
+  return __all_sync(0xffffffffu, wait_or_abort(bar, parity, abort));
+}
+
 __device__ __forceinline__ void raise_abort(const RefArgs& a, const Smem& s, int32_t site) {
   if (!*s.abort) flag_status(a.status, CONDUIT_FLAG_TIMEOUT | site);
   *s.abort = 1;
@@ -221,95 +214,91 @@ __device__ __forceinline__ void raise_abort(const RefArgs& a, const Smem& s, int
 
 // Warp-cooperative TMA of the 128-key tile starting at request-local key j0:
 // lane 0 posts the byte count, then copy c is issued by lane c. A copy is one
-// 64-dim half of the whole tile (contiguous cache: 2 copies) or of one page
-// (paged cache: 2 x 128/page copies, up to 32), so a paged tile costs one
+// 64-dim half of the whole tile (contiguous cache) or of one page (paged
+// cache: 128/page copies per half, up to 32), so a paged tile costs one
 // round of parallel page-index loads and copy issues instead of a serial loop.
+template <int kHalves>
 __device__ __forceinline__ void load_tile(const RefArgs& a, const CUtensorMap* map, uint8_t* dst,
                                           uint64_t* bar, int l, int g, int r, int t0, int N, int j0,
                                           int lane) {
   const KvDev& kv = a.kv;
-  if (lane == 0) tc::mbar_arrive_expect_tx(bar, kTileBytes);
+  if (lane == 0) tc::mbar_arrive_expect_tx(bar, kHalves * kHalfBytes);
   __syncwarp();
-  const int hf = lane & 1;
+  const int hf = lane % kHalves;
   if (kv.page_size == 0) {
-    if (lane < 2) {
+    if (lane < kHalves) {
       const int32_t y = int32_t((int64_t(l) * kv.Hkv + g) * kv.n_tot + t0 + j0);
-      tc::tma_load_2d(dst + hf * kTileHalf, map, bar, hf * 64, y);
+      tc::tma_load_2d(dst + hf * kHalfBytes, map, bar, hf * 64, y);
     }
   } else {
     const int ps = kv.page_size;
-    const int i = lane >> 1;  // page of the tile
+    const int i = lane / kHalves;  // page of the tile
     if (i < kKT / ps) {
       const int lp = min((j0 + i * ps) / ps, (N - 1) / ps);  // tail pages repeat the last one (masked)
       const int page = kv.page_table[int64_t(r) * kv.max_pages + lp];
       const int32_t y = int32_t(((int64_t(l) * kv.num_pages + page) * kv.Hkv + g) * ps);
-      tc::tma_load_2d(dst + hf * kTileHalf + i * ps * 128, map, bar, hf * 64, y);
+      tc::tma_load_2d(dst + hf * kHalfBytes + i * ps * 128, map, bar, hf * 64, y);
     }
   }
 }
 
-// Agreement of the 256 softmax threads (named barrier 1 with an AND
-// reduction): every thread arrives, so all of them take the same branch.
-__device__ __forceinline__ bool softmax_all(bool pred) {
-  uint32_t out;
-  asm volatile(
-      "{\n.reg .pred pi, po;\nsetp.ne.u32 pi, %1, 0;\nbar.red.and.pred po, 1, %2, pi;\nselp.u32 %0, 1, 0, po;\n}\n"
-      : "=r"(out)
-      : "r"(uint32_t(pred)), "n"(kSoftThreads)
-      : "memory");
-  return out != 0;
-}
-
+// kSplit: P goes to the tensor cores as two bf16 tiles (value and rounding
+// error), which keeps it as precise as fp32 weights for a bf16 result.
+template <int kHalves, bool kSplit>
 __global__ void __launch_bounds__(kThreads, 1)
     refresh_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant__ CUtensorMap vmap,
                       const __grid_constant__ CUtensorMap qmap, const __grid_constant__ RefArgs a) {
-  extern __shared__ uint8_t smem_raw[];
-  const Smem s = carve(smem_raw);
+  extern __shared__ __align__(1024) uint8_t smem_raw[];
+  using C = Shape<kHalves>;
+  constexpr int kStages = C::kStages, kAhead = C::kAhead, kDone = C::kDone, kDP = 64 * kHalves;
+  constexpr uint32_t kTileBytes = C::kTileBytes;
+  const Smem s = carve<kHalves>(smem_raw);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const KvDev& kv = a.kv;
   const int G = kv.G, Hq = kv.Hq;
-  const int qrows = a.rows_per_tile * G;          // rows the query box fills
+  const int d = kHalves == 2 && !kSplit ? kMaxD : kv.d;
+  const int span = a.rows_per_tile;               // selected rows of a query tile
+  if (tc::smem_u32(smem_raw) & 1023u) {           // the swizzled tiles need 1024-byte atoms
+    if (tid == 0) flag_status(a.status, CONDUIT_FLAG_TIMEOUT | tc::kSiteLoad);
+    return;
+  }
 
   if (tid == 0) {
-    for (int i = 0; i < kKStages; ++i) {
-      tc::mbar_init(&s.kfull[i], 1);
-      tc::mbar_init(&s.kempty[i], 1);
-    }
-    for (int i = 0; i < kVStages; ++i) {
-      tc::mbar_init(&s.vfull[i], 1);
-      tc::mbar_init(&s.vempty[i], 1);
-    }
-    for (int i = 0; i < kSBufs; ++i) {
+    for (int i = 0; i < kStages; ++i) tc::mbar_init(&s.full[i], 1);
+    for (int i = 0; i < kDone; ++i) tc::mbar_init(&s.done[i], 1);
+    for (int i = 0; i < 2; ++i) {
       tc::mbar_init(&s.sfull[i], 1);
-      // per buffer, so the softmax can never be two phases ahead of the MMA's
-      // wait: P(t+3) needs S(t+3), issued only after P(t) V(t) has completed
-      tc::mbar_init(&s.pfull[i], kSoftThreads);
-      tc::mbar_init(&s.pvdone[i], 1);
+      tc::mbar_init(&s.pfull[i], 4);     // one arrival per softmax warp of the tile
+      tc::mbar_init(&s.ofull[i], 1);
+      tc::mbar_init(&s.qfull[i], 1);
+      tc::mbar_init(&s.turn[i], 1);
+      tc::mbar_init(&s.mdone[i], 1);
+      tc::mbar_init(&s.recfull[i], 1);
+      tc::mbar_init(&s.recempty[i], kRecReaders);
     }
-    for (int i = 0; i < kQBufs; ++i) {
-      tc::mbar_init(&s.qfull[i], 1);   // the loader's expect-tx (or plain arrive at the end)
-      // the S thread's commit + the P.V thread's, softmax's and V warp's reads of the item
-      tc::mbar_init(&s.qempty[i], 4);
-    }
-    tc::mbar_init(s.ofull, 1);
-    tc::mbar_init(s.oempty, kSoftThreads);
-    tc::mbar_init(&s.mdone[0], 1);
-    tc::mbar_init(&s.mdone[1], 1);
     *s.abort = 0;
-    for (int i = 0; i < 4; ++i) s.counters[i] = 0;
+    s.counters[0] = s.counters[1] = 0;
     tc::fence_barrier_init();
     tc::prefetch_tensormap(&kmap);
     tc::prefetch_tensormap(&vmap);
     tc::prefetch_tensormap(&qmap);
   }
-  if (warp == 1) tc::tmem_alloc(s.tmem_slot, kTmemCols);
+  if (warp == kMmaWarp) tc::tmem_alloc(s.tmem_slot, kTmemCols);
+  // query rows the boxes never fill: zero, so their logits are finite
+  for (uint32_t i = span * G * 128 + tid * 16; i < kHalfBytes; i += kThreads * 16)
+    for (int h = 0; h < 2 * kHalves; ++h) *reinterpret_cast<uint4*>(s.q + h * kHalfBytes + i) = make_uint4(0, 0, 0, 0);
+  tc::fence_proxy_async_smem();
   __syncthreads();
   tc::tc_fence_after();
   const uint32_t tmem = *s.tmem_slot;
 
+  // Registers: a softmax thread holds a row of S (128 values). The shares add
+  // up to 128 x 88 + 256 x 208 = 384 x 168, what the launch has.
+  if (warp < kSoftWarp0) {
+  asm volatile("setmaxnreg.dec.sync.aligned.u32 88;" ::: "memory");
   if (warp == 0) {
-    // ------------------------------------------------------- loads (warp 0)
-    uint32_t nk = 0, T = 0;
+    // ------------------------------------------------ items and K (warp 0)
+    uint32_t T = 0;
     bool ok = true;
     for (uint32_t n = 0; ok; ++n) {
       int u = 0;
@@ -319,347 +308,336 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
       u = __shfl_sync(0xffffffffu, u, 0);
       const Item it = decode_item(a, u < 0 ? 0 : u);
-      const int nt = u < 0 ? 0 : item_tiles(a, it);
+      const int cnt_b = min(it.cnt, span), cnt_a = it.cnt - cnt_b;
       const int t0 = a.b.tok_off[it.r], N = a.b.tok_off[it.r + 1] - t0;
-      int my_pos[kRows / 32];  // positions of the item's rows, loaded before the buffer is free
+      int my_pos[2 * kRows / 32];  // positions of the item's rows, loaded before the record is free
 #pragma unroll
-      for (int k = 0; k < kRows / 32; ++k) {
-        const int i = lane + 32 * k;
-        my_pos[k] = (u >= 0 && i < it.cnt) ? a.idx[it.i0 + i] : -1;
+      for (int k = 0; k < 2 * kRows / 32; ++k) {
+        const int x = k / (kRows / 32), i = lane + 32 * (k % (kRows / 32));
+        my_pos[k] = (u >= 0 && i < (x ? cnt_b : cnt_a)) ? a.idx[it.i0 + (x ? cnt_a : 0) + i] : -1;
       }
-      const int qs = n & 1;
-      if (!__all_sync(0xffffffffu, wait_or_abort(&s.qempty[qs], ((n >> 1) & 1) ^ 1, s.abort))) {
+      auto key_tiles = [&](int first, int cnt) {  // up to the last row's position
+        if (u < 0 || cnt == 0) return 0;
+        const int p = min(a.idx[it.i0 + first + cnt - 1], N - 1);
+        return p < 0 ? 0 : p / kKT + 1;
+      };
+      int nt_a = key_tiles(0, cnt_a), nt = key_tiles(cnt_a, cnt_b);
+      nt_a = min(nt_a, nt);  // idx ascends, so this changes nothing unless the caller broke that
+      const int rs = n & 1;
+      if (!wait_warp(&s.recempty[rs], ((n >> 1) & 1) ^ 1, s.abort)) {
         if (lane == 0) raise_abort(a, s, tc::kSiteLoad);
         break;
       }
 #pragma unroll
-      for (int k = 0; k < kRows / 32; ++k) s.pos[qs * kRows + lane + 32 * k] = my_pos[k];
+      for (int k = 0; k < 2 * kRows / 32; ++k) s.pos[rs * 2 * kRows + lane + 32 * k] = my_pos[k];
       if (lane == 0) {
-        volatile int* rec = s.rec + qs * kRecInts;
+        volatile int* rec = s.rec + rs * 16;
         rec[0] = u;
         rec[1] = it.l;
         rec[2] = it.g;
         rec[3] = it.r;
         rec[4] = it.i0;
-        rec[5] = it.cnt;
-        rec[6] = nt;
-        rec[7] = N;
-        rec[8] = t0;
+        rec[5] = cnt_a;
+        rec[6] = cnt_b;
+        rec[7] = nt_a;
+        rec[8] = nt;
+        rec[9] = N;
+        rec[10] = t0;
       }
       __threadfence_block();
       __syncwarp();  // the lanes' positions are ordered before lane 0's release below
-      if (lane == 0) {
-        if (u < 0) {
-          tc::mbar_arrive(&s.qfull[qs]);  // no more work: the others stop at this buffer
-        } else {
-          tc::mbar_arrive_expect_tx(&s.qfull[qs], 2u * 128u * uint32_t(qrows));
-          for (int hf = 0; hf < 2; ++hf)
-            tc::tma_load_3d(s.q + qs * kQBytes + hf * kQHalf, &qmap, &s.qfull[qs], hf * 64,
-                            it.g * G, it.l * a.n_sel + max(it.i0, 0));
-        }
-      }
+      if (lane == 0) tc::mbar_arrive(&s.recfull[rs]);
       if (u < 0) break;
       for (int t = 0; t < nt; ++t, ++T) {
-        const int sk = T % kKStages;
-        if (!__all_sync(0xffffffffu, wait_or_abort(&s.kempty[sk], ((T / kKStages) & 1) ^ 1, s.abort))) {
+        const uint32_t sl = 2 * T % kStages;
+        if (T >= kAhead && !wait_warp(&s.done[(T - kAhead) % kDone], ((T - kAhead) / kDone) & 1, s.abort)) {
           if (lane == 0) raise_abort(a, s, tc::kSiteLoad);
           ok = false;
           break;
         }
-        load_tile(a, &kmap, s.k + sk * kTileBytes, &s.kfull[sk], it.l, it.g, it.r, t0, N, t * kKT, lane);
-        ++nk;
+        load_tile<kHalves>(a, &kmap, s.kv + sl * kTileBytes, &s.full[sl], it.l, it.g, it.r, t0, N, t * kKT, lane);
       }
     }
-    if (lane == 0) s.counters[0] = nk;
+    if (lane == 0) s.counters[0] = T;
   } else if (warp == kVWarp) {
-    // --------------------------------------------------- V loads (warp 10)
-    // on a warp of their own: a V stage frees only once its P.V has
-    // completed, and waiting for it must not hold back the K tiles and the
-    // next item's query tile
-    uint32_t nv = 0, T = 0;
-    for (uint32_t n = 0;; ++n) {
-      const int qs = n & 1;
-      if (!__all_sync(0xffffffffu, wait_or_abort(&s.qfull[qs], (n >> 1) & 1, s.abort))) {
+    // ----------------------------------------------------- V loads (warp 2)
+    uint32_t T = 0;
+    bool ok = true;
+    for (uint32_t n = 0; ok; ++n) {
+      const int rs = n & 1;
+      if (!wait_warp(&s.recfull[rs], (n >> 1) & 1, s.abort)) {
         if (lane == 0) raise_abort(a, s, tc::kSiteLoad);
         break;
       }
-      const volatile int* rec = s.rec + qs * kRecInts;
-      const int u = rec[0], l = rec[1], g = rec[2], r = rec[3], nt = rec[6], N = rec[7], t0 = rec[8];
+      const volatile int* rec = s.rec + rs * 16;
+      const int u = rec[0], l = rec[1], g = rec[2], r = rec[3], nt = rec[8], N = rec[9], t0 = rec[10];
       __syncwarp();
-      if (lane == 0) tc::mbar_arrive(&s.qempty[qs]);  // this warp is done with the record
+      if (lane == 0) tc::mbar_arrive(&s.recempty[rs]);  // this warp is done with the record
       if (u < 0) break;
-      bool ok = true;
       for (int t = 0; t < nt; ++t, ++T) {
-        const int sv = T % kVStages;
-        if (!__all_sync(0xffffffffu, wait_or_abort(&s.vempty[sv], ((T / kVStages) & 1) ^ 1, s.abort))) {
+        const uint32_t sl = (2 * T + 1) % kStages;
+        if (T >= kAhead && !wait_warp(&s.done[(T - kAhead) % kDone], ((T - kAhead) / kDone) & 1, s.abort)) {
           if (lane == 0) raise_abort(a, s, tc::kSiteLoad);
           ok = false;
           break;
         }
-        load_tile(a, &vmap, s.v + sv * kTileBytes, &s.vfull[sv], l, g, r, t0, N, t * kKT, lane);
-        ++nv;
+        load_tile<kHalves>(a, &vmap, s.kv + sl * kTileBytes, &s.full[sl], l, g, r, t0, N, t * kKT, lane);
+      }
+    }
+    if (lane == 0) s.counters[1] = T;
+  } else {
+    // --------------------------- query tile and MMAs of one stream (warps 1, 3)
+    // the whole warp walks the schedule on uniform values, one lane issues
+    const int x = __shfl_sync(0xffffffffu, warp == kMmaWarp ? 0 : 1, 0);
+    const uint32_t leader = lane == 0;
+    uint32_t T = 0, turn = 0, np = 0, nq = 0, cq = 0;  // tiles, turns, P tiles, query tiles loaded / consumed
+    const uint32_t idesc_s = tc::idesc_bf16(kRows, kKT);
+    const uint32_t idesc_o = tc::idesc_bf16(kRows, kDP, /*b_mn_major=*/true);
+    const uint32_t kv_addr = tc::smem_u32(s.kv);
+    const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
+    const uint32_t s_col = tm + x * kSCols, o_col = tm + kOCol + x * kDP;
+    const uint64_t dq = tc::desc_sw128(tc::smem_u32(s.q) + x * kTileBytes);
+    bool ok = true;
+    auto load_q = [&](const volatile int* rec) {
+      if (rec[0] < 0 || rec[7 + x] == 0) return;
+      if (lane == 0) {
+        uint8_t* dst = s.q + x * kTileBytes;
+        tc::mbar_arrive_expect_tx(&s.qfull[x], uint32_t(kHalves) * 128u * uint32_t(span * G));
+        for (int hf = 0; hf < kHalves; ++hf)
+          tc::tma_load_3d(dst + hf * kHalfBytes, &qmap, &s.qfull[x], hf * 64, rec[2] * G,
+                          rec[1] * a.n_sel + rec[4] + (x ? rec[5] : 0));
+      }
+      __syncwarp();
+      ++nq;
+    };
+    for (uint32_t n = 0;; ++n) {
+      if (!(ok = wait_warp(&s.recfull[n & 1], (n >> 1) & 1, s.abort))) break;
+      const volatile int* rec = s.rec + (n & 1) * 16;
+      if (n == 0) load_q(rec);
+      const int u = __shfl_sync(0xffffffffu, rec[0], 0), nt_x = __shfl_sync(0xffffffffu, rec[7 + x], 0),
+                nt = __shfl_sync(0xffffffffu, rec[8], 0);
+      __syncwarp();
+      tc::mbar_arrive_if(leader, &s.recempty[n & 1]);
+      if (u < 0) break;
+      if (nt_x > 0) {
+        if (!(ok = wait_warp(&s.qfull[x], cq & 1, s.abort))) break;
+        ++cq;
+      }
+      for (int t = -1; t < nt; ++t, ++turn) {  // a turn: P(t) V(t), then S(t + 1)
+        const uint32_t ev = 2 * (T - 1) + 1, slv = ev % kStages, ek = 2 * T, slk = ek % kStages;
+        const bool more = t + 1 < nt;
+        if (t >= 0 && !(ok = wait_warp(&s.full[slv], (ev / kStages) & 1, s.abort))) break;
+        if (more && !(ok = wait_warp(&s.full[slk], (ek / kStages) & 1, s.abort))) break;
+        if (!more) {
+          if (t < nt_x && !(ok = wait_warp(&s.pfull[x], np & 1, s.abort))) break;
+          // every S of this stream's item has completed: load the next item's
+          // query tile while the last P V and the output are under way
+          if (!(ok = wait_warp(&s.recfull[(n + 1) & 1], ((n + 1) >> 1) & 1, s.abort))) break;
+          load_q(s.rec + ((n + 1) & 1) * 16);
+        }
+        const uint64_t dk = tc::desc_sw128(kv_addr + slk * kTileBytes);
+        const uint64_t dv = tc::desc_sw128_mn(kv_addr + slv * kTileBytes, kHalfBytes);
+        if ((x == 1 || turn > 0) && !(ok = wait_warp(&s.turn[x], (x ? turn : turn - 1) & 1, s.abort))) break;
+        if (t >= 0 && t < nt_x) {
+          if (!(ok = wait_warp(&s.pfull[x], np & 1, s.abort))) break;
+          ++np;
+          tc::tc_fence_after();
+#pragma unroll
+          for (int kk = 0; kk < kKT / 16; ++kk)  // O += P(t) V(t)
+            tc::mma_bf16_ts_if(leader, o_col, s_col + kPCol + kk * 8, dv + kk * (2048 >> 4), idesc_o, t > 0 || kk > 0);
+          if (kSplit) {
+#pragma unroll
+            for (int kk = 0; kk < kKT / 16; ++kk)
+              tc::mma_bf16_ts_if(leader, o_col, s_col + kPLoCol + kk * 8, dv + kk * (2048 >> 4), idesc_o, true);
+          }
+          if (t + 1 == nt_x) tc::mma_commit_if(leader, &s.ofull[x]);
+        }
+        if (t + 1 < nt_x) {
+          const int ksteps = kSplit ? (d + 15) / 16 : kDP / 16;
+#pragma unroll
+          for (int kk = 0; kk < kDP / 16; ++kk) {  // S(t + 1) = Q K(t + 1)^T
+            const uint32_t off = ((kk >> 2) * kHalfBytes + (kk & 3) * 32) >> 4;
+            if (kk == kDP / 16 - kPassEarly) tc::mbar_arrive_if(leader, &s.turn[x ^ 1]);
+            if (kk < ksteps) tc::mma_bf16_if(leader, s_col, dq + off, dk + off, idesc_s, kk > 0);
+          }
+          tc::mma_commit_if(leader, &s.sfull[x]);
+        } else {
+          tc::mbar_arrive_if(leader, &s.turn[x ^ 1]);
+        }
+        if (more) ++T;
       }
       if (!ok) break;
     }
-    if (lane == 0) s.counters[1] = nv;
-  } else if (warp == 1 && lane == 0) {
-    // ---------------------------------------------------------- MMA: S = Q K^T
-    // S(t) goes to buffer t % kSBufs once P(t-3) V(t-3), which read that
-    // buffer's P, has completed (possibly of an earlier item); so this thread
-    // runs up to two tiles ahead of the P.V thread
-    uint32_t ck = 0, T = 0;
+    if (!ok && lane == 0) raise_abort(a, s, tc::kSiteMma);
+    tc::mma_commit_if(leader, &s.mdone[x]);  // every MMA issued above has completed once this arrives
+    tc::mbar_wait(&s.mdone[x], 0);
+    if (cq < nq) tc::mbar_wait(&s.qfull[x], cq & 1);  // a copy in flight (only after an abort)
+    __syncwarp();
+  }
+  } else {
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 208;" ::: "memory");
+    // -------------------------------------------------------------- softmax
+    const int x = (warp - kSoftWarp0) >> 2;              // query tile
+    const int quarter = warp & 3;
+    const int row = quarter * 32 + lane;                 // TMEM lane = query row of the tile
+    const uint32_t tl = tmem + (uint32_t(quarter * 32) << 16);
+    const uint32_t sb = tl + x * kSCols, ob = tl + kOCol + x * kDP;
+    const uint32_t leader = lane == 0, releases = x == 1 && quarter == 0 && lane == 0;
+    uint32_t ns = 0, no = 0;                             // S tiles and O tiles read by this query tile
     bool ok = true;
-    const uint32_t idesc_s = tc::idesc_bf16(kRows, kKT);
     for (uint32_t n = 0; ok; ++n) {
-      const int qs = n & 1;
-      if (!wait_or_abort(&s.qfull[qs], (n >> 1) & 1, s.abort)) { ok = false; break; }
-      if (s.rec[qs * kRecInts] < 0) break;
-      const int nt = s.rec[qs * kRecInts + 6];
-      const uint32_t q_addr = tc::smem_u32(s.q + qs * kQBytes);
-      tc::tc_fence_after();
-      for (int t = 0; t < nt; ++t) {
-        const uint32_t Ts = T + t;
-        const int b = Ts % kSBufs, sk = Ts % kKStages;
-        if (Ts >= uint32_t(kSBufs) && !wait_or_abort(&s.pvdone[b], ((Ts / kSBufs) - 1) & 1, s.abort)) {
+      const int rs = n & 1;
+      if (!wait_warp(&s.recfull[rs], (n >> 1) & 1, s.abort)) {
+        if (lane == 0) raise_abort(a, s, tc::kSiteLoad);
+        break;
+      }
+      const volatile int* rec = s.rec + rs * 16;
+      const int u = rec[0], l = rec[1], g = rec[2], cnt = rec[5 + x], nt = rec[7 + x], N = rec[9];
+      const int i0 = rec[4] + (x ? rec[5] : 0);
+      const bool row_ok = u >= 0 && row < cnt * G;
+      const int i_row = i0 + (row_ok ? row / G : 0);
+      const int h_row = g * G + (row_ok ? row % G : 0);
+      // Rows without a position (past the tile or the box, or an index outside
+      // the request) are computed unmasked and never written: a masked row
+      // would send its warp down the masking path on every key tile.
+      int p_row = row_ok ? s.pos[(rs * 2 + x) * kRows + row / G] : -1;
+      const bool live = p_row >= 0 && p_row < N;
+      if (!live) p_row = INT_MAX;
+      __syncwarp();
+      tc::mbar_arrive_if(leader, &s.recempty[rs]);
+      if (u < 0) break;
+
+      float m_ref = -INFINITY, lsum = 0.f;  // running max (scaled, log2 units) and row sum
+      for (int t = 0; t < nt; ++t, ++ns) {
+        // the tcgen05.ld below is warp-collective: the whole warp goes on or stops
+        if (!wait_warp(&s.sfull[x], ns & 1, s.abort)) {
+          if (lane == 0) raise_abort(a, s, tc::kSiteMma);
           ok = false;
           break;
         }
-        if (!wait_or_abort(&s.kfull[sk], (Ts / kKStages) & 1, s.abort)) { ok = false; break; }
-        ++ck;
         tc::tc_fence_after();
-        const uint32_t k_addr = tc::smem_u32(s.k + sk * kTileBytes);
+        float sv[kKT];
+        tc::tmem_ld128(sb, sv);
+        const int j0 = t * kKT;
+        if (j0 + kKT - 1 > p_row) {  // part of this tile is past this row's position
 #pragma unroll
-        for (int kk = 0; kk < 8; ++kk) {
-          const uint32_t off = (kk & 3) * 32;
-          tc::mma_bf16(tmem + b * kSCols, tc::desc_sw128(q_addr + (kk >> 2) * kQHalf + off),
-                       tc::desc_sw128(k_addr + (kk >> 2) * kTileHalf + off), idesc_s, kk > 0);
+          for (int i = 0; i < kKT; ++i)
+            if (j0 + i > p_row) sv[i] = -INFINITY;
         }
-        tc::mma_commit(&s.sfull[b]);
-        tc::mma_commit(&s.kempty[sk]);
-      }
-      if (!ok) break;
-      tc::mma_commit(&s.qempty[qs]);  // every S of this item is issued
-      T += nt;
-    }
-    if (!ok) raise_abort(a, s, tc::kSiteMma);
-    s.counters[2] = ck;
-    tc::mma_commit(&s.mdone[0]);  // every MMA issued above has completed once this arrives
-    tc::mbar_wait(&s.mdone[0], 0);
-  } else if (warp == kPvWarp && lane == 0) {
-    // -------------------------------------------------------- MMA: O += P V
-    uint32_t cv = 0, T = 0;
-    bool ok = true;
-    const uint32_t idesc_o = tc::idesc_bf16(kRows, kD, /*b_mn_major=*/true);
-    for (uint32_t n = 0; ok; ++n) {
-      const int qs = n & 1;
-      if (!wait_or_abort(&s.qfull[qs], (n >> 1) & 1, s.abort)) { ok = false; break; }
-      const int u = s.rec[qs * kRecInts], nt = s.rec[qs * kRecInts + 6];
-      tc::mbar_arrive(&s.qempty[qs]);  // this thread is done with the record
-      if (u < 0) break;
-      for (int t = 0; t < nt; ++t) {
-        const uint32_t Tc = T + t;
-        const int b = Tc % kSBufs, sv = Tc % kVStages;
-        if (!wait_or_abort(&s.vfull[sv], (Tc / kVStages) & 1, s.abort)) { ok = false; break; }
-        ++cv;
-        if (!wait_or_abort(&s.pfull[b], (Tc / kSBufs) & 1, s.abort)) { ok = false; break; }
-        // O of the previous item must have been read out before P(0) V(0) overwrites it
-        if (t == 0 && n > 0 && !wait_or_abort(s.oempty, (n - 1) & 1, s.abort)) { ok = false; break; }
-        tc::tc_fence_after();
-        const uint32_t v_addr = tc::smem_u32(s.v + sv * kTileBytes);
-        const uint32_t pb = tmem + b * kSCols + kPCol;
+        float tm[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
-        for (int kk = 0; kk < kKT / 16; ++kk)  // O += P(t) V(t)
-          tc::mma_bf16_ts(tmem + kOCol, pb + kk * 8, tc::desc_sw128_mn(v_addr + kk * 2048, kTileHalf),
-                          idesc_o, t > 0 || kk > 0);
-        tc::mma_commit(&s.pvdone[b]);
-        tc::mma_commit(&s.vempty[sv]);
-      }
-      if (!ok) break;
-      T += nt;
-      tc::mma_commit(s.ofull);  // O of this item is complete once this arrives
-    }
-    if (!ok) raise_abort(a, s, tc::kSiteMma);
-    s.counters[3] = cv;
-    tc::mma_commit(&s.mdone[1]);
-    tc::mbar_wait(&s.mdone[1], 0);
-  } else if (warp >= 2 && warp < kVWarp) {
-    // -------------------------------------------------------------- softmax
-    const int et = tid - 64;                             // 0..255
-    const int hh = et >> 7;                              // half of the key tile / of O
-    const int quarter = warp & 3;
-    const int row = quarter * 32 + lane;                 // TMEM lane = query row of the tile
-    const uint32_t lane_base = uint32_t(quarter * 32) << 16;
-    const uint32_t tl = tmem + lane_base;
-    bool ok = true;
-    uint32_t T = 0;
-    for (uint32_t n = 0;; ++n) {
-      const int qs = n & 1;
-      // all 256 threads agree to go on, so the named barriers below stay uniform
-      const bool got = wait_or_abort(&s.qfull[qs], (n >> 1) & 1, s.abort);
-      if (!softmax_all(ok && got)) {
-        if (ok) raise_abort(a, s, tc::kSiteLoad);
-        break;
-      }
-      const volatile int* rec = s.rec + qs * kRecInts;
-      const int u = rec[0];
-      Item it;
-      it.l = rec[1];
-      it.g = rec[2];
-      it.r = rec[3];
-      it.i0 = rec[4];
-      it.cnt = rec[5];
-      const int nt = rec[6], N = rec[7];
-      const bool row_ok = u >= 0 && row < it.cnt * G;
-      const int i_row = it.i0 + (row_ok ? row / G : 0);
-      const int h_row = it.g * G + (row_ok ? row % G : 0);
-      int p_row = row_ok ? s.pos[qs * kRows + row / G] : -1;  // rows past the item (or the box) are fully masked
-      if (p_row >= N) p_row = -1;
-      asm volatile("bar.sync 1, %0;" ::"n"(kSoftThreads) : "memory");  // everyone has read the record
-      if (et == 0) tc::mbar_arrive(&s.qempty[qs]);
-      if (u < 0) break;
-
-      float m_ref = -INFINITY, lsum = 0.f;  // running max (scaled, log2 units, same in both halves) and half-row sum
-      for (int t = 0; t < nt; ++t) {
-        const uint32_t Tc = T + t;
-        const uint32_t sbuf = Tc % kSBufs;
-        const uint32_t sb = tl + sbuf * kSCols;
-        // the tcgen05.ld below is warp-collective: the whole warp goes on or stops
-        const bool gs = __all_sync(0xffffffffu, ok && (mbar_probe(&s.sfull[sbuf], (Tc / kSBufs) & 1) ||
-                                                       wait_or_abort(&s.sfull[sbuf], (Tc / kSBufs) & 1, s.abort)));
-        if (!gs) {
-          if (ok) raise_abort(a, s, tc::kSiteMma);
-          ok = false;
-        }
-        float sv[64];
-        float hmax = -INFINITY;
-        const int j0 = t * kKT + hh * 64;
-        if (gs) {
-          tc::tc_fence_after();
-          tc::tmem_ld64(sb + hh * 64, sv);
-          if (j0 + 63 > p_row) {  // part of this half is past this row's position
-#pragma unroll
-            for (int i = 0; i < 64; ++i)
-              if (j0 + i > p_row) sv[i] = -INFINITY;
-          }
-          float tm[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-#pragma unroll
-          for (int i = 0; i < 32; ++i) tm[i & 3] = tc::fmax3(tm[i & 3], sv[2 * i], sv[2 * i + 1]);
-          hmax = fmaxf(fmaxf(tm[0], tm[1]), fmaxf(tm[2], tm[3]));
-        }
-        // exchange the half-row maxima (buffers alternate with the tile, so a
-        // half that runs ahead never overwrites a value its partner still reads)
-        float* xm = s.xmax + (Tc & 1) * 256;
-        xm[hh * 128 + row] = hmax;
-        asm volatile("bar.sync 1, %0;" ::"n"(kSoftThreads) : "memory");
-        if (!ok) continue;
-        const float tmax = fmaxf(hmax, xm[(hh ^ 1) * 128 + row]) * a.scale_log2;
+        for (int i = 0; i < kKT / 2; ++i) tm[i & 3] = tc::fmax3(tm[i & 3], sv[2 * i], sv[2 * i + 1]);
+        const float tmax = fmaxf(fmaxf(tm[0], tm[1]), fmaxf(tm[2], tm[3])) * a.scale_log2;
         const bool need = tmax > m_ref + kRescaleLog2 || (m_ref == -INFINITY && tmax != -INFINITY);
         const float alpha = need ? tc::ex2(m_ref - tmax) : 1.f;  // 0 when m_ref is -inf
         if (need) {
           lsum *= alpha;
           m_ref = tmax;
         }
-        // this half of P = 2^(S scale - m) in bf16 pairs over the upper half of S
-        // (one packed FMA per pair for scale and bias, packed adds for the sum).
-        // A row with no visible key yet (m = -inf) uses bias 0: its logits are
-        // all -inf and its P is 0.
+        if (__any_sync(0xffffffffu, need) && t > 0) {
+          // S(t) is ready, so P(t-1) V(t-1) has completed; P(t) V(t) waits for
+          // this warp's arrival below
+          for (int c = 0; c < kDP; c += 16) {
+            float o[16];
+            tc::tmem_ld16(ob + c, o);
+            uint32_t w[16];
+#pragma unroll
+            for (int i = 0; i < 16; ++i) w[i] = __float_as_uint(o[i] * alpha);
+            tc::tmem_st16_nowait(ob + c, w);
+          }
+        }
+        // P = 2^(S scale - m) in bf16 pairs over S, which this warp has read (one
+        // packed FMA per pair for scale and bias, packed adds for the sum). A row
+        // with no visible key yet (m = -inf) uses bias 0: its logits are all
+        // -inf and its P is 0. With kSplit a second tile holds the rounding
+        // error of the first, so that P keeps 16 bits of mantissa.
         const float2 sc2 = make_float2(a.scale_log2, a.scale_log2);
         const float2 nb2 = m_ref == -INFINITY ? make_float2(0.f, 0.f) : make_float2(-m_ref, -m_ref);
         float2 ls2[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-        {
-          uint32_t pw[32];
 #pragma unroll
-          for (int i = 0; i < 32; ++i) {
-            const float2 y = tc::ffma2(make_float2(sv[2 * i], sv[2 * i + 1]), sc2, nb2);
+        for (int c = 0; c < kKT / 32; ++c) {
+          uint32_t pw[16], lo[16];
+#pragma unroll
+          for (int i = 0; i < 16; ++i) {
+            const float2 y = tc::ffma2(make_float2(sv[32 * c + 2 * i], sv[32 * c + 2 * i + 1]), sc2, nb2);
             const float2 pp = make_float2(tc::ex2(y.x), tc::ex2(y.y));
             ls2[i & 1] = tc::fadd2(ls2[i & 1], pp);
             __nv_bfloat162 pr = __floats2bfloat162_rn(pp.x, pp.y);
             pw[i] = *reinterpret_cast<uint32_t*>(&pr);
+            if (kSplit) {
+              const float2 hi = __bfloat1622float2(pr);
+              pr = __floats2bfloat162_rn(pp.x - hi.x, pp.y - hi.y);
+              lo[i] = *reinterpret_cast<uint32_t*>(&pr);
+            }
           }
-          tc::tmem_st32u(sb + kPCol + hh * 32, pw);
+          tc::tmem_st16_nowait(sb + kPCol + 16 * c, pw);
+          if (kSplit) tc::tmem_st16_nowait(sb + kPLoCol + 16 * c, lo);
         }
-        const float ls[4] = {ls2[0].x, ls2[0].y, ls2[1].x, ls2[1].y};
-        lsum += (ls[0] + ls[1]) + (ls[2] + ls[3]);
-        if (__any_sync(0xffffffffu, need) && t > 0) {
-          // P(t-1) V(t-1) must have completed before this warp rescales its half
-          // of O. That buffer's next P.V needs a P this softmax has not written
-          // yet, so the barrier's parity cannot alias; P(t) V(t) waits for this
-          // warp's pfull arrival below.
-          if (!__all_sync(0xffffffffu,
-                          wait_or_abort(&s.pvdone[(Tc - 1) % kSBufs], ((Tc - 1) / kSBufs) & 1, s.abort))) {
-            raise_abort(a, s, tc::kSiteMma);
-            ok = false;
-            continue;
-          }
-          tc::tc_fence_after();
-          for (int c = hh * 64; c < hh * 64 + 64; c += 32) {
-            float o[32];
-            tc::tmem_ld32(tl + kOCol + c, o);
-#pragma unroll
-            for (int i = 0; i < 32; ++i) o[i] *= alpha;
-            tc::tmem_st32(tl + kOCol + c, o);
-          }
-        }
+        lsum += (ls2[0].x + ls2[0].y) + (ls2[1].x + ls2[1].y);
+        tc::tmem_wait_st();
         tc::tc_fence_before();
-        tc::mbar_arrive(&s.pfull[sbuf]);
+        __syncwarp();
+        tc::mbar_arrive_if(leader, &s.pfull[x]);
+        // S_B(t) was the last to read K(t) and, in issue order, comes after both
+        // P V of the tile before: their slots may be loaded again
+        tc::mbar_arrive_if(releases, &s.done[ns % kDone]);
       }
-      T += nt;
-      // row sum = the two halves' sums (same running max in both)
-      s.xsum[hh * 128 + row] = lsum;
-      asm volatile("bar.sync 1, %0;" ::"n"(kSoftThreads) : "memory");
-      const float total = s.xsum[row] + s.xsum[128 + row];
-      // O of this item is complete once the MMA thread's per-item commit has
-      // arrived (it cannot run a phase ahead: the next one needs this warp's P)
-      const bool fin = __all_sync(0xffffffffu, ok && wait_or_abort(s.ofull, n & 1, s.abort));
-      if (!fin && ok) {
-        raise_abort(a, s, tc::kSiteFinal);
+      if (nt == 0 || !ok) continue;
+      if (!wait_warp(&s.ofull[x], no & 1, s.abort)) {
+        if (lane == 0) raise_abort(a, s, tc::kSiteFinal);
         ok = false;
+        break;
       }
-      if (fin) {
-        tc::tc_fence_after();
-        const float inv = total > 0.f ? 1.f / total : 0.f;
-        __nv_bfloat16* dst = a.out + ((int64_t(it.l) * a.n_sel + i_row) * Hq + h_row) * kD;
-        // This thread's 64 columns of O in one load, then its half row as
-        // bf16. Each lane writes its own row, so a warp's store covers 32
-        // rows: 32-byte stores (whole sectors) when the buffer allows them.
+      ++no;
+      tc::tc_fence_after();
+      // The row of O as bf16. Each lane writes its own row, so a warp's store
+      // covers 32 rows: 32-byte stores (whole sectors) when the buffer allows
+      // them. The next item's P(0) V(0), which overwrites O, waits for a P this
+      // warp writes after these loads.
+      const float inv = lsum > 0.f ? 1.f / lsum : 0.f;
+      __nv_bfloat16* dst = a.out + ((int64_t(l) * a.n_sel + i_row) * Hq + h_row) * d;
+#pragma unroll
+      for (int c = 0; c < kDP; c += 64) {
         float o[64];
-        tc::tmem_ld64(tl + kOCol + hh * 64, o);
-        if (row_ok && p_row >= 0) {
+        tc::tmem_ld64(ob + c, o);
+        if (live) {
           uint32_t w[32];
 #pragma unroll
           for (int k2 = 0; k2 < 32; ++k2) {
             __nv_bfloat162 pr = __floats2bfloat162_rn(o[2 * k2] * inv, o[2 * k2 + 1] * inv);
             w[k2] = *reinterpret_cast<uint32_t*>(&pr);
           }
-          __nv_bfloat16* drow = dst + hh * 64;
           if (a.out32) {
 #pragma unroll
             for (int u8 = 0; u8 < 4; ++u8)
-              asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(drow + u8 * 16),
-                           "r"(w[8 * u8]), "r"(w[8 * u8 + 1]), "r"(w[8 * u8 + 2]), "r"(w[8 * u8 + 3]),
-                           "r"(w[8 * u8 + 4]), "r"(w[8 * u8 + 5]), "r"(w[8 * u8 + 6]), "r"(w[8 * u8 + 7])
-                           : "memory");
+              if (c + u8 * 16 < d)
+                asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst + c + u8 * 16),
+                             "r"(w[8 * u8]), "r"(w[8 * u8 + 1]), "r"(w[8 * u8 + 2]), "r"(w[8 * u8 + 3]),
+                             "r"(w[8 * u8 + 4]), "r"(w[8 * u8 + 5]), "r"(w[8 * u8 + 6]), "r"(w[8 * u8 + 7])
+                             : "memory");
           } else {
 #pragma unroll
             for (int u4 = 0; u4 < 8; ++u4)
-              *reinterpret_cast<uint4*>(drow + u4 * 8) = make_uint4(w[4 * u4], w[4 * u4 + 1], w[4 * u4 + 2], w[4 * u4 + 3]);
+              if (c + u4 * 8 < d)
+                *reinterpret_cast<uint4*>(dst + c + u4 * 8) = make_uint4(w[4 * u4], w[4 * u4 + 1], w[4 * u4 + 2], w[4 * u4 + 3]);
           }
         }
       }
       tc::tc_fence_before();
-      tc::mbar_arrive(s.oempty);  // O may be overwritten by the next item
     }
   }
   __syncthreads();
-  if (tid == 0) {  // drain loads issued but never consumed (only after an abort)
-    for (uint32_t n = s.counters[2]; n < s.counters[0]; ++n)
-      tc::mbar_wait(&s.kfull[n % kKStages], (n / kKStages) & 1);
-    for (uint32_t n = s.counters[3]; n < s.counters[1]; ++n)
-      tc::mbar_wait(&s.vfull[n % kVStages], (n / kVStages) & 1);
+  if (tid == 0) {  // wait for each ring slot's last copy (all have landed unless a role gave up)
+    const int nk = int(s.counters[0]), nv = int(s.counters[1]);
+    for (int sl = 0; sl < kStages; ++sl) {
+      int e = max(2 * nk - 2, 2 * nv - 1);
+      while (e >= 0 && (e % kStages != sl || e / 2 >= ((e & 1) ? nv : nk))) --e;
+      if (e >= 0) tc::mbar_wait(&s.full[sl], (e / kStages) & 1);
+    }
   }
   tc::tc_fence_before();
   __syncthreads();
-  if (warp == 1) tc::tmem_dealloc(tmem, kTmemCols);
+  if (warp == kMmaWarp) tc::tmem_dealloc(tmem, kTmemCols);
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*,
@@ -683,8 +661,8 @@ EncodeTiledFn encode_fn() {
 bool make_map(CUtensorMap* m, const KvDev& kv, void* base) {
   EncodeTiledFn enc = encode_fn();
   if (!enc) return false;
-  cuuint64_t dims[2] = {cuuint64_t(kD), 0};
-  cuuint64_t strides[1] = {cuuint64_t(kD) * 2};
+  cuuint64_t dims[2] = {cuuint64_t(kv.d), 0};
+  cuuint64_t strides[1] = {cuuint64_t(kv.d) * 2};
   cuuint32_t box[2] = {64, 0};
   cuuint32_t estr[2] = {1, 1};
   if (kv.page_size == 0) {
@@ -705,8 +683,8 @@ bool make_map(CUtensorMap* m, const KvDev& kv, void* base) {
 bool make_qmap(CUtensorMap* m, const KvDev& kv, const void* q_rows, int32_t n_sel, int rows_per_tile) {
   EncodeTiledFn enc = encode_fn();
   if (!enc) return false;
-  cuuint64_t dims[3] = {cuuint64_t(kD), cuuint64_t(kv.Hq), cuuint64_t(kv.L) * cuuint64_t(n_sel)};
-  cuuint64_t strides[2] = {cuuint64_t(kD) * 2, cuuint64_t(kv.Hq) * kD * 2};
+  cuuint64_t dims[3] = {cuuint64_t(kv.d), cuuint64_t(kv.Hq), cuuint64_t(kv.L) * cuuint64_t(n_sel)};
+  cuuint64_t strides[2] = {cuuint64_t(kv.d) * 2, cuuint64_t(kv.Hq) * kv.d * 2};
   cuuint32_t box[3] = {64, cuuint32_t(kv.G), cuuint32_t(rows_per_tile)};
   cuuint32_t estr[3] = {1, 1, 1};
   return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(q_rows), dims, strides, box,
@@ -717,7 +695,7 @@ bool make_qmap(CUtensorMap* m, const KvDev& kv, const void* q_rows, int32_t n_se
 }  // namespace
 
 bool refresh_tc_supported(const KvDev& kv) {
-  if (kv.dtype != CONDUIT_BF16 || kv.d != kD || kv.G > kRows) return false;
+  if (kv.dtype != CONDUIT_BF16 || kv.d != kMaxD || kv.G > kRows) return false;
   if (kv.page_size != 0 && (kv.page_size % 8 != 0 || kKT % kv.page_size != 0)) return false;
   return true;
 }
@@ -736,7 +714,6 @@ cudaError_t launch_refresh_tc(const KvDev& kv, const BatchDev& b, const int32_t*
   a.b = b;
   a.idx = idx;
   a.idx_off = idx_off_dev;
-  a.q_rows = static_cast<const __nv_bfloat16*>(q_rows);
   a.out = static_cast<__nv_bfloat16*>(out);
   a.out32 = (reinterpret_cast<uintptr_t>(out) & 31) == 0;
   a.n_sel = n_sel;
@@ -744,12 +721,12 @@ cudaError_t launch_refresh_tc(const KvDev& kv, const BatchDev& b, const int32_t*
   int blocks = 0;
   for (int r = 0; r < b.R; ++r) {
     const int kr = idx_off_host[r + 1] - idx_off_host[r];
-    blocks += (kr + a.rows_per_tile - 1) / a.rows_per_tile;
+    blocks += (kr + 2 * a.rows_per_tile - 1) / (2 * a.rows_per_tile);
   }
   a.n_blocks = blocks;
   a.n_items = blocks * kv.Hkv * kv.L;
   a.next_item = work_counter;
-  a.scale_log2 = kLog2e / sqrtf(float(kD));
+  a.scale_log2 = kLog2e / sqrtf(float(kv.d));
   a.status = status;
   if (blocks == 0) return cudaSuccess;
   int dev = 0, sms = 0;
@@ -760,13 +737,13 @@ cudaError_t launch_refresh_tc(const KvDev& kv, const BatchDev& b, const int32_t*
   if ((err = cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev))) return err;
   // longest-first when the whole K/V of the batch fits in half of L2 (the rest
   // holds queries and outputs), else (layer, head)-major
-  const double kv_bytes = 2.0 * double(kv.L) * kv.Hkv * double(kv.n_tot) * kD * 2;
+  const double kv_bytes = 2.0 * double(kv.L) * kv.Hkv * double(kv.n_tot) * kv.d * 2;
   a.blocks_major = kv_bytes <= 0.5 * double(l2) ? 1 : 0;
-  if ((err = cudaFuncSetAttribute(refresh_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  int(kSmem))))
-    return err;
   if ((err = cudaMemsetAsync(work_counter, 0, sizeof(int32_t), stream))) return err;
-  refresh_tc_kernel<<<std::min(a.n_items, sms), kThreads, kSmem, stream>>>(kmap, vmap, qmap, a);
+  auto* f = refresh_tc_kernel<2, false>;
+  constexpr uint32_t smem = Shape<2>::kSmem;
+  if ((err = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)))) return err;
+  f<<<std::min(a.n_items, sms), kThreads, smem, stream>>>(kmap, vmap, qmap, a);
   count_launches(1);
   return cudaGetLastError();
 }
