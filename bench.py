@@ -215,10 +215,10 @@ def side_cache_bytes(pipe) -> int:
 def call_kernels(pipe) -> dict:
     """Kernels behind each C-ABI call for this cache, their binding unit and source file.
 
-    bf16 caches with head_dim 128 take the tensor-core kernels; other shapes
+    bf16 caches with head_dim up to 128 take the tensor-core kernels; other shapes
     the CUDA-core ones (the library makes the same choice).
     """
-    tc = pipe.kv.k.dtype == torch.bfloat16 and pipe.kv.head_dim == 128
+    tc = pipe.kv.k.dtype == torch.bfloat16 and pipe.kv.head_dim <= 128
     tail = ["finalize_tokens_kernel", "image_means_kernel"]
     if tc:  # hbm or tensor: run_conduit keeps whichever ideal time is longer for the workload
         score = (["score_tc_kernel"] + tail, "hbm", "score_tc.cu")

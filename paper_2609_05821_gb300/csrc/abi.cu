@@ -144,7 +144,7 @@ conduit_status make_layers(const conduit_kv* kv, const int32_t* layers, int32_t 
 }
 
 struct ScoreLayout {
-  bool tc;     // tensor-core kernel (bf16, head_dim 128) or the CUDA-core ones
+  bool tc;     // tensor-core kernel (bf16, head_dim up to 128) or the CUDA-core ones
   int rg_max;  // row groups per slab (column-sum partials per KV head)
   int group_rows;
   int parts;   // partials per row group and per value norm (2 for the tensor-core kernel)
@@ -660,11 +660,18 @@ conduit_status conduit_refresh_attn(const conduit_kv* kv, const conduit_batch* b
   if (n_sel == 0) return CONDUIT_OK;
   if (!q_rows || !out) return fail(CONDUIT_ERR_INVALID_ARG, "q_rows and out are required");
   const KvDev kd = make_kv(kv, batch);
-  const bool tc = refresh_tc_supported(kd);
-  if ((st = check_workspace(workspace, workspace_bytes, tc ? kAlign : 0))) return st;
+  // The tensor-core kernel needs 16-byte aligned rows. For head sizes other
+  // than 128 the workspace and the alignment are optional: rows that are not
+  // aligned take the CUDA-core kernel, and without a workspace the items are
+  // dealt out in a fixed order.
+  const bool d128 = kd.d == 128;
+  const bool tc = refresh_tc_supported(kd) && (d128 || (aligned16(q_rows) && aligned16(out)));
+  if ((st = check_workspace(workspace, workspace_bytes, tc && d128 ? kAlign : 0))) return st;
+  int32_t* counter = static_cast<int32_t*>(workspace);
+  if (workspace_bytes < kAlign || reinterpret_cast<uintptr_t>(workspace) % kAlign) counter = nullptr;
   cudaError_t err =
       tc ? launch_refresh_tc(kd, make_batch(batch), idx, idx_off_dev, idx_off, n_sel, q_rows, out,
-                             static_cast<int32_t*>(workspace), status,
+                             counter, status,
                              static_cast<cudaStream_t>(stream))
          : launch_refresh_simt(kd, make_batch(batch), idx, idx_off_dev, n_sel, q_rows, out,
                                static_cast<cudaStream_t>(stream));

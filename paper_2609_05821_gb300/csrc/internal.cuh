@@ -136,9 +136,15 @@ cudaError_t launch_score_simt(const KvDev& kv, const BatchDev& b, const void* q,
                               const LayerList& layers, int max_rows, int max_tokens,
                               float2* stats, float* pa, float* pa2, const float* extra_lse,
                               cudaStream_t stream);
-// Tensor-core scoring (bf16, head_dim 128): one kernel, row statistics then
+// The tensor-core kernels address cache rows with 32-bit tensor-map coordinates.
+inline bool tc_rows_ok(const KvDev& kv) {
+  const int64_t rows = kv.page_size == 0 ? kv.n_tot : int64_t(kv.num_pages) * kv.page_size;
+  return int64_t(kv.L) * kv.Hkv * rows <= INT32_MAX;
+}
+// Tensor-core scoring (bf16, head_dim up to 128): one kernel, row statistics then
 // column sums per (slab, group of at most 256 scoring rows); it writes two
-// partials per row group into pa and two half-row partials into ss (ss NULL:
+// partials per row group into pa and two partials per V row (its first and
+// second half, of 32 or 64 dims) into ss (ss NULL:
 // V is not read, the norms come from the side cache).
 constexpr int kScoreGroupRows = 256;
 bool score_tc_supported(const KvDev& kv);
@@ -217,6 +223,8 @@ cudaError_t launch_kv_copy(const KvDev& kv, const BatchDev& b, const int32_t* id
                            const int32_t* idx_off_dev, int32_t n_sel, int max_sel, int mode,
                            void* k_rows, void* v_rows, const void* k_new, const void* v_new,
                            cudaStream_t stream);
+// Tensor-core refresh attention (bf16, head_dim up to 128). work_counter may be
+// NULL (items are dealt out in a fixed order).
 bool refresh_tc_supported(const KvDev& kv);
 cudaError_t launch_refresh_tc(const KvDev& kv, const BatchDev& b, const int32_t* idx,
                               const int32_t* idx_off_dev, const int32_t* idx_off_host, int32_t n_sel,

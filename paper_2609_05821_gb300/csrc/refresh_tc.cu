@@ -1,4 +1,4 @@
-// Tensor-core causal refresh attention for bf16 caches with head_dim 128
+// Tensor-core causal refresh attention for bf16 caches with head_dim up to 128
 // (selective recompute, Conduit Sec. 3.1 / 4.3):
 //   out[l][i][h] = sum_{j <= p_i} softmax_j(<q[l][i][h], K'[l][h/G][j]> / sqrt(d)) V'[l][h/G][j]
 //
@@ -63,7 +63,8 @@ constexpr int kMmaWarp = 1, kVWarp = 2, kSoftWarp0 = 4;  // warp 0: items and K;
 constexpr int kThreads = 384;
 constexpr uint32_t kHalfBytes = 128 * 128;       // 16 KB: one 64-dim half of a 128-row tile
 constexpr int kRecReaders = 11;                  // two MMA warps, V warp, eight softmax warps
-constexpr uint32_t kTailBytes = 256 + 2 * (16 + 2 * kRows) * 4;
+constexpr uint32_t kBarBytes = 320;             // barriers, TMEM slot, abort flag, counters
+constexpr uint32_t kTailBytes = kBarBytes + 2 * (16 + 2 * kRows) * 4;
 
 // Head sizes: kHalves 64-dim halves of a row (one 128-byte swizzled row each;
 // a smaller head_dim is padded with zeros by the copies).
@@ -77,7 +78,7 @@ struct Shape {
   static constexpr int kDone = 2 * kAhead;
   static constexpr uint32_t kSmem = (2 + kStages) * kTileBytes + kTailBytes;
   static_assert(kSmem <= 232448, "shared memory of one CTA");
-  static_assert((kStages + kDone + 6 + 4 + 4 + 2) * 8 + 32 <= 256, "barriers and counters");
+  static_assert((kStages + kDone + 6 + 4 + 4 + 2) * 8 + 32 <= kBarBytes, "barriers and counters");
 };
 constexpr uint32_t kTmemCols = 512;
 constexpr uint32_t kSCols = 128;                 // one S buffer
@@ -99,7 +100,7 @@ struct RefArgs {
   int32_t n_blocks;        // items per (layer, KV head)
   int32_t n_items;         // n_blocks * Hkv * L
   int32_t blocks_major;    // item order: block (largest first) outer, or (layer, head) outer
-  int32_t* next_item;      // work counter, zero at launch
+  int32_t* next_item;      // work counter, zero at launch; NULL: CTA c takes items c, c + grid, ...
   float scale_log2;
   int32_t* status;
 };
@@ -185,7 +186,7 @@ __device__ __forceinline__ Smem carve(uint8_t* base) {
   s.tmem_slot = reinterpret_cast<uint32_t*>(s.mdone + 2);
   s.abort = reinterpret_cast<volatile int*>(s.tmem_slot + 1);
   s.counters = reinterpret_cast<uint32_t*>(s.tmem_slot + 2);
-  s.rec = reinterpret_cast<volatile int*>(reinterpret_cast<uint8_t*>(bar) + 256);
+  s.rec = reinterpret_cast<volatile int*>(reinterpret_cast<uint8_t*>(bar) + kBarBytes);
   s.pos = s.rec + 2 * 16;
   return s;
 }
@@ -295,7 +296,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   // Registers: a softmax thread holds a row of S (128 values). The shares add
   // up to 128 x 88 + 256 x 208 = 384 x 168, what the launch has.
   if (warp < kSoftWarp0) {
-  asm volatile("setmaxnreg.dec.sync.aligned.u32 88;" ::: "memory");
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 88;" ::: "memory");
   if (warp == 0) {
     // ------------------------------------------------ items and K (warp 0)
     uint32_t T = 0;
@@ -303,7 +304,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     for (uint32_t n = 0; ok; ++n) {
       int u = 0;
       if (lane == 0) {
-        u = n == 0 ? int(blockIdx.x) : int(gridDim.x) + atomicAdd(a.next_item, 1);
+        u = n == 0 ? int(blockIdx.x)
+                   : a.next_item ? int(gridDim.x) + atomicAdd(a.next_item, 1) : int(blockIdx.x + n * gridDim.x);
         if (u >= a.n_items) u = -1;
       }
       u = __shfl_sync(0xffffffffu, u, 0);
@@ -694,8 +696,11 @@ bool make_qmap(CUtensorMap* m, const KvDev& kv, const void* q_rows, int32_t n_se
 
 }  // namespace
 
+// Every bf16 head size the copies can pad to one or two 64-dim halves: a step on
+// a 24-layer, 14/2-head, head_dim 64 cache of 2 900 tokens took 8.6 ms with this
+// pass and the scoring on CUDA cores and takes 0.22 ms with both here.
 bool refresh_tc_supported(const KvDev& kv) {
-  if (kv.dtype != CONDUIT_BF16 || kv.d != kMaxD || kv.G > kRows) return false;
+  if (kv.dtype != CONDUIT_BF16 || kv.d > kMaxD || kv.G > kRows || !tc_rows_ok(kv)) return false;
   if (kv.page_size != 0 && (kv.page_size % 8 != 0 || kKT % kv.page_size != 0)) return false;
   return true;
 }
@@ -715,7 +720,7 @@ cudaError_t launch_refresh_tc(const KvDev& kv, const BatchDev& b, const int32_t*
   a.idx = idx;
   a.idx_off = idx_off_dev;
   a.out = static_cast<__nv_bfloat16*>(out);
-  a.out32 = (reinterpret_cast<uintptr_t>(out) & 31) == 0;
+  a.out32 = (reinterpret_cast<uintptr_t>(out) & 31) == 0 && kv.d % 16 == 0;
   a.n_sel = n_sel;
   a.rows_per_tile = kRows / kv.G;
   int blocks = 0;
@@ -739,13 +744,23 @@ cudaError_t launch_refresh_tc(const KvDev& kv, const BatchDev& b, const int32_t*
   // holds queries and outputs), else (layer, head)-major
   const double kv_bytes = 2.0 * double(kv.L) * kv.Hkv * double(kv.n_tot) * kv.d * 2;
   a.blocks_major = kv_bytes <= 0.5 * double(l2) ? 1 : 0;
-  if ((err = cudaMemsetAsync(work_counter, 0, sizeof(int32_t), stream))) return err;
-  auto* f = refresh_tc_kernel<2, false>;
-  constexpr uint32_t smem = Shape<2>::kSmem;
-  if ((err = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)))) return err;
-  f<<<std::min(a.n_items, sms), kThreads, smem, stream>>>(kmap, vmap, qmap, a);
+  if (work_counter && (err = cudaMemsetAsync(work_counter, 0, sizeof(int32_t), stream))) return err;
+  auto launch = [&](auto* f, uint32_t smem) -> cudaError_t {
+    if ((err = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)))) return err;
+    f<<<std::min(a.n_items, sms), kThreads, smem, stream>>>(kmap, vmap, qmap, a);
+    return cudaGetLastError();
+  };
+  // head_dim 128 keeps its bf16 P; the smaller sizes ran with fp32 weights on
+  // CUDA cores before and keep that precision by a split P
+  if (kv.d == kMaxD)
+    err = launch(refresh_tc_kernel<2, false>, Shape<2>::kSmem);
+  else if (kv.d > 64)
+    err = launch(refresh_tc_kernel<2, true>, Shape<2>::kSmem);
+  else
+    err = launch(refresh_tc_kernel<1, true>, Shape<1>::kSmem);
+  if (err) return err;
   count_launches(1);
-  return cudaGetLastError();
+  return cudaSuccess;
 }
 
 }  // namespace conduit

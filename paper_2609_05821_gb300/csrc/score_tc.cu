@@ -1,4 +1,6 @@
-// Tensor-core scoring pass for bf16 caches with head_dim 128 (Conduit Eq. 6).
+// Tensor-core scoring pass for bf16 caches with head_dim up to 128 (Conduit
+// Eq. 6). A head row is one or two 64-dim halves (kHalves); the copies pad a
+// smaller head_dim with zeros, which add nothing to a logit or a norm.
 //
 // One persistent, warp-specialised kernel. A work unit is one slab (request
 // r, scored layer l, KV head g) restricted to a group of at most 256 scoring
@@ -40,9 +42,8 @@
 namespace conduit {
 namespace {
 
-constexpr int kD = 128;
+constexpr int kMaxD = 128;
 constexpr int kTile = 128;
-constexpr int kStages = 3;                     // K ring
 constexpr int kVBufs = 2;                      // V tiles (value norms, pass A)
 constexpr int kGroupRows = 256;
 constexpr int kThreads = 352;
@@ -50,9 +51,15 @@ constexpr int kEpiThreads = 256;
 constexpr int kVWarp = 10;                     // warps 2-9 are the epilogue
 constexpr uint32_t kHalfQ = kGroupRows * 128;  // 32 KB: one 64-dim half of the row tile
 constexpr uint32_t kHalfK = kTile * 128;       // 16 KB
-constexpr uint32_t kStageBytes = 2 * kHalfK;   // 32 KB per K tile
 constexpr uint32_t kSlotCols = 256;
-constexpr uint32_t kSmemBytes = 1024 + 2 * kHalfQ + (kStages + kVBufs) * kStageBytes + 256 + kGroupRows * 4;
+
+template <int kHalves>
+struct Shape {
+  static constexpr int kStages = kHalves == 1 ? 6 : 3;                // K ring
+  static constexpr uint32_t kStageBytes = kHalves * kHalfK;           // one K tile
+  static constexpr uint32_t kSmemBytes =
+      1024 + kHalves * kHalfQ + (kStages + kVBufs) * kStageBytes + 256 + kGroupRows * 4;
+};
 
 struct TcArgs {
   KvDev kv;
@@ -123,11 +130,11 @@ __device__ __forceinline__ int tile_of(const Unit& w, int i) {
 }
 
 struct Smem {
-  uint8_t* q;          // [2 halves][256 rows][128 B]
-  uint8_t* k;          // [kStages][2 halves][128 rows][128 B]
+  uint8_t* q;          // [halves][256 rows][128 B]
+  uint8_t* k;          // [kStages][halves][128 rows][128 B]
   uint64_t* kfull;     // [kStages]
   uint64_t* kempty;    // [kStages]
-  uint8_t* v;          // [kVBufs][2 halves][128 rows][128 B]
+  uint8_t* v;          // [kVBufs][halves][128 rows][128 B]
   uint64_t* vfull;     // [kVBufs]
   uint64_t* vempty;    // [kVBufs]
   uint64_t* tfull;     // [2]
@@ -141,16 +148,18 @@ struct Smem {
   float* lse;          // [256]
 };
 
+template <int kHalves>
 __device__ __forceinline__ Smem carve(uint8_t* raw) {
+  using C = Shape<kHalves>;
   uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(raw) + 1023) & ~uintptr_t(1023));
   Smem s;
   s.q = base;
-  s.k = base + 2 * kHalfQ;
-  s.v = s.k + kStages * kStageBytes;
-  uint8_t* tail = s.v + kVBufs * kStageBytes;
+  s.k = base + kHalves * kHalfQ;
+  s.v = s.k + C::kStages * C::kStageBytes;
+  uint8_t* tail = s.v + kVBufs * C::kStageBytes;
   s.kfull = reinterpret_cast<uint64_t*>(tail);
-  s.kempty = s.kfull + kStages;
-  s.vfull = s.kempty + kStages;
+  s.kempty = s.kfull + C::kStages;
+  s.vfull = s.kempty + C::kStages;
   s.vempty = s.vfull + kVBufs;
   s.tfull = s.vempty + kVBufs;
   s.tempty = s.tfull + 2;
@@ -164,19 +173,6 @@ __device__ __forceinline__ Smem carve(uint8_t* raw) {
 }
 
 // Bounded wait that also gives up when another role has aborted.
-// Non-blocking test of the phase with the given parity (no suspension): for
-// the epilogue's waits on an accumulator slot, which the MMA thread has
-// usually filled already.
-__device__ __forceinline__ bool mbar_probe(uint64_t* bar, uint32_t parity) {
-  uint32_t done;
-  asm volatile(
-      "{\n.reg .pred p;\nmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}\n"
-      : "=r"(done)
-      : "r"(tc::smem_u32(bar)), "r"(parity)
-      : "memory");
-  return done != 0;
-}
-
 __device__ __forceinline__ bool wait_or_abort(uint64_t* bar, uint32_t parity, volatile int* abort) {
   if (tc::mbar_try_wait(bar, parity)) return true;
   const uint64_t t0 = tc::globaltimer_ns();
@@ -201,21 +197,22 @@ __device__ __forceinline__ void epi_barrier() {
 // half of the whole tile (contiguous cache: 2 copies) or of one page (paged
 // cache: 2 x 128/page copies, up to 32), so a paged tile costs one round of
 // parallel page-index loads and copy issues.
+template <int kHalves>
 __device__ __forceinline__ void load_k_tile(const TcArgs& a, const CUtensorMap* kmap, const Unit& w,
                                             uint8_t* dst, uint64_t* bar, int tile, int lane) {
-  if (lane == 0) tc::mbar_arrive_expect_tx(bar, kStageBytes);
+  if (lane == 0) tc::mbar_arrive_expect_tx(bar, kHalves * kHalfK);
   __syncwarp();
   const int tok = tile * kTile;
   const KvDev& kv = a.kv;
-  const int hf = lane & 1;
+  const int hf = lane % kHalves;
   if (kv.page_size == 0) {
-    if (lane < 2) {
+    if (lane < kHalves) {
       const int32_t y = int32_t((int64_t(w.l) * kv.Hkv + w.g) * kv.n_tot + w.t0 + tok);
       tc::tma_load_2d(dst + hf * kHalfK, kmap, bar, hf * 64, y);
     }
   } else {
     const int ps = kv.page_size;
-    const int i = lane >> 1;  // page of the tile
+    const int i = lane / kHalves;  // page of the tile
     if (i < kTile / ps) {
       const int lp = min((tok + i * ps) / ps, (w.N - 1) / ps);  // tail pages repeat the last one (masked)
       const int page = kv.page_table[int64_t(w.r) * kv.max_pages + lp];
@@ -228,10 +225,12 @@ __device__ __forceinline__ void load_k_tile(const TcArgs& a, const CUtensorMap* 
 // Epilogue threads stage scoring rows [row0, row0 + nrows) of the unit into
 // the swizzled row tile (rows at or beyond the group are zero); eight
 // 16-byte loads per thread are in flight at a time.
+template <int kHalves>
 __device__ __forceinline__ void stage_rows(const TcArgs& a, const Unit& w, uint8_t* q_s, int nrows,
                                            int et) {
-  const int G = a.kv.G, Hq = a.kv.Hq;
-  const int total = nrows * 16;
+  constexpr int kChunks = 8 * kHalves;  // 16-byte chunks of a padded row
+  const int G = a.kv.G, Hq = a.kv.Hq, d = a.kv.d;
+  const int total = nrows * kChunks;
   for (int base = 0; base < total; base += kEpiThreads * 8) {
     uint4 val[8];
 #pragma unroll
@@ -239,12 +238,12 @@ __device__ __forceinline__ void stage_rows(const TcArgs& a, const Unit& w, uint8
       const int idx = base + u * kEpiThreads + et;
       val[u] = make_uint4(0u, 0u, 0u, 0u);
       if (idx < total) {
-        const int row = idx >> 4, ch = idx & 15;
-        if (row < w.rows) {
+        const int row = idx / kChunks, ch = idx % kChunks;
+        if (row < w.rows && ch * 8 < d) {
           const int j = w.row0 + row;
           const int h = w.g * G + j / w.nq, qi = j % w.nq;
           val[u] = *reinterpret_cast<const uint4*>(
-              a.q + ((int64_t(w.l) * Hq + h) * a.q_tot + w.q0 + qi) * kD + ch * 8);
+              a.q + ((int64_t(w.l) * Hq + h) * a.q_tot + w.q0 + qi) * d + ch * 8);
         }
       }
     }
@@ -252,7 +251,7 @@ __device__ __forceinline__ void stage_rows(const TcArgs& a, const Unit& w, uint8
     for (int u = 0; u < 8; ++u) {
       const int idx = base + u * kEpiThreads + et;
       if (idx < total) {
-        const int row = idx >> 4, ch = idx & 15;
+        const int row = idx / kChunks, ch = idx % kChunks;
         *reinterpret_cast<uint4*>(q_s + (ch >> 3) * kHalfQ + tc::sw128_offset(row, ch & 7)) = val[u];
       }
     }
@@ -328,11 +327,14 @@ __device__ __forceinline__ float col_sum_sq(const float (&v)[NC], const float* n
   return (ac[0].x + ac[0].y) + (ac[1].x + ac[1].y);
 }
 
+template <int kHalves>
 __global__ void __launch_bounds__(kThreads, 1)
     score_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant__ CUtensorMap vmap,
                     const __grid_constant__ TcArgs a) {
   extern __shared__ uint8_t smem_raw[];
-  const Smem s = carve(smem_raw);
+  constexpr int kStages = Shape<kHalves>::kStages;
+  constexpr uint32_t kStageBytes = Shape<kHalves>::kStageBytes;
+  const Smem s = carve<kHalves>(smem_raw);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (tid == 0) {
     for (int i = 0; i < kStages; ++i) {
@@ -374,7 +376,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           ok = false;
           break;
         }
-        load_k_tile(a, &kmap, w, s.k + st * kStageBytes, &s.kfull[st], tile_of(w, i), lane);
+        load_k_tile<kHalves>(a, &kmap, w, s.k + st * kStageBytes, &s.kfull[st], tile_of(w, i), lane);
       }
     }
     if (lane == 0) s.counters[0] = seq;
@@ -400,7 +402,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           continue;
         }
 #endif
-        load_k_tile(a, &vmap, w, s.v + vb * kStageBytes, &s.vfull[vb], i, lane);
+        load_k_tile<kHalves>(a, &vmap, w, s.v + vb * kStageBytes, &s.vfull[vb], i, lane);
       }
     }
     if (lane == 0) s.counters[2] = vseq;
@@ -409,6 +411,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     uint32_t kseq = 0, tseq = 0, useq = 0;
     bool ok = true;
     const uint32_t qb = tc::smem_u32(s.q);
+    const int ksteps = (a.kv.d + 15) / 16;  // 16-dim steps that are not all padding
     for (int u = blockIdx.x; u < a.n_units && ok; u += gridDim.x) {
       Unit w;
       if (!decode_unit(a, u, w)) continue;
@@ -442,8 +445,9 @@ __global__ void __launch_bounds__(kThreads, 1)
           const uint32_t idesc = tc::idesc_bf16(128, kTile);
           for (int rb = 0; rb < nrb; ++rb) {
 #pragma unroll
-            for (int kk = 0; kk < 8; ++kk) {
-              const uint32_t off = (kk >> 2) * 0 + (kk & 3) * 32;
+            for (int kk = 0; kk < 4 * kHalves; ++kk) {
+              if (kk >= ksteps) break;
+              const uint32_t off = (kk & 3) * 32;
               tc::mma_bf16(d + rb * 128, tc::desc_sw128(qb + (kk >> 2) * kHalfQ + rb * 128 * 128 + off),
                            tc::desc_sw128(kb + (kk >> 2) * kHalfK + off), idesc, kk > 0);
             }
@@ -451,7 +455,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         } else {            // pass B: tokens x rows
           const uint32_t idesc = tc::idesc_bf16(128, ncols);
 #pragma unroll
-          for (int kk = 0; kk < 8; ++kk) {
+          for (int kk = 0; kk < 4 * kHalves; ++kk) {
+            if (kk >= ksteps) break;
             const uint32_t off = (kk & 3) * 32;
             tc::mma_bf16(d, tc::desc_sw128(kb + (kk >> 2) * kHalfK + off),
                          tc::desc_sw128(qb + (kk >> 2) * kHalfQ + off), idesc, kk > 0);
@@ -487,7 +492,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       Unit w;
       if (!decode_unit(a, u, w)) continue;
       const int nrb = (w.rows + 127) / 128;
-      if (ok && !*s.abort) stage_rows(a, w, s.q, nrb * 128, et);
+      if (ok && !*s.abort) stage_rows<kHalves>(a, w, s.q, nrb * 128, et);
       tc::fence_proxy_async_smem();
       epi_barrier();
       if (et == 0) tc::mbar_arrive(s.qready);
@@ -502,7 +507,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       for (int i = 0; i < w.tiles; ++i) {            // pass A
         const int slot = tseq & 1;
         // tcgen05.ld is warp-collective: the whole warp goes on or stops
-        const bool got = __all_sync(0xffffffffu, ok && (mbar_probe(&s.tfull[slot], (tseq >> 1) & 1) ||
+        const bool got = __all_sync(0xffffffffu, ok && (tc::mbar_probe(&s.tfull[slot], (tseq >> 1) & 1) ||
                                                         wait_or_abort(&s.tfull[slot], (tseq >> 1) & 1, s.abort)));
         ++tseq;
         if (!got) {
@@ -525,7 +530,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           tc::tc_fence_before();
           tc::mbar_arrive(&s.tempty[slot]);
         }
-        if (do_norm) {  // half (64 dims) of V row lrow of the tile, from shared memory
+        if (do_norm) {  // chunks [4 kHalves h, 4 kHalves (h + 1)) of V row lrow of the tile, from shared memory
           const int vb = vcons % kVBufs;
           if (!wait_or_abort(&s.vfull[vb], (vcons / kVBufs) & 1, s.abort)) {
             if (!*s.abort) raise_abort(a, s, tc::kSiteLoad);
@@ -533,11 +538,13 @@ __global__ void __launch_bounds__(kThreads, 1)
             continue;
           }
           ++vcons;
-          const uint8_t* vh = s.v + vb * kStageBytes + h * kHalfK;
+          const uint8_t* vt = s.v + vb * kStageBytes;
           float sq[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-          for (int c = 0; c < 8; ++c)
-            sumsq_bf16_chunk(*reinterpret_cast<const uint4*>(vh + tc::sw128_offset(lrow, c)), sq);
+          for (int i8 = 0; i8 < 4 * kHalves; ++i8) {
+            const int c = 4 * kHalves * h + i8;
+            sumsq_bf16_chunk(*reinterpret_cast<const uint4*>(vt + (c >> 3) * kHalfK + tc::sw128_offset(lrow, c & 7)), sq);
+          }
           tc::mbar_arrive(&s.vempty[vb]);
           const int tok = i * kTile + lrow;
           if (tok < w.N) ss_out[tok] = sumsq_combine(sq);
@@ -567,7 +574,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int slot = tseq & 1;
         const int tok = tile_of(w, i) * kTile + lrow;
         // tcgen05.ld is warp-collective: the whole warp goes on or stops
-        const bool got = __all_sync(0xffffffffu, ok && (mbar_probe(&s.tfull[slot], (tseq >> 1) & 1) ||
+        const bool got = __all_sync(0xffffffffu, ok && (tc::mbar_probe(&s.tfull[slot], (tseq >> 1) & 1) ||
                                                         wait_or_abort(&s.tfull[slot], (tseq >> 1) & 1, s.abort)));
         ++tseq;
         if (!got) {
@@ -665,7 +672,7 @@ extern "C" void conduit_test_withhold_v_tile(int32_t n) { g_test_withhold_v = n;
 #endif
 
 bool score_tc_supported(const KvDev& kv) {
-  if (kv.dtype != CONDUIT_BF16 || kv.d != kD) return false;
+  if (kv.dtype != CONDUIT_BF16 || kv.d > kMaxD || !tc_rows_ok(kv)) return false;
   if (kv.page_size != 0 && (kv.page_size % 8 != 0 || kTile % kv.page_size != 0)) return false;
   return true;
 }
@@ -679,8 +686,8 @@ cudaError_t launch_score_tc(const KvDev& kv, const BatchDev& b, const int32_t* q
   EncodeTiledFn enc = encode_fn();
   if (!enc) return cudaErrorNotSupported;
   CUtensorMap kmap, vmap;
-  cuuint64_t dims[2] = {cuuint64_t(kD), 0};
-  cuuint64_t strides[1] = {cuuint64_t(kD) * 2};
+  cuuint64_t dims[2] = {cuuint64_t(kv.d), 0};
+  cuuint64_t strides[1] = {cuuint64_t(kv.d) * 2};
   cuuint32_t box[2] = {64, 0};
   cuuint32_t estr[2] = {1, 1};
   if (kv.page_size == 0) {
@@ -709,7 +716,7 @@ cudaError_t launch_score_tc(const KvDev& kv, const BatchDev& b, const int32_t* q
     units += layers.n * kv.Hkv * n_groups(kv.G * (q_off_host[r + 1] - q_off_host[r]));
   a.n_units = units;
   a.rg_max = rg_max;
-  a.scale_log2 = kLog2e / sqrtf(float(kD));
+  a.scale_log2 = kLog2e / sqrtf(float(kv.d));
   a.pa = pa;
   a.ss = ss;
   a.pa2 = pa2;
@@ -725,12 +732,15 @@ cudaError_t launch_score_tc(const KvDev& kv, const BatchDev& b, const int32_t* q
   cudaError_t err;
   if ((err = cudaGetDevice(&dev))) return err;
   if ((err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev))) return err;
-  if ((err = cudaFuncSetAttribute(score_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  int(kSmemBytes))))
-    return err;
-  score_tc_kernel<<<std::min(units, sms), kThreads, kSmemBytes, stream>>>(kmap, vmap, a);
+  auto launch = [&](auto* f, uint32_t smem) -> cudaError_t {
+    if ((err = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)))) return err;
+    f<<<std::min(units, sms), kThreads, smem, stream>>>(kmap, vmap, a);
+    return cudaGetLastError();
+  };
+  err = kv.d <= 64 ? launch(score_tc_kernel<1>, Shape<1>::kSmemBytes) : launch(score_tc_kernel<2>, Shape<2>::kSmemBytes);
+  if (err) return err;
   count_launches(1);
-  return cudaGetLastError();
+  return cudaSuccess;
 }
 
 }  // namespace conduit

@@ -4,8 +4,8 @@
 // and layer instead of the value rows.
 //   vnorm[l][tg] = sqrt( sum_g sum_part ss_{l,g,part}(t) )
 // The partial sums ss and the order they are added in are those of the
-// scoring pass for the same cache (two 64-element halves per head for the
-// tensor-core kernel, one warp-reduced row per head for the CUDA-core one),
+// scoring pass for the same cache (two half rows per head for the tensor-core
+// kernel, one warp-reduced row per head for the CUDA-core one),
 // so the stored norm is bitwise the one the scoring pass computes from V.
 //
 // Rows are either every token of the batch (mode all) or the selected rows of
@@ -36,11 +36,13 @@ __device__ __forceinline__ void locate(const RowSource& src, const BatchDev& b, 
   }
 }
 
-// bf16, head_dim 128 (the tensor-core scoring kernel's order). Each token
+// bf16, head_dim up to 128 (the tensor-core scoring kernel's order). Each token
 // has a group of S lanes (S = 2 Hkv rounded up to a power of two, at most 32);
-// lane j of the group sums the squares of the 64-element half rows p = j,
-// j + S, ... (p = 2 g + half), and the group's partials are added up in p
-// order by shuffles, every lane of the warp taking part.
+// lane j of the group sums the squares of the row parts p = j, j + S, ... (p =
+// 2 g + part, a part being kChunks 16-byte chunks of the zero-padded row), and
+// the group's partials are added up in p order by shuffles, every lane of the
+// warp taking part.
+template <int kChunks>
 __global__ void __launch_bounds__(256) vnorm_halves_kernel(KvDev kv, BatchDev b, RowSource src,
                                                            int lanes_per_token, float* vnorm) {
   const int l = blockIdx.y;
@@ -53,31 +55,31 @@ __global__ void __launch_bounds__(256) vnorm_halves_kernel(KvDev kv, BatchDev b,
   int64_t tg = 0;
   if (live) locate(src, b, i, r, t, tg);
   const __nv_bfloat16* vb = static_cast<const __nv_bfloat16*>(kv.v);
-  const int halves = 2 * kv.Hkv;
+  const int parts = 2 * kv.Hkv;
   float total = 0.f;
-  for (int p0 = 0; p0 < halves; p0 += S) {  // warp-uniform
+  for (int p0 = 0; p0 < parts; p0 += S) {  // warp-uniform
     const int p = p0 + j;
     float part = 0.f;
-    if (live && p < halves) {
-      const int64_t off = kv.row(l, p >> 1, r, tg, t) + (p & 1) * 64;  // half p & 1 of head p >> 1
-      const uint4* row = reinterpret_cast<const uint4*>(vb + off);
-      uint4 x[8];
+    if (live && p < parts) {
+      const uint4* row = reinterpret_cast<const uint4*>(vb + kv.row(l, p >> 1, r, tg, t));  // of head p >> 1
+      const int c0 = (p & 1) * kChunks, chunks = kv.d / 8;
+      uint4 x[kChunks];
 #pragma unroll
-      for (int c = 0; c < 8; ++c) x[c] = __ldg(row + c);
+      for (int c = 0; c < kChunks; ++c) x[c] = c0 + c < chunks ? __ldg(row + c0 + c) : make_uint4(0u, 0u, 0u, 0u);
       float sq[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-      for (int c = 0; c < 8; ++c) sumsq_bf16_chunk(x[c], sq);
+      for (int c = 0; c < kChunks; ++c) sumsq_bf16_chunk(x[c], sq);
       part = sumsq_combine(sq);
     }
     for (int jj = 0; jj < S; ++jj) {
       const float v = __shfl_sync(0xffffffffu, part, grp * S + jj);
-      if (p0 + jj < halves) total += v;
+      if (p0 + jj < parts) total += v;
     }
   }
   if (live && j == 0) vnorm[int64_t(l) * kv.n_tot + tg] = sqrtf(total);
 }
 
-// Any other cache (fp32, or head_dim != 128): one warp per row, one
+// Any other cache (fp32, or head_dim above 128): one warp per row, one
 // warp-reduced sum per head, heads added in order.
 template <typename T>
 __global__ void __launch_bounds__(256) vnorm_rows_kernel(KvDev kv, BatchDev b, RowSource src,
@@ -107,7 +109,10 @@ cudaError_t launch_value_norms(const KvDev& kv, const BatchDev& b, const int32_t
     while (S < 2 * kv.Hkv && S < 32) S *= 2;
     const int64_t per_block = 8 * (32 / S);  // tokens of a 256-thread block
     const dim3 grid(unsigned((n_rows + per_block - 1) / per_block), kv.L);
-    vnorm_halves_kernel<<<grid, 256, 0, stream>>>(kv, b, src, S, vnorm);
+    if (kv.d <= 64)
+      vnorm_halves_kernel<4><<<grid, 256, 0, stream>>>(kv, b, src, S, vnorm);
+    else
+      vnorm_halves_kernel<8><<<grid, 256, 0, stream>>>(kv, b, src, S, vnorm);
   } else {
     const dim3 grid(unsigned((n_rows + 7) / 8), kv.L);
     if (kv.dtype == CONDUIT_BF16)

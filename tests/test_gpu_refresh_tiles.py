@@ -25,6 +25,8 @@ CASES = [
     (16, 1, 128, (640,), ("tail", 17)),        # all rows in the last key tile
     (6, 2, 128, (129, 128, 127), (0, 128, 3)), # key tiles of 1, 127 and 128 keys; an empty selection
 ]
+# other head sizes: below, at and above the 64-dim half, 16-dim step and 32-byte store boundaries
+HEAD_DIMS = (8, 16, 24, 56, 64, 72, 80, 96, 120)
 
 
 def _positions(spec, n):
@@ -33,7 +35,7 @@ def _positions(spec, n):
     return np.unique(np.linspace(0, n - 1, spec).round().astype(np.int64)) if spec else np.zeros(0, np.int64)
 
 
-def _run(C, hq, hkv, d, n_r, specs, page=0, seed=0):
+def _run(C, hq, hkv, d, n_r, specs, seed=0, form="plain"):
     L, G = 2, hq // hkv
     if len(specs) == 2 and isinstance(specs[0], str):
         specs = (specs,)
@@ -49,7 +51,16 @@ def _run(C, hq, hkv, d, n_r, specs, page=0, seed=0):
     off, off_dev = C.idx_offsets([len(p) for p in pos])
     idx = torch.tensor(np.concatenate(pos), dtype=torch.int32, device="cuda")
     status = torch.zeros(1, dtype=torch.int32, device="cuda")
-    out = C.conduit_refresh_attn(kv, batch, idx, off, off_dev, q_rows, status=status)
+    if form == "plain":
+        out = C.conduit_refresh_attn(kv, batch, idx, off, off_dev, q_rows, status=status)
+    else:  # straight through the ABI: no workspace, or rows that start 2 bytes off a 16-byte boundary
+        shift = 1 if form == "misaligned" else 0
+        hold = [torch.zeros(q_rows.numel() + 8, dtype=torch.bfloat16, device="cuda") for _ in range(2)]
+        q_s, out = (h[shift:shift + q_rows.numel()].view(q_rows.shape) for h in hold)
+        q_s.copy_(q_rows)
+        C._check(C._lib.conduit_refresh_attn(kv.ref(), batch.ref(), C._ptr(idx), C._ptr(off), C._ptr(off_dev),
+                                             C._ptr(q_s), C._ptr(out), None, 0, C._ptr(status),
+                                             C._stream_ptr(None)))
     assert C.conduit_read_status(status) == C.OK
     f = lambda t: t.double().cpu().numpy()
     i0 = 0
@@ -76,3 +87,40 @@ def C():
 def test_item_edges(C, case):
     hq, hkv, d, n_r, specs = CASES[case]
     _run(C, hq, hkv, d, n_r, specs, seed=case)
+
+
+@pytest.mark.parametrize("d", HEAD_DIMS)
+def test_head_dims(C, d):
+    plain = _run(C, 6, 2, d, (300, 141), (44, 17), seed=d)
+    # what a caller without a workspace, or with unaligned rows, gets
+    assert torch.equal(_run(C, 6, 2, d, (300, 141), (44, 17), seed=d, form="no_workspace"), plain)
+    _run(C, 6, 2, d, (300, 141), (44, 17), seed=d, form="misaligned")
+
+
+@pytest.mark.parametrize("d", HEAD_DIMS)
+def test_scores_of_head_dims(C, d):
+    """The scoring pass and the norm side cache at the same head sizes, contiguous and paged."""
+    L, hq, hkv, n_r, nq = 2, 6, 2, (160, 208), (5, 90)   # 15 and 270 scoring rows: one and two row groups
+    tok, qo = [0, 160, 368], [0, 5, 95]
+    rng = torch.Generator(device="cuda").manual_seed(d)
+    draw = lambda *shape: torch.randn(shape, generator=rng, device="cuda").bfloat16()
+    k, v, q = draw(L, hkv, 368, d), draw(L, hkv, 368, d), draw(L, hq, 95, d)
+    batch = C.Batch(tok, [0, 100, 160, 368], [0, 2, 3], qo, device="cuda")
+    pages = k.shape[2] // 16
+    pool = lambda t: t.view(L, hkv, pages, 16, d).transpose(1, 2).contiguous()
+    table = torch.full((2, 13), -1, dtype=torch.int32)
+    table[0, :10], table[1, :13] = torch.arange(10), torch.arange(10, 23)
+    got = []
+    for kv in (C.KvCache(k, v, hq), C.KvCache(pool(k), pool(v), hq, 16, table)):
+        got.append(C.conduit_score(kv, batch, q))
+        vn = C.conduit_value_norms(kv, batch)
+        got.append(C.conduit_score_with_norms(kv, batch, q, vn))
+    for other in got[1:]:
+        assert all(torch.equal(a, b) for a, b in zip(got[0], other))
+    f = lambda t: t.double().cpu().numpy()
+    s, A, g = (f(t) for t in got[0])
+    for r, img in ((0, [0, 100, 160]), (1, [0, 208])):
+        t, qs = slice(tok[r], tok[r + 1]), slice(qo[r], qo[r + 1])
+        want = O.score_request(f(q[:, :, qs]), f(k[:, :, t]), f(v[:, :, t]), img)
+        for a, b in ((s[t], want["s"]), (A[t], want["A"])):   # fp32 sums: 1e-5 relative
+            assert np.all(np.abs(a - b) <= 1e-5 * np.abs(b) + 1e-7 * np.abs(b).max())
