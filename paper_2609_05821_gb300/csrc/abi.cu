@@ -685,7 +685,7 @@ conduit_status conduit_staleness_iso_workspace_size(const conduit_kv* kv, const 
   if (!bytes) return fail(CONDUIT_ERR_INVALID_ARG, "bytes is NULL");
   if ((st = check_batch(batch)) || (st = check_kv(kv, batch))) return st;
   if (M < 1) return fail(CONDUIT_ERR_INVALID_ARG, "M must be >= 1");
-  *bytes = stale_layout(make_kv(kv, batch), make_batch(batch), batch->q_off[batch->num_requests], M).total;
+  *bytes = stale_layout(make_kv(kv, batch), make_batch(batch), batch->q_off, M).total;
   return CONDUIT_OK;
 }
 
@@ -704,7 +704,7 @@ conduit_status conduit_staleness_iso(const conduit_kv* kv, const conduit_batch* 
   const KvDev kd = make_kv(kv, batch);
   const BatchDev bd = make_batch(batch);
   const int32_t q_tot = batch->q_off[batch->num_requests];
-  if ((st = check_workspace(workspace, workspace_bytes, stale_layout(kd, bd, q_tot, M).total))) return st;
+  if ((st = check_workspace(workspace, workspace_bytes, stale_layout(kd, bd, batch->q_off, M).total))) return st;
   cudaError_t err_c = launch_staleness_iso(kd, bd, batch->q_off, q_tot, q, refreshed, z, M, kappa, err,
                                            err_layers, workspace, status,
                                            static_cast<cudaStream_t>(stream));

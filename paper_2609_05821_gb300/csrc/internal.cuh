@@ -171,12 +171,21 @@ cudaError_t launch_value_norms(const KvDev& kv, const BatchDev& b, const int32_t
                                const int32_t* idx_off_dev, int64_t n_rows, float* vnorm,
                                cudaStream_t stream);
 // Isotropic Monte Carlo staleness estimator (App. D): workspace carving and
-// the launcher (M draws of refresh attention over (K, xi^(m)), then ||O||^2).
+// the launcher. On the tensor-core path (tc) one launch takes all draws; else M
+// draws of refresh attention over (K, xi^(m)), then ||O||^2.
 struct StaleLayout {
-  size_t xi, rows, out, pos, part, scale, counter, total;
+  bool tc;
+  int n_blocks;
+  size_t xi, rows, out, pos, part, scale, counter, items, total;
   size_t xi_bytes;
 };
-StaleLayout stale_layout(const KvDev& kv, const BatchDev& b, int32_t q_tot, int M);
+StaleLayout stale_layout(const KvDev& kv, const BatchDev& b, const int32_t* q_off_host, int M);
+// Work items per (layer, KV head, draw) and the launch of `draws` draws starting
+// at z: part gets [draws][L * Hkv][blocks][8] sums of ||O / rowsum||^2.
+int stale_tc_blocks(const KvDev& kv, const BatchDev& b, const int32_t* q_off_host);
+cudaError_t launch_stale_tc(const KvDev& kv, const BatchDev& b, const int32_t* q_off_host, int32_t q_tot,
+                            const void* q, const void* z, int draws, const float* key_scale, double* part,
+                            int32_t* work_counter, int32_t* status, cudaStream_t stream);
 cudaError_t launch_staleness_iso(const KvDev& kv, const BatchDev& b, const int32_t* q_off_host,
                                  int32_t q_tot, const void* q, const uint8_t* refreshed,
                                  const void* z, int M, float kappa, double* err, double* err_rl,

@@ -41,6 +41,14 @@
 // rows a box leaves empty (G not a power of two) no longer take the masking
 // path.
 //
+// The staleness estimator (kStale) runs the same schedule with every scoring row
+// of a request at its last key: V is the draw z itself, the softmax warps scale
+// each V tile by its keys' standard deviations in shared memory while they would
+// wait for their next S (in place of a pass that writes xi = scale z to memory),
+// and a row ends as ||O / rowsum||^2, summed over its warp's rows, instead of an
+// output row. (Scaling P instead costs accuracy: a row's largest weight is then
+// no longer exactly 1.)
+//
 // Rows are sorted by position, so an item needs keys up to its last row's
 // position only (tile A often fewer than tile B). Every barrier phase follows
 // from per-CTA sequence numbers that all roles advance alike. Every wait is
@@ -63,7 +71,7 @@ constexpr int kMmaWarp = 1, kVWarp = 2, kSoftWarp0 = 4;  // warp 0: items and K;
 constexpr int kThreads = 384;
 constexpr uint32_t kHalfBytes = 128 * 128;       // 16 KB: one 64-dim half of a 128-row tile
 constexpr int kRecReaders = 11;                  // two MMA warps, V warp, eight softmax warps
-constexpr uint32_t kBarBytes = 320;             // barriers, TMEM slot, abort flag, counters
+constexpr uint32_t kBarBytes = 384;             // barriers, TMEM slot, abort flag, counters
 constexpr uint32_t kTailBytes = kBarBytes + 2 * (16 + 2 * kRows) * 4;
 
 // Head sizes: kHalves 64-dim halves of a row (one 128-byte swizzled row each;
@@ -78,7 +86,7 @@ struct Shape {
   static constexpr int kDone = 2 * kAhead;
   static constexpr uint32_t kSmem = (2 + kStages) * kTileBytes + kTailBytes;
   static_assert(kSmem <= 232448, "shared memory of one CTA");
-  static_assert((kStages + kDone + 6 + 4 + 4 + 2) * 8 + 32 <= kBarBytes, "barriers and counters");
+  static_assert((kStages + 2 * kDone + 6 + 4 + 4 + 2) * 8 + 32 <= kBarBytes, "barriers and counters");
 };
 constexpr uint32_t kTmemCols = 512;
 constexpr uint32_t kSCols = 128;                 // one S buffer
@@ -103,6 +111,10 @@ struct RefArgs {
   int32_t* next_item;      // work counter, zero at launch; NULL: CTA c takes items c, c + grid, ...
   float scale_log2;
   int32_t* status;
+  // kStale: idx_off holds the requests' query offsets, n_sel the query count
+  int32_t draws;           // n_items = draws * n_blocks * Hkv * L
+  const float* key_scale;  // [L][Hkv][n_tot]
+  double* part;            // [draws][L * Hkv][n_blocks][2 query tiles][4 warps]
 };
 
 // A work item: block `blk` of (layer l, KV head g), counted from the largest
@@ -114,17 +126,24 @@ struct RefArgs {
 // longest-first scheduling; the (layer, head)-major order keeps the CTAs in
 // flight on few K/V prefixes, which L2 then shares when the cache exceeds it.
 struct Item {
-  int l, g, r, i0, cnt;
+  int l, g, r, i0, cnt, m, blk;
 };
 
+template <bool kStale>
 __device__ __forceinline__ Item decode_item(const RefArgs& a, int u) {
   Item it;
   const int n_lg = a.kv.Hkv * a.kv.L;
+  it.m = 0;
+  if (kStale) {  // a (layer, head)'s blocks and draws follow one another: its K stays in L2
+    it.m = u / a.n_blocks % a.draws;
+    u = u / (a.n_blocks * a.draws) * a.n_blocks + u % a.n_blocks;
+  }
   const int x = a.blocks_major ? u / n_lg : u % a.n_blocks;
   const int lg = a.blocks_major ? u % n_lg : u / a.n_blocks;
   it.g = lg % a.kv.Hkv;
   it.l = lg / a.kv.Hkv;
   int blk = a.n_blocks - 1 - x;
+  it.blk = blk;
   it.r = 0;
   it.i0 = 0;
   it.cnt = 0;
@@ -159,11 +178,12 @@ struct Smem {
   volatile int* abort;
   uint32_t* counters;  // [0] K tiles, [1] V tiles loaded
   // per item parity, written by the loader: the decoded item {u (-1: no more
-  // work), l, g, r, i0, rows of A, rows of B, key tiles of A, of B, N_r, t0}
+  // work), l, g, r, i0, rows of A, rows of B, key tiles of A, of B, N_r, t0, m, block}
   // and the positions of its selected rows, so that the other roles read no
   // global memory between items
   volatile int* rec;   // [2][16]
   volatile int* pos;   // [2][2 tiles][kRows]
+  uint64_t* scaled;    // [kDone] (kStale) tile T's V has been scaled
 };
 
 template <int kHalves>
@@ -183,7 +203,8 @@ __device__ __forceinline__ Smem carve(uint8_t* base) {
   s.recfull = s.turn + 2;
   s.recempty = s.recfull + 2;
   s.mdone = s.recempty + 2;
-  s.tmem_slot = reinterpret_cast<uint32_t*>(s.mdone + 2);
+  s.scaled = s.mdone + 2;
+  s.tmem_slot = reinterpret_cast<uint32_t*>(s.scaled + C::kDone);
   s.abort = reinterpret_cast<volatile int*>(s.tmem_slot + 1);
   s.counters = reinterpret_cast<uint32_t*>(s.tmem_slot + 2);
   s.rec = reinterpret_cast<volatile int*>(reinterpret_cast<uint8_t*>(bar) + kBarBytes);
@@ -245,7 +266,7 @@ __device__ __forceinline__ void load_tile(const RefArgs& a, const CUtensorMap* m
 
 // kSplit: P goes to the tensor cores as two bf16 tiles (value and rounding
 // error), which keeps it as precise as fp32 weights for a bf16 result.
-template <int kHalves, bool kSplit>
+template <int kHalves, bool kSplit, bool kStale = false>
 __global__ void __launch_bounds__(kThreads, 1)
     refresh_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant__ CUtensorMap vmap,
                       const __grid_constant__ CUtensorMap qmap, const __grid_constant__ RefArgs a) {
@@ -267,6 +288,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (tid == 0) {
     for (int i = 0; i < kStages; ++i) tc::mbar_init(&s.full[i], 1);
     for (int i = 0; i < kDone; ++i) tc::mbar_init(&s.done[i], 1);
+    for (int i = 0; i < kDone; ++i) tc::mbar_init(&s.scaled[i], 8);  // the softmax warps
     for (int i = 0; i < 2; ++i) {
       tc::mbar_init(&s.sfull[i], 1);
       tc::mbar_init(&s.pfull[i], 4);     // one arrival per softmax warp of the tile
@@ -309,17 +331,18 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (u >= a.n_items) u = -1;
       }
       u = __shfl_sync(0xffffffffu, u, 0);
-      const Item it = decode_item(a, u < 0 ? 0 : u);
+      const Item it = decode_item<kStale>(a, u < 0 ? 0 : u);
       const int cnt_b = min(it.cnt, span), cnt_a = it.cnt - cnt_b;
       const int t0 = a.b.tok_off[it.r], N = a.b.tok_off[it.r + 1] - t0;
       int my_pos[2 * kRows / 32];  // positions of the item's rows, loaded before the record is free
 #pragma unroll
       for (int k = 0; k < 2 * kRows / 32; ++k) {
         const int x = k / (kRows / 32), i = lane + 32 * (k % (kRows / 32));
-        my_pos[k] = (u >= 0 && i < (x ? cnt_b : cnt_a)) ? a.idx[it.i0 + (x ? cnt_a : 0) + i] : -1;
+        my_pos[k] = (!kStale && u >= 0 && i < (x ? cnt_b : cnt_a)) ? a.idx[it.i0 + (x ? cnt_a : 0) + i] : -1;
       }
       auto key_tiles = [&](int first, int cnt) {  // up to the last row's position
         if (u < 0 || cnt == 0) return 0;
+        if (kStale) return (N - 1) / kKT + 1;
         const int p = min(a.idx[it.i0 + first + cnt - 1], N - 1);
         return p < 0 ? 0 : p / kKT + 1;
       };
@@ -330,8 +353,10 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (lane == 0) raise_abort(a, s, tc::kSiteLoad);
         break;
       }
+      if (!kStale) {
 #pragma unroll
-      for (int k = 0; k < 2 * kRows / 32; ++k) s.pos[rs * 2 * kRows + lane + 32 * k] = my_pos[k];
+        for (int k = 0; k < 2 * kRows / 32; ++k) s.pos[rs * 2 * kRows + lane + 32 * k] = my_pos[k];
+      }
       if (lane == 0) {
         volatile int* rec = s.rec + rs * 16;
         rec[0] = u;
@@ -345,6 +370,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         rec[8] = nt;
         rec[9] = N;
         rec[10] = t0;
+        rec[11] = it.m;
+        rec[12] = it.blk;
       }
       __threadfence_block();
       __syncwarp();  // the lanes' positions are ordered before lane 0's release below
@@ -372,7 +399,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         break;
       }
       const volatile int* rec = s.rec + rs * 16;
-      const int u = rec[0], l = rec[1], g = rec[2], r = rec[3], nt = rec[8], N = rec[9], t0 = rec[10];
+      const int u = rec[0], l = rec[1], g = rec[2], r = rec[3], nt = rec[8], N = rec[9], t0 = rec[10], m = rec[11];
       __syncwarp();
       if (lane == 0) tc::mbar_arrive(&s.recempty[rs]);  // this warp is done with the record
       if (u < 0) break;
@@ -383,7 +410,16 @@ __global__ void __launch_bounds__(kThreads, 1)
           ok = false;
           break;
         }
-        load_tile<kHalves>(a, &vmap, s.kv + sl * kTileBytes, &s.full[sl], l, g, r, t0, N, t * kKT, lane);
+        if (kStale) {
+          const int64_t row = (int64_t(l) * kv.Hkv + g) * kv.n_tot + t0;  // of the request's first key
+          const int64_t z_row = int64_t(m) * kv.L * kv.Hkv * kv.n_tot + row + t * kKT;
+          if (lane == 0) tc::mbar_arrive_expect_tx(&s.full[sl], kTileBytes);
+          __syncwarp();
+          if (lane < kHalves)
+            tc::tma_load_2d(s.kv + sl * kTileBytes + lane * kHalfBytes, &vmap, &s.full[sl], lane * 64, int32_t(z_row));
+        } else {
+          load_tile<kHalves>(a, &vmap, s.kv + sl * kTileBytes, &s.full[sl], l, g, r, t0, N, t * kKT, lane);
+        }
       }
     }
     if (lane == 0) s.counters[1] = T;
@@ -406,8 +442,12 @@ __global__ void __launch_bounds__(kThreads, 1)
         uint8_t* dst = s.q + x * kTileBytes;
         tc::mbar_arrive_expect_tx(&s.qfull[x], uint32_t(kHalves) * 128u * uint32_t(span * G));
         for (int hf = 0; hf < kHalves; ++hf)
-          tc::tma_load_3d(dst + hf * kHalfBytes, &qmap, &s.qfull[x], hf * 64, rec[2] * G,
-                          rec[1] * a.n_sel + rec[4] + (x ? rec[5] : 0));
+          if (kStale)
+            tc::tma_load_3d(dst + hf * kHalfBytes, &qmap, &s.qfull[x], hf * 64, rec[4] + (x ? rec[5] : 0),
+                            rec[1] * Hq + rec[2] * G);
+          else
+            tc::tma_load_3d(dst + hf * kHalfBytes, &qmap, &s.qfull[x], hf * 64, rec[2] * G,
+                            rec[1] * a.n_sel + rec[4] + (x ? rec[5] : 0));
       }
       __syncwarp();
       ++nq;
@@ -428,7 +468,9 @@ __global__ void __launch_bounds__(kThreads, 1)
       for (int t = -1; t < nt; ++t, ++turn) {  // a turn: P(t) V(t), then S(t + 1)
         const uint32_t ev = 2 * (T - 1) + 1, slv = ev % kStages, ek = 2 * T, slk = ek % kStages;
         const bool more = t + 1 < nt;
-        if (t >= 0 && !(ok = wait_warp(&s.full[slv], (ev / kStages) & 1, s.abort))) break;
+        if (t >= 0 && !(ok = kStale ? wait_warp(&s.scaled[(T - 1) % kDone], ((T - 1) / kDone) & 1, s.abort)
+                                    : wait_warp(&s.full[slv], (ev / kStages) & 1, s.abort)))
+          break;
         if (more && !(ok = wait_warp(&s.full[slk], (ek / kStages) & 1, s.abort))) break;
         if (!more) {
           if (t < nt_x && !(ok = wait_warp(&s.pfull[x], np & 1, s.abort))) break;
@@ -485,6 +527,37 @@ __global__ void __launch_bounds__(kThreads, 1)
     const uint32_t tl = tmem + (uint32_t(quarter * 32) << 16);
     const uint32_t sb = tl + x * kSCols, ob = tl + kOCol + x * kDP;
     const uint32_t leader = lane == 0, releases = x == 1 && quarter == 0 && lane == 0;
+    uint32_t Tv = 0;                                     // (kStale) the CTA's V tiles
+    // (kStale) this query tile's share of scaling V tile t of the item: thread j
+    // scales its half of row j by the key's deviation
+    auto scale_v = [&](const float* scale, int t, int N) {
+      const int j = t * kKT + row;
+      const float sc = j < N ? scale[j] : 0.f;
+      const uint32_t e = 2 * Tv + 1, sl = e % kStages;
+      if (!wait_warp(&s.full[sl], (e / kStages) & 1, s.abort)) {
+        if (lane == 0) raise_abort(a, s, tc::kSiteLoad);
+        return false;
+      }
+      uint8_t* tile = s.kv + sl * kTileBytes;
+#pragma unroll
+      for (int i8 = 0; i8 < 4 * kHalves; ++i8) {
+        const int c = 4 * kHalves * x + i8;
+        uint4* p = reinterpret_cast<uint4*>(tile + (c >> 3) * kHalfBytes + tc::sw128_offset(row, c & 7));
+        uint4 v = *p;
+        __nv_bfloat162* h = reinterpret_cast<__nv_bfloat162*>(&v);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const float2 f = __bfloat1622float2(h[i]);
+          h[i] = __floats2bfloat162_rn(sc * f.x, sc * f.y);
+        }
+        *p = v;
+      }
+      tc::fence_proxy_async_smem();
+      __syncwarp();
+      tc::mbar_arrive_if(leader, &s.scaled[Tv % kDone]);
+      ++Tv;
+      return true;
+    };
     uint32_t ns = 0, no = 0;                             // S tiles and O tiles read by this query tile
     bool ok = true;
     for (uint32_t n = 0; ok; ++n) {
@@ -495,22 +568,37 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
       const volatile int* rec = s.rec + rs * 16;
       const int u = rec[0], l = rec[1], g = rec[2], cnt = rec[5 + x], nt = rec[7 + x], N = rec[9];
-      const int i0 = rec[4] + (x ? rec[5] : 0);
-      const bool row_ok = u >= 0 && row < cnt * G;
-      const int i_row = i0 + (row_ok ? row / G : 0);
-      const int h_row = g * G + (row_ok ? row % G : 0);
-      // Rows without a position (past the tile or the box, or an index outside
-      // the request) are computed unmasked and never written: a masked row
-      // would send its warp down the masking path on every key tile.
-      int p_row = row_ok ? s.pos[(rs * 2 + x) * kRows + row / G] : -1;
-      const bool live = p_row >= 0 && p_row < N;
-      if (!live) p_row = INT_MAX;
+      const int i0 = rec[4] + (x ? rec[5] : 0), nt_all = rec[8], t0 = rec[10];
+      bool live;
+      int p_row, i_row = 0, h_row = 0;
+      if (kStale) {  // a tile's rows are head major; every row sees every key of the request
+        live = u >= 0 && row < span * G && row % span < cnt;
+        p_row = N - 1;
+        i_row = (rec[11] * kv.L + l) * kv.Hkv + g;
+        h_row = rec[12];
+      } else {
+        // Rows without a position (past the tile or the box, or an index outside
+        // the request) are computed unmasked and never written: a masked row
+        // would send its warp down the masking path on every key tile.
+        const bool row_ok = u >= 0 && row < cnt * G;
+        i_row = i0 + (row_ok ? row / G : 0);
+        h_row = g * G + (row_ok ? row % G : 0);
+        p_row = row_ok ? s.pos[(rs * 2 + x) * kRows + row / G] : -1;
+        live = p_row >= 0 && p_row < N;
+        if (!live) p_row = INT_MAX;
+      }
       __syncwarp();
       tc::mbar_arrive_if(leader, &s.recempty[rs]);
       if (u < 0) break;
 
+      const float* key_scale = nullptr;
+      if (kStale) {
+        key_scale = a.key_scale + (int64_t(l) * kv.Hkv + g) * kv.n_tot + t0;
+        // V(0), or every V tile when no rows of the item are in this query tile
+        for (int t = 0; t < (nt == 0 ? nt_all : 1) && ok; ++t) ok = scale_v(key_scale, t, N);
+      }
       float m_ref = -INFINITY, lsum = 0.f;  // running max (scaled, log2 units) and row sum
-      for (int t = 0; t < nt; ++t, ++ns) {
+      for (int t = 0; t < nt && ok; ++t, ++ns) {
         // the tcgen05.ld below is warp-collective: the whole warp goes on or stops
         if (!wait_warp(&s.sfull[x], ns & 1, s.abort)) {
           if (lane == 0) raise_abort(a, s, tc::kSiteMma);
@@ -583,7 +671,13 @@ __global__ void __launch_bounds__(kThreads, 1)
         // S_B(t) was the last to read K(t) and, in issue order, comes after both
         // P V of the tile before: their slots may be loaded again
         tc::mbar_arrive_if(releases, &s.done[ns % kDone]);
+        if (kStale && t + 1 < nt && !scale_v(key_scale, t + 1, N)) {
+          ok = false;
+          break;
+        }
       }
+      double* const part = kStale ? a.part + ((int64_t(i_row) * a.n_blocks + h_row) * 2 + x) * 4 + quarter : nullptr;
+      if (kStale && nt == 0 && lane == 0) *part = 0.0;  // no rows in this tile
       if (nt == 0 || !ok) continue;
       if (!wait_warp(&s.ofull[x], no & 1, s.abort)) {
         if (lane == 0) raise_abort(a, s, tc::kSiteFinal);
@@ -597,6 +691,25 @@ __global__ void __launch_bounds__(kThreads, 1)
       // them. The next item's P(0) V(0), which overwrites O, waits for a P this
       // warp writes after these loads.
       const float inv = lsum > 0.f ? 1.f / lsum : 0.f;
+      if (kStale) {  // ||O / rowsum||^2 (in the cache's type) over the warp's rows, in a fixed order
+        float ss[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int c = 0; c < kDP; c += 64) {
+          float o[64];
+          tc::tmem_ld64(ob + c, o);
+#pragma unroll
+          for (int i = 0; i < 64; ++i) {
+            const float x1 = __bfloat162float(__float2bfloat16_rn(o[i] * inv));
+            ss[i & 3] = fmaf(x1, x1, ss[i & 3]);
+          }
+        }
+        double row_ss = live ? double((ss[0] + ss[1]) + (ss[2] + ss[3])) : 0.0;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) row_ss += __shfl_xor_sync(0xffffffffu, row_ss, o);
+        if (lane == 0) *part = row_ss;
+        tc::tc_fence_before();
+        continue;
+      }
       __nv_bfloat16* dst = a.out + ((int64_t(l) * a.n_sel + i_row) * Hq + h_row) * d;
 #pragma unroll
       for (int c = 0; c < kDP; c += 64) {
@@ -705,6 +818,14 @@ bool refresh_tc_supported(const KvDev& kv) {
   return true;
 }
 
+// Rows of a (layer, KV head, request) in blocks of two query tiles.
+static int query_blocks(const BatchDev& b, const int32_t* off_host, int rows_per_tile) {
+  int blocks = 0;
+  for (int r = 0; r < b.R; ++r)
+    blocks += (off_host[r + 1] - off_host[r] + 2 * rows_per_tile - 1) / (2 * rows_per_tile);
+  return blocks;
+}
+
 cudaError_t launch_refresh_tc(const KvDev& kv, const BatchDev& b, const int32_t* idx,
                               const int32_t* idx_off_dev, const int32_t* idx_off_host, int32_t n_sel,
                               const void* q_rows, void* out, int32_t* work_counter, int32_t* status,
@@ -723,11 +844,7 @@ cudaError_t launch_refresh_tc(const KvDev& kv, const BatchDev& b, const int32_t*
   a.out32 = (reinterpret_cast<uintptr_t>(out) & 31) == 0 && kv.d % 16 == 0;
   a.n_sel = n_sel;
   a.rows_per_tile = kRows / kv.G;
-  int blocks = 0;
-  for (int r = 0; r < b.R; ++r) {
-    const int kr = idx_off_host[r + 1] - idx_off_host[r];
-    blocks += (kr + 2 * a.rows_per_tile - 1) / (2 * a.rows_per_tile);
-  }
+  const int blocks = query_blocks(b, idx_off_host, a.rows_per_tile);
   a.n_blocks = blocks;
   a.n_items = blocks * kv.Hkv * kv.L;
   a.next_item = work_counter;
@@ -758,6 +875,64 @@ cudaError_t launch_refresh_tc(const KvDev& kv, const BatchDev& b, const int32_t*
     err = launch(refresh_tc_kernel<2, true>, Shape<2>::kSmem);
   else
     err = launch(refresh_tc_kernel<1, true>, Shape<1>::kSmem);
+  if (err) return err;
+  count_launches(1);
+  return cudaSuccess;
+}
+
+int stale_tc_blocks(const KvDev& kv, const BatchDev& b, const int32_t* q_off_host) {
+  return query_blocks(b, q_off_host, kRows / kv.G);
+}
+
+cudaError_t launch_stale_tc(const KvDev& kv, const BatchDev& b, const int32_t* q_off_host, int32_t q_tot,
+                            const void* q, const void* z, int draws, const float* key_scale, double* part,
+                            int32_t* work_counter, int32_t* status, cudaStream_t stream) {
+  CUtensorMap kmap, zmap, qmap;
+  RefArgs a{};
+  a.kv = kv;
+  a.b = b;
+  a.idx_off = b.q_off;
+  a.n_sel = q_tot;
+  a.rows_per_tile = kRows / kv.G;
+  a.n_blocks = query_blocks(b, q_off_host, a.rows_per_tile);
+  a.draws = draws;
+  a.n_items = draws * a.n_blocks * kv.Hkv * kv.L;
+  a.next_item = work_counter;
+  a.scale_log2 = kLog2e / sqrtf(float(kv.d));
+  a.status = status;
+  a.key_scale = key_scale;
+  a.part = part;
+  if (a.n_items == 0) return cudaSuccess;
+  KvDev kz = kv;  // the draws are contiguous whatever the cache is
+  kz.page_size = 0;
+  kz.L = kv.L * draws;
+  EncodeTiledFn enc = encode_fn();
+  if (!enc || !make_map(&kmap, kv, kv.k) || !make_map(&zmap, kz, const_cast<void*>(z))) return cudaErrorInvalidValue;
+  // the scoring queries [L * Hq][q_tot][d]: box (64 dims, rows_per_tile queries, G heads)
+  cuuint64_t dims[3] = {cuuint64_t(kv.d), cuuint64_t(q_tot), cuuint64_t(kv.L) * kv.Hq};
+  cuuint64_t strides[2] = {cuuint64_t(kv.d) * 2, cuuint64_t(q_tot) * kv.d * 2};
+  cuuint32_t box[3] = {64, cuuint32_t(a.rows_per_tile), cuuint32_t(kv.G)};
+  cuuint32_t estr[3] = {1, 1, 1};
+  if (enc(&qmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(q), dims, strides, box, estr,
+          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+    return cudaErrorInvalidValue;
+  int dev = 0, sms = 0;
+  cudaError_t err;
+  if ((err = cudaGetDevice(&dev))) return err;
+  if ((err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev))) return err;
+  if ((err = cudaMemsetAsync(work_counter, 0, sizeof(int32_t), stream))) return err;
+  auto launch = [&](auto* f, uint32_t smem) -> cudaError_t {
+    if ((err = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)))) return err;
+    f<<<std::min(a.n_items, sms), kThreads, smem, stream>>>(kmap, zmap, qmap, a);
+    return cudaGetLastError();
+  };
+  if (kv.d == kMaxD)
+    err = launch(refresh_tc_kernel<2, false, true>, Shape<2>::kSmem);
+  else if (kv.d > 64)
+    err = launch(refresh_tc_kernel<2, true, true>, Shape<2>::kSmem);
+  else
+    err = launch(refresh_tc_kernel<1, true, true>, Shape<1>::kSmem);
   if (err) return err;
   count_launches(1);
   return cudaSuccess;

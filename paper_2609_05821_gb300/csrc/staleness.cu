@@ -5,8 +5,16 @@
 // sum_t alpha_{q,t} xi_t is the attention output of query row q over all the
 // request's visual keys with the values xi (zero for t in T), so each draw m
 // runs the refresh attention kernels with every scoring row at position
-// N_r - 1 over (K, xi^(m)); these kernels build xi^(m) in the cache's own
-// layout, lay the scoring queries out as refresh rows, and reduce ||O||^2.
+// N_r - 1 over (K, xi^(m)). bf16 caches with head_dim up to 128 run all draws
+// in one tensor-core launch (refresh_tc.cu) that reads the draws z and the
+// scoring queries as they are; for the other caches the kernels here build
+// xi^(m) in the cache's own layout, lay the scoring queries out as refresh rows,
+// and reduce ||O||^2.
+// Multi-image prompt, five draws: 2 965 us with a pass over the values, a refresh
+// launch and a 28-block reduction per draw, 1 090 us in one launch (about 970 us
+// of it, bound as the refresh is; the deviations take 85 us).
+#include <algorithm>
+
 #include "internal.cuh"
 
 namespace conduit {
@@ -30,6 +38,70 @@ __global__ void __launch_bounds__(256) stale_scale_kernel(KvDev kv, BatchDev b,
   const T* vb = static_cast<const T*>(kv.v);
   const float ss = warp_row_sumsq(vb + kv.row(lg / kv.Hkv, lg % kv.Hkv, r, tg, t), kv.d, lane);
   if (lane == 0) scale[row] = refreshed[tg] ? 0.f : kappa * sqrtf(ss / float(kv.d));
+}
+
+// The same for bf16 rows of at most 32 16-byte chunks, contiguous lanes of a
+// warp taking the chunks of a row and each lane kRowsPerLane rows, so that enough
+// loads are in flight to stream V.
+constexpr int kRowsPerLane = 4;
+__global__ void __launch_bounds__(256) stale_scale_chunks_kernel(KvDev kv, BatchDev b, const uint8_t* refreshed,
+                                                                 float kappa, int lanes, unsigned blocks_lg,
+                                                                 float* scale) {
+  const int64_t n_tot = kv.n_tot;
+  const int per_warp = 32 / lanes, c = threadIdx.x % lanes, chunks = kv.d / 8;
+  const int lg = int(blockIdx.x / blocks_lg);
+  const int64_t tg0 = (int64_t(blockIdx.x % blocks_lg) * 8 + threadIdx.x / 32) * per_warp * kRowsPerLane +
+                      (threadIdx.x % 32) / lanes;
+  const __nv_bfloat16* vb = static_cast<const __nv_bfloat16*>(kv.v);
+  uint4 x[kRowsPerLane];
+#pragma unroll
+  for (int k = 0; k < kRowsPerLane; ++k) {
+    const int64_t tg = tg0 + k * per_warp;
+    x[k] = make_uint4(0u, 0u, 0u, 0u);
+    if (tg < n_tot && c < chunks) {
+      const int r = request_of(b.tok_off, b.R, tg);
+      const int64_t off = kv.row(lg / kv.Hkv, lg % kv.Hkv, r, tg, int(tg - b.tok_off[r]));
+      x[k] = __ldg(reinterpret_cast<const uint4*>(vb + off) + c);
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < kRowsPerLane; ++k) {
+    const int64_t tg = tg0 + k * per_warp;
+    float sq[4] = {0.f, 0.f, 0.f, 0.f};
+    sumsq_bf16_chunk(x[k], sq);
+    float ss = sumsq_combine(sq);
+    for (int o = lanes / 2; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+    if (c == 0 && tg < n_tot)
+      scale[int64_t(lg) * n_tot + tg] = refreshed[tg] ? 0.f : kappa * sqrtf(ss / float(kv.d));
+  }
+}
+
+// err_rl[r][l] = part sums of (request, layer) / M in a fixed order: part is
+// [M][L * Hkv][n_blocks][8] and request r owns blocks of floor(128/G) x 2
+// queries each, in request order. One block of 256 threads per (layer, request).
+__global__ void __launch_bounds__(256) stale_part_kernel(const double* part, BatchDev b, int L, int Hkv, int M,
+                                                         int n_blocks, int block_rows, double* sums) {
+  __shared__ double warp_s[8];
+  const int l = blockIdx.x, r = blockIdx.y;
+  int blk0 = 0;
+  for (int rr = 0; rr < r; ++rr) blk0 += (b.q_off[rr + 1] - b.q_off[rr] + block_rows - 1) / block_rows;
+  const int nb = (b.q_off[r + 1] - b.q_off[r] + block_rows - 1) / block_rows;
+  const int64_t n = int64_t(M) * Hkv * nb * 8;
+  double a = 0.0;
+  for (int64_t i = threadIdx.x; i < n; i += blockDim.x) {
+    const int64_t mg = i / (nb * 8);
+    const int m = int(mg / Hkv), g = int(mg % Hkv);
+    a += part[((int64_t(m) * L + l) * Hkv + g) * n_blocks * 8 + blk0 * 8 + i % (nb * 8)];
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+  if ((threadIdx.x & 31) == 0) warp_s[threadIdx.x >> 5] = a;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double tot = 0.0;
+    for (int w = 0; w < 8; ++w) tot += warp_s[w];
+    sums[int64_t(r) * L + l] = tot;
+  }
 }
 
 // xi^(m) rows in the layout of kv.v (contiguous or paged): one warp per
@@ -101,24 +173,26 @@ __global__ void __launch_bounds__(256) stale_reduce_kernel(const T* out, BatchDe
   }
 }
 
-// err[r] = sum_l part[r][l] / M, and per layer err_rl[r][l] = part[r][l] / M.
-__global__ void stale_final_kernel(const double* part, int R, int L, int M, double* err,
-                                   double* err_rl) {
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= R) return;
+// err[r] = sum_l part[r][l] / M, and per layer err_rl[r][l] = part[r][l] / M; one
+// warp per request, fixed-order reduction.
+__global__ void __launch_bounds__(32) stale_final_kernel(const double* part, int L, int M, double* err,
+                                                         double* err_rl) {
+  const int r = blockIdx.x;
   double tot = 0.0;
-  for (int l = 0; l < L; ++l) {
+  for (int l = threadIdx.x; l < L; l += 32) {
     const double x = part[int64_t(r) * L + l] / double(M);
     if (err_rl) err_rl[int64_t(r) * L + l] = x;
     tot += x;
   }
-  err[r] = tot;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
+  if (threadIdx.x == 0) err[r] = tot;
 }
 
 }  // namespace
 
-StaleLayout stale_layout(const KvDev& kv, const BatchDev& b, int32_t q_tot, int M) {
-  (void)M;
+StaleLayout stale_layout(const KvDev& kv, const BatchDev& b, const int32_t* q_off_host, int M) {
+  const int32_t q_tot = q_off_host[b.R];
   const size_t esz = kv.dtype == CONDUIT_BF16 ? 2 : 4;
   auto up = [](size_t x) { return (x + 255) / 256 * 256; };
   StaleLayout s{};
@@ -127,6 +201,20 @@ StaleLayout stale_layout(const KvDev& kv, const BatchDev& b, int32_t q_tot, int 
                              : size_t(kv.L) * kv.num_pages * kv.Hkv * size_t(kv.page_size) * kv.d;
   s.xi_bytes = v_elems * esz;
   size_t off = 0;
+  s.tc = refresh_tc_supported(kv);
+  if (s.tc) {  // the key scales, one partial per warp of every work item, the (request, layer) sums, the work counter
+    s.n_blocks = stale_tc_blocks(kv, b, q_off_host);
+    s.scale = off;
+    off += up(size_t(kv.L) * kv.Hkv * size_t(kv.n_tot) * 4);
+    s.items = off;
+    off += up(size_t(M) * kv.L * kv.Hkv * s.n_blocks * 8 * 8);
+    s.part = off;
+    off += up(size_t(b.R) * kv.L * 8);
+    s.counter = off;
+    off += 256;
+    s.total = off;
+    return s;
+  }
   s.xi = off;
   off += up(s.xi_bytes);
   s.rows = off;
@@ -149,7 +237,7 @@ cudaError_t launch_staleness_iso(const KvDev& kv, const BatchDev& b, const int32
                                  int32_t q_tot, const void* q, const uint8_t* refreshed,
                                  const void* z, int M, float kappa, double* err, double* err_rl,
                                  void* workspace, int32_t* status, cudaStream_t stream) {
-  const StaleLayout lay = stale_layout(kv, b, q_tot, M);
+  const StaleLayout lay = stale_layout(kv, b, q_off_host, M);
   char* ws = static_cast<char*>(workspace);
   void* xi = ws + lay.xi;
   void* rows = ws + lay.rows;
@@ -160,6 +248,33 @@ cudaError_t launch_staleness_iso(const KvDev& kv, const BatchDev& b, const int32
   int32_t* counter = reinterpret_cast<int32_t*>(ws + lay.counter);
   const bool bf16 = kv.dtype == CONDUIT_BF16;
   cudaError_t err_c;
+  if (lay.tc) {
+    if (kv.n_tot == 0) return cudaSuccess;
+    int lanes = 1;
+    while (lanes * 8 < kv.d) lanes *= 2;
+    const int64_t per_block = 8 * (32 / lanes) * kRowsPerLane;
+    const unsigned blocks_lg = unsigned((kv.n_tot + per_block - 1) / per_block);
+    stale_scale_chunks_kernel<<<blocks_lg * kv.L * kv.Hkv, 256, 0, stream>>>(kv, b, refreshed, kappa, lanes,
+                                                                             blocks_lg, scale);
+    count_launches(1);
+    if ((err_c = cudaGetLastError())) return err_c;
+    // as many draws per launch as 32-bit row coordinates reach
+    const int64_t rows = int64_t(kv.L) * kv.Hkv * kv.n_tot;
+    const int64_t item_parts = int64_t(kv.L) * kv.Hkv * lay.n_blocks * 8;
+    const int step = int(std::max<int64_t>(1, std::min<int64_t>(M, INT32_MAX / std::max(rows, item_parts))));
+    double* items = reinterpret_cast<double*>(ws + lay.items);
+    for (int m = 0; m < M; m += step)
+      if ((err_c = launch_stale_tc(kv, b, q_off_host, q_tot, q, static_cast<const __nv_bfloat16*>(z) + m * rows * kv.d,
+                                   std::min(step, M - m), scale, items + m * item_parts, counter, status, stream)))
+        return err_c;
+    stale_part_kernel<<<dim3(kv.L, b.R), 256, 0, stream>>>(items, b, kv.L, kv.Hkv, M, lay.n_blocks,
+                                                           2 * (128 / kv.G), part);
+    count_launches(1);
+    if ((err_c = cudaGetLastError())) return err_c;
+    stale_final_kernel<<<b.R, 32, 0, stream>>>(part, kv.L, M, err, err_rl);
+    count_launches(1);
+    return cudaGetLastError();
+  }
   // pool rows that hold no token (a partial last page) stay zero for every draw
   if ((err_c = cudaMemsetAsync(xi, 0, lay.xi_bytes, stream))) return err_c;
   if ((err_c = cudaMemsetAsync(part, 0, size_t(b.R) * kv.L * 8, stream))) return err_c;
@@ -199,10 +314,7 @@ cudaError_t launch_staleness_iso(const KvDev& kv, const BatchDev& b, const int32
     count_launches(1);
     if ((err_c = cudaGetLastError())) return err_c;
     if (q_tot > 0) {
-      err_c = refresh_tc_supported(kx)
-                  ? launch_refresh_tc(kx, b, pos, b.q_off, q_off_host, q_tot, rows, out, counter, status,
-                                      stream)
-                  : launch_refresh_simt(kx, b, pos, b.q_off, q_tot, rows, out, stream);
+      err_c = launch_refresh_simt(kx, b, pos, b.q_off, q_tot, rows, out, stream);
       if (err_c) return err_c;
       const dim3 grid(kv.L, b.R);
       if (bf16)
@@ -215,7 +327,7 @@ cudaError_t launch_staleness_iso(const KvDev& kv, const BatchDev& b, const int32
       if ((err_c = cudaGetLastError())) return err_c;
     }
   }
-  stale_final_kernel<<<(b.R + 127) / 128, 128, 0, stream>>>(part, b.R, kv.L, M, err, err_rl);
+  stale_final_kernel<<<b.R, 32, 0, stream>>>(part, kv.L, M, err, err_rl);
   count_launches(1);
   return cudaGetLastError();
 }
