@@ -331,7 +331,7 @@ conduit_status score_impl(const conduit_kv* kv, const conduit_batch* batch, cons
   if (fused && (err = cudaMemsetAsync(arrivals, 0, size_t(R) * sizeof(int32_t), cs)))
     return cuda_fail(err, "score_select");
   if (lay.tc) {  // the tensor-core kernel also streams V for the value norms (unless normed)
-    err = launch_score_tc(kd, bd, batch->q_off, q, batch->q_off[R], ll, lay.rg_max, pa, ss, pa2,
+    err = launch_score_tc(kd, bd, batch->q_off, max_tok, q, batch->q_off[R], ll, lay.rg_max, pa, ss, pa2,
                           mode.extra_lse, status, cs);
   } else {
     if (!normed && (err = launch_value_sumsq(kd, bd, ll, max_tok, ss, cs)))

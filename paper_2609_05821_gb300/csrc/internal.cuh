@@ -149,7 +149,7 @@ inline bool tc_rows_ok(const KvDev& kv) {
 constexpr int kScoreGroupRows = 256;
 bool score_tc_supported(const KvDev& kv);
 int score_tc_groups(int rows);
-cudaError_t launch_score_tc(const KvDev& kv, const BatchDev& b, const int32_t* q_off_host,
+cudaError_t launch_score_tc(const KvDev& kv, const BatchDev& b, const int32_t* q_off_host, int max_tokens,
                             const void* q, int32_t q_tot, const LayerList& layers, int rg_max,
                             float* pa, float* ss, float* pa2, const float* extra_lse,
                             int32_t* status, cudaStream_t stream);

@@ -1,0 +1,49 @@
+"""Scoring units split over a cluster of two CTAs against the oracle and one CTA.
+
+The library takes two CTAs per unit when that trims the last wave of units, so
+the cases have a little more than one wave of units on a 152-SM GPU: 160 units
+(20 layers x 8 KV heads) of an odd number of key tiles, the last one ragged, and
+of a few tiles. The bar is the 1e-3 of tests/parity.py for bf16 scores; the split
+itself only adds a rounding of each row's log2-sum-exp, so 1e-5 is asked for.
+"""
+
+import numpy as np
+import pytest
+import torch
+
+from oracle import conduit_oracle as O
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def C():
+    from paper_2609_05821_gb300 import _build
+    _build.build()
+    from paper_2609_05821_gb300 import conduit
+    return conduit
+
+
+@pytest.mark.parametrize("n,nq,d,extra", [(3713, 4, 128, False), (3713, 40, 128, True), (2049, 3, 64, False),
+                                          (2900, 5, 128, False)])
+def test_split_units(C, n, nq, d, extra):
+    L, hq, hkv = 20, 16, 8
+    gen = torch.Generator(device="cuda").manual_seed(n + nq)
+    draw = lambda *shape: torch.randn(shape, generator=gen, device="cuda").bfloat16()
+    k, v, q = draw(L, hkv, n, d), draw(L, hkv, n, d), draw(L, hq, nq, d)
+    batch = C.Batch([0, n], [0, n // 3, n], [0, 2], [0, nq], device="cuda")
+    kv = C.KvCache(k, v, hq)
+    lse = torch.randn((L, hq, nq), generator=gen, device="cuda") + 8.0 if extra else None
+    s, A, g = C.conduit_score_ex(kv, batch, q, extra_lse=lse)
+    again = C.conduit_score_ex(kv, batch, q, extra_lse=lse)
+    assert all(torch.equal(a, b) for a, b in zip((s, A, g), again))
+    f = lambda t: t.double().cpu().numpy()
+    kw = {} if lse is None else {"extra_lse": f(lse)}
+    want = O.score_request(f(q), f(k), f(v), [0, n // 3, n], **kw)
+    for got, ref in ((s, want["s"]), (A, want["A"]), (g, want["g"])):
+        assert np.all(np.abs(f(got) - ref) <= 1e-5 * np.abs(ref) + 1e-7 * np.abs(ref).max())
+    # a NaN in one CTA's keys reaches the rows' weights in the other's
+    k[:, :, 5] = float("nan")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    s, _, _ = C.conduit_score(kv, batch, q, status=status)
+    assert torch.isnan(s).all() and C.conduit_read_status(status) == C.ERR_NONFINITE
