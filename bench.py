@@ -224,11 +224,9 @@ def call_kernels(pipe) -> dict:
         score = (["score_tc_kernel"] + tail, "hbm", "score_tc.cu")
         refresh = (["refresh_tc_kernel"], "tensor", "refresh_tc.cu")
     else:
-        score = (["value_sumsq_kernel", "rowstats_kernel", "colsum_kernel"] + tail, "alu", "score_simt.cu")
+        score = (["rowstats_kernel", "colsum_kernel"] + tail, "alu", "score_simt.cu")
         refresh = (["refresh_simt_kernel"], "alu", "refresh_simt.cu")
     norms = (["vnorm_halves_kernel" if tc else "vnorm_rows_kernel"], "hbm", "vnorm.cu")
-    if pipe.value_norm != "v" and not tc:  # no separate value pass
-        score = (["rowstats_kernel", "colsum_kernel"] + tail, "alu", "score_simt.cu")
     sel = ["quota_kernel", "select_kernel"] if pipe.selection == "quota" else ["select_kernel"]
     # conduit_score_select_topk: the scoring kernels, then one launch for the
     # tail and the selection when every request holds at most 8192 tokens

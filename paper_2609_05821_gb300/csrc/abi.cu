@@ -148,6 +148,7 @@ struct ScoreLayout {
   int rg_max;  // row groups per slab (column-sum partials per KV head)
   int group_rows;
   int parts;   // partials per row group and per value norm (2 for the tensor-core kernel)
+  int chunks;  // key chunks of the CUDA-core row statistics
   size_t stats, pa, pa2, ss, attn, total;
 };
 
@@ -196,7 +197,15 @@ ScoreLayout score_layout(const conduit_kv* kv, const conduit_batch* b, int n_lay
   const int64_t total_rows = int64_t(n_layers) * kv->num_q_heads * int64_t(q_tot);
   size_t off = 0;
   s.stats = off;
-  if (!s.tc) off += align_up(size_t(total_rows) * sizeof(float2));  // (max, sum) per row
+  if (!s.tc) {  // (max, sum) per row and key chunk
+    int max_tok = 0, rows = 0;
+    for (int r = 0; r < R; ++r) {
+      max_tok = std::max(max_tok, b->tok_off[r + 1] - b->tok_off[r]);
+      rows += kv->num_q_heads / kv->num_kv_heads * (b->q_off[r + 1] - b->q_off[r]);
+    }
+    s.chunks = score_simt_chunks(make_kv(kv, b), n_layers, rows, max_tok);
+    off += align_up(size_t(total_rows) * s.chunks * sizeof(float2));
+  }
   const size_t pa_bytes =
       align_up(size_t(n_layers) * kv->num_kv_heads * s.rg_max * s.parts * n_tot * sizeof(float));
   s.pa = off;
@@ -334,10 +343,8 @@ conduit_status score_impl(const conduit_kv* kv, const conduit_batch* batch, cons
     err = launch_score_tc(kd, bd, batch->q_off, max_tok, q, batch->q_off[R], ll, lay.rg_max, pa, ss, pa2,
                           mode.extra_lse, status, cs);
   } else {
-    if (!normed && (err = launch_value_sumsq(kd, bd, ll, max_tok, ss, cs)))
-      return cuda_fail(err, "value_sumsq");
-    err = launch_score_simt(kd, bd, q, batch->q_off[R], ll, max_rows, max_tok, stats, pa, pa2,
-                            mode.extra_lse, cs);
+    err = launch_score_simt(kd, bd, q, batch->q_off[R], ll, max_rows, max_tok, lay.chunks, stats, pa, pa2,
+                            mode.extra_lse, ss, cs);
   }
   if (err) return cuda_fail(err, "score");
   if (fused) {
@@ -673,7 +680,7 @@ conduit_status conduit_refresh_attn(const conduit_kv* kv, const conduit_batch* b
       tc ? launch_refresh_tc(kd, make_batch(batch), idx, idx_off_dev, idx_off, n_sel, q_rows, out,
                              counter, status,
                              static_cast<cudaStream_t>(stream))
-         : launch_refresh_simt(kd, make_batch(batch), idx, idx_off_dev, n_sel, q_rows, out,
+         : launch_refresh_simt(kd, make_batch(batch), idx, idx_off_dev, idx_off, n_sel, q_rows, out,
                                static_cast<cudaStream_t>(stream));
   if (err) return cuda_fail(err, "refresh_attn");
   return CONDUIT_OK;

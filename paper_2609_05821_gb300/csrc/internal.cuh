@@ -128,14 +128,14 @@ void count_launches(int n);
 // ------------------------------------------------------------------ launchers
 // Each returns a cudaError_t from the launch (cudaGetLastError) and enqueues
 // on `stream`.
-cudaError_t launch_value_sumsq(const KvDev& kv, const BatchDev& b, const LayerList& layers,
-                               int max_tokens, float* ss, cudaStream_t stream);
-// pa2 (sums of alpha^2, RMS statistic) and extra_lse ([L][Hq][q_tot] natural-log
-// log-sum-exp of each scoring row over keys outside the visual span) may be NULL.
+// pa2 (sums of alpha^2, RMS statistic), extra_lse ([L][Hq][q_tot] natural-log
+// log-sum-exp of each scoring row over keys outside the visual span) and ss (value
+// sums of squares) may be NULL. stats holds (max, sum) of every scoring row for up
+// to `chunks` = score_simt_chunks(...) chunks of keys.
+int score_simt_chunks(const KvDev& kv, int n_layers, int rows, int max_tokens);
 cudaError_t launch_score_simt(const KvDev& kv, const BatchDev& b, const void* q, int32_t q_tot,
-                              const LayerList& layers, int max_rows, int max_tokens,
-                              float2* stats, float* pa, float* pa2, const float* extra_lse,
-                              cudaStream_t stream);
+                              const LayerList& layers, int max_rows, int max_tokens, int chunks, float2* stats,
+                              float* pa, float* pa2, const float* extra_lse, float* ss, cudaStream_t stream);
 // The tensor-core kernels address cache rows with 32-bit tensor-map coordinates.
 inline bool tc_rows_ok(const KvDev& kv) {
   const int64_t rows = kv.page_size == 0 ? kv.n_tot : int64_t(kv.num_pages) * kv.page_size;
@@ -240,7 +240,7 @@ cudaError_t launch_refresh_tc(const KvDev& kv, const BatchDev& b, const int32_t*
                               const void* q_rows, void* out, int32_t* work_counter, int32_t* status,
                               cudaStream_t stream);
 cudaError_t launch_refresh_simt(const KvDev& kv, const BatchDev& b, const int32_t* idx,
-                                const int32_t* idx_off_dev, int32_t n_sel, const void* q_rows,
-                                void* out, cudaStream_t stream);
+                                const int32_t* idx_off_dev, const int32_t* idx_off_host, int32_t n_sel,
+                                const void* q_rows, void* out, cudaStream_t stream);
 
 }  // namespace conduit

@@ -2,277 +2,230 @@
 //
 // Conduit Eq. 6 needs, per (request, layer, KV head g), the softmax over all
 // N_r visual keys of every scoring row (query head h of group g, query q):
-//   pass 1  row statistics: m = max_t x_t and Z = sum_t 2^(x_t - m), with
-//           x = <q, k_t> log2(e) / sqrt(d) (the log2 domain keeps exp2 exact
-//           to the same softmax);
-//   pass 2  column sums pa[l][g][t] = sum_rows 2^(x_t - m - log2 Z), i.e. the
-//           sum over the group's heads and the span of alpha_{q,t}.
-// Value norms (Sec. 3.3, concatenated heads) are a separate streaming
-// reduction ss[l][t] = sum_g sum_e V[l][g][t][e]^2.
+//   pass 1  row statistics over chunks of the keys: m = max_t x_t and Z = sum_t
+//           2^(x_t - m), with x = <q, k_t> log2(e) / sqrt(d) (the log2 domain
+//           keeps exp2 exact to the same softmax);
+//   pass 2  column sums pa[l][g][t] = sum_rows 2^(x_t - lse), lse the rows'
+//           log2-sum-exp merged over the chunks: the sum over the group's heads
+//           and the span of alpha_{q,t}. The same blocks reduce their tokens' value
+//           rows, ss[l][g][t] = sum_e V[l][g][t][e]^2 (Sec. 3.3, concatenated heads).
+// Pass 1 splits the keys into chunks because a small call has few row blocks: on
+// one layer, 2 KV heads, 32 rows and 256 keys two blocks walked all keys in 59 us
+// (fp32, 64 dims); four chunks each take 7 us, and pass 2 with the norms
+// 13.4 us (14 + 4.6 us in two launches before).
 // All reductions run in a fixed order, so results are deterministic.
-#include "internal.cuh"
+#include <algorithm>
+
+#include "simt_tile.cuh"
 
 namespace conduit {
 namespace {
 
-constexpr int kRowBlock = 32;   // scoring rows per CTA block
-constexpr int kTokTile = 32;    // tokens per tile
-constexpr int kThreads = 256;   // 32 rows x 8 token lanes
+using namespace simt;
 
-template <typename T>
-__device__ __forceinline__ void load_rows_to_smem(float* dst, int ld, const T* src_base,
-                                                  const int64_t* row_off, int nrows, int d) {
-  // row_off[i] < 0 marks a missing row (filled with zeros)
-  for (int idx = threadIdx.x; idx < nrows * d; idx += blockDim.x) {
-    const int i = idx / d, e = idx % d;
-    const int64_t off = row_off[i];
-    dst[i * ld + e] = off >= 0 ? to_float(src_base[off + e]) : 0.f;
-  }
-}
-
-// Pass 1: one CTA per (row block, layer*Hkv + g, request); sweeps all tokens.
-template <typename T>
-__global__ void __launch_bounds__(kThreads) rowstats_kernel(KvDev kv, BatchDev b, const T* q,
-                                                            int32_t q_tot, LayerList layers,
-                                                            float2* stats) {
-  extern __shared__ float smem[];
-  const int d = kv.d, ld = d + 1;
-  float* q_s = smem;                       // [32][d+1]
-  float* k_s = smem + kRowBlock * ld;      // [32][d+1]
-  __shared__ int64_t q_off_s[kRowBlock], k_off_s[kTokTile];
-
-  const int r = blockIdx.z;
-  const int li = blockIdx.y / kv.Hkv, g = blockIdx.y % kv.Hkv;
-  const int l = layers.ids[li];
-  const int q0 = b.q_off[r], nq = b.q_off[r + 1] - q0;
-  const int R = kv.G * nq;
-  const int row0 = blockIdx.x * kRowBlock;
-  if (row0 >= R || nq == 0) return;
-  const int t0 = b.tok_off[r], N = b.tok_off[r + 1] - t0;
-
-  if (threadIdx.x < kRowBlock) {
+// Scoring rows [row0, row0 + 32) of slab (l, g, r) as element offsets into q.
+__device__ __forceinline__ void row_offsets(const KvDev& kv, int l, int g, int q0, int nq, int32_t q_tot, int row0,
+                                            int64_t* off) {
+  if (threadIdx.x < kRowTile) {
     const int rr = row0 + threadIdx.x;
-    int64_t off = -1;
-    if (rr < R) {
-      const int h = g * kv.G + rr / nq, qi = rr % nq;
-      off = ((int64_t(l) * kv.Hq + h) * q_tot + q0 + qi) * d;
-    }
-    q_off_s[threadIdx.x] = off;
-  }
-  __syncthreads();
-  load_rows_to_smem(q_s, ld, q, q_off_s, kRowBlock, d);
-
-  const int i = threadIdx.x / 8, j = threadIdx.x % 8;
-  const float scale = kLog2e * rsqrtf(float(d));
-  float m_run = -INFINITY, z_run = 0.f;
-  const T* kbase = static_cast<const T*>(kv.k);
-
-  for (int tt = 0; tt < N; tt += kTokTile) {
-    __syncthreads();
-    if (threadIdx.x < kTokTile) {
-      const int t = tt + threadIdx.x;
-      k_off_s[threadIdx.x] = t < N ? kv.row(l, g, r, int64_t(t0) + t, t) : -1;
-    }
-    __syncthreads();
-    load_rows_to_smem(k_s, ld, kbase, k_off_s, kTokTile, d);
-    __syncthreads();
-    float x[4];
-#pragma unroll
-    for (int m = 0; m < 4; ++m) x[m] = 0.f;
-    for (int e = 0; e < d; ++e) {
-      const float qe = q_s[i * ld + e];
-#pragma unroll
-      for (int m = 0; m < 4; ++m) x[m] = fmaf(qe, k_s[(j + 8 * m) * ld + e], x[m]);
-    }
-    float tmax = -INFINITY;
-#pragma unroll
-    for (int m = 0; m < 4; ++m) {
-      x[m] = (tt + j + 8 * m < N) ? x[m] * scale : -INFINITY;
-      tmax = fmaxf(tmax, x[m]);
-    }
-    tmax = fmaxf(tmax, __shfl_xor_sync(0xffffffffu, tmax, 1));
-    tmax = fmaxf(tmax, __shfl_xor_sync(0xffffffffu, tmax, 2));
-    tmax = fmaxf(tmax, __shfl_xor_sync(0xffffffffu, tmax, 4));
-    const float m_new = fmaxf(m_run, tmax);
-    float psum = 0.f;
-#pragma unroll
-    for (int m = 0; m < 4; ++m) psum += exp2f(x[m] - m_new);
-    psum += __shfl_xor_sync(0xffffffffu, psum, 1);
-    psum += __shfl_xor_sync(0xffffffffu, psum, 2);
-    psum += __shfl_xor_sync(0xffffffffu, psum, 4);
-    z_run = z_run * exp2f(m_run - m_new) + psum;
-    m_run = m_new;
-  }
-  const int rr = row0 + i;
-  if (j == 0 && rr < R) {
-    const int64_t base = int64_t(blockIdx.y) * kv.G * q_tot + int64_t(kv.G) * q0;
-    stats[base + rr] = make_float2(m_run, z_run);
+    off[threadIdx.x] =
+        rr < kv.G * nq ? ((int64_t(l) * kv.Hq + g * kv.G + rr / nq) * q_tot + q0 + rr % nq) * kv.d : -1;
   }
 }
 
-// Pass 2: one CTA per (token tile, layer*Hkv + g, request); loops over all
-// row blocks of the slab and writes the complete column sums of its tile.
+__device__ __forceinline__ void key_offsets(const KvDev& kv, int l, int g, int r, int t0, int N, int tt, int64_t* off) {
+  if (threadIdx.x < kKeyTile) {
+    const int t = tt + threadIdx.x;
+    off[threadIdx.x] = t < N ? kv.row(l, g, r, int64_t(t0) + t, t) : -1;
+  }
+}
+
+// Pass 1: one CTA per (row block x key chunk, layer * Hkv + g, request); writes
+// (max, sum) of its rows over its chunk to stats[chunk][l][h][q].
 template <typename T>
-__global__ void __launch_bounds__(kThreads) colsum_kernel(KvDev kv, BatchDev b, const T* q,
-                                                          int32_t q_tot, LayerList layers,
-                                                          const float2* stats, float* pa,
-                                                          float* pa2, const float* extra_lse) {
-  extern __shared__ float smem[];
-  const int d = kv.d, ld = d + 1;
-  float* q_s = smem;
-  float* k_s = smem + kRowBlock * ld;
-  __shared__ int64_t q_off_s[kRowBlock], k_off_s[kTokTile];
-  __shared__ float lse_s[kRowBlock];
-  __shared__ float red_s[kThreads / 32][kTokTile];
-  __shared__ float red2_s[kThreads / 32][kTokTile];
+__global__ void __launch_bounds__(kThreads) rowstats_kernel(KvDev kv, BatchDev b, const T* q, int32_t q_tot,
+                                                            const __grid_constant__ LayerList layers, int chunk_keys,
+                                                            int chunks, float2* stats) {
+  extern __shared__ __align__(16) float smem[];
+  const int d = kv.d;
+  float* q_s = smem;                                 // [32][d + 4]
+  float* k_s = smem + kRowTile * row_stride(d);      // [64][d + 4]
+  __shared__ int64_t q_off_s[kRowTile], k_off_s[kKeyTile];
 
   const int r = blockIdx.z;
-  const int li = blockIdx.y / kv.Hkv, g = blockIdx.y % kv.Hkv;
-  const int l = layers.ids[li];
+  const int li = blockIdx.y / kv.Hkv, g = blockIdx.y % kv.Hkv, l = layers.ids[li];
+  const int q0 = b.q_off[r], nq = b.q_off[r + 1] - q0, R = kv.G * nq;
+  const int chunk = blockIdx.x % chunks, row0 = int(blockIdx.x / chunks) * kRowTile;
+  if (row0 >= R) return;
   const int t0 = b.tok_off[r], N = b.tok_off[r + 1] - t0;
-  const int tt = blockIdx.x * kTokTile;
-  if (tt >= N) return;
-  const int q0 = b.q_off[r], nq = b.q_off[r + 1] - q0;
-  const int R = kv.G * nq;
-  const int64_t sbase = int64_t(blockIdx.y) * kv.G * q_tot + int64_t(kv.G) * q0;
+  const int t_end = min(N, (chunk + 1) * chunk_keys);
 
-  if (threadIdx.x < kTokTile) {
-    const int t = tt + threadIdx.x;
-    k_off_s[threadIdx.x] = t < N ? kv.row(l, g, r, int64_t(t0) + t, t) : -1;
-  }
+  row_offsets(kv, l, g, q0, nq, q_tot, row0, q_off_s);
   __syncthreads();
-  load_rows_to_smem(k_s, ld, static_cast<const T*>(kv.k), k_off_s, kTokTile, d);
-
-  const int i = threadIdx.x / 8, j = threadIdx.x % 8;
-  const float scale = kLog2e * rsqrtf(float(d));
-  float acc[4] = {0.f, 0.f, 0.f, 0.f};
-  float acc2[4] = {0.f, 0.f, 0.f, 0.f};
-
-  for (int row0 = 0; row0 < R; row0 += kRowBlock) {
+  load_rows(q_s, q, q_off_s, kRowTile, d, kLog2e * rsqrtf(float(d)));
+  const int i = threadIdx.x / 16, j = threadIdx.x % 16;
+  float m_run[2] = {-INFINITY, -INFINITY}, z_run[2] = {0.f, 0.f};
+  for (int tt = chunk * chunk_keys; tt < t_end; tt += kKeyTile) {
     __syncthreads();
-    if (threadIdx.x < kRowBlock) {
+    key_offsets(kv, l, g, r, t0, N, tt, k_off_s);
+    __syncthreads();
+    load_rows(k_s, static_cast<const T*>(kv.k), k_off_s, kKeyTile, d, 1.f);
+    __syncthreads();
+    float x[2][4];
+    dots(q_s, k_s, d, x);
+#pragma unroll
+    for (int a = 0; a < 2; ++a) {
+      float tmax = -INFINITY;
+#pragma unroll
+      for (int m = 0; m < 4; ++m) {
+        if (tt + j + 16 * m >= N) x[a][m] = -INFINITY;
+        tmax = fmaxf(tmax, x[a][m]);
+      }
+      const float m_new = fmaxf(m_run[a], lanes_max(tmax));
+      float psum = 0.f;
+#pragma unroll
+      for (int m = 0; m < 4; ++m) psum += exp2f(x[a][m] - m_new);
+      z_run[a] = z_run[a] * exp2f(m_run[a] - m_new) + lanes_sum(psum);
+      m_run[a] = m_new;
+    }
+  }
+  if (j < 2) {
+    const int rr = row0 + 2 * i + j;
+    const int64_t rows_all = int64_t(gridDim.y) * kv.G * q_tot;  // of one chunk
+    if (rr < R)
+      stats[chunk * rows_all + int64_t(blockIdx.y) * kv.G * q_tot + int64_t(kv.G) * q0 + rr] =
+          make_float2(j ? m_run[1] : m_run[0], j ? z_run[1] : z_run[0]);
+  }
+}
+
+// Pass 2: one CTA per (64 tokens, layer * Hkv + g, request); loops over all row
+// blocks of the slab and writes the complete column sums of its tokens, and their
+// value sums of squares when ss is not NULL.
+template <typename T>
+__global__ void __launch_bounds__(kThreads) colsum_kernel(KvDev kv, BatchDev b, const T* q, int32_t q_tot,
+                                                          const __grid_constant__ LayerList layers, int chunk_keys,
+                                                          int chunks, const float2* stats, float* pa, float* pa2,
+                                                          const float* extra_lse, float* ss) {
+  extern __shared__ __align__(16) float smem[];
+  const int d = kv.d;
+  float* q_s = smem;
+  float* k_s = smem + kRowTile * row_stride(d);
+  __shared__ int64_t q_off_s[kRowTile], k_off_s[kKeyTile];
+  __shared__ float lse_s[kRowTile];
+  __shared__ float red_s[kRowTile / 2][kKeyTile + 1];
+
+  const int r = blockIdx.z;
+  const int li = blockIdx.y / kv.Hkv, g = blockIdx.y % kv.Hkv, l = layers.ids[li];
+  const int t0 = b.tok_off[r], N = b.tok_off[r + 1] - t0;
+  const int tt = blockIdx.x * kKeyTile;
+  if (tt >= N) return;
+  const int q0 = b.q_off[r], nq = b.q_off[r + 1] - q0, R = kv.G * nq;
+  const int64_t rows_all = int64_t(gridDim.y) * kv.G * q_tot;
+  const float2* st_slab = stats + int64_t(blockIdx.y) * kv.G * q_tot + int64_t(kv.G) * q0;
+  const int64_t out0 = int64_t(blockIdx.y) * kv.n_tot + t0 + tt;
+
+  key_offsets(kv, l, g, r, t0, N, tt, k_off_s);
+  __syncthreads();
+  load_rows(k_s, static_cast<const T*>(kv.k), k_off_s, kKeyTile, d, 1.f);
+  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+  if (ss != nullptr) {
+    for (int t = warp; t < kKeyTile && tt + t < N; t += kThreads / 32) {
+      const float acc = warp_row_sumsq(static_cast<const T*>(kv.v) + k_off_s[t], d, lane);
+      if (lane == 0) ss[out0 + t] = acc;
+    }
+  }
+
+  const int i = threadIdx.x / 16, j = threadIdx.x % 16;
+  const int n_chunks = (N + chunk_keys - 1) / chunk_keys;
+  float acc[4] = {0.f, 0.f, 0.f, 0.f}, acc2[4] = {0.f, 0.f, 0.f, 0.f};
+  for (int row0 = 0; row0 < R; row0 += kRowTile) {
+    __syncthreads();
+    row_offsets(kv, l, g, q0, nq, q_tot, row0, q_off_s);
+    if (threadIdx.x < kRowTile) {
       const int rr = row0 + threadIdx.x;
-      int64_t off = -1;
       float lse = 0.f;
       if (rr < R) {
-        const int h = g * kv.G + rr / nq, qi = rr % nq;
-        off = ((int64_t(l) * kv.Hq + h) * q_tot + q0 + qi) * d;
-        const float2 st = stats[sbase + rr];
-        lse = st.x + log2f(st.y);
-        if (extra_lse)  // full-context softmax: keys outside the visual span join the denominator
+        float m = -INFINITY, z = 0.f;  // (max, sum) over the chunks, in order
+        for (int c = 0; c < n_chunks; ++c) m = fmaxf(m, st_slab[c * rows_all + rr].x);
+        for (int c = 0; c < n_chunks; ++c) {
+          const float2 st = st_slab[c * rows_all + rr];
+          z += n_chunks == 1 ? st.y : st.y * exp2f(st.x - m);
+        }
+        lse = m + log2f(z);
+        if (extra_lse) {  // full-context softmax: keys outside the visual span join the denominator
+          const int h = g * kv.G + rr / nq, qi = rr % nq;
           lse = log2_add(lse, extra_lse[(int64_t(l) * kv.Hq + h) * q_tot + q0 + qi] * kLog2e);
+        }
       }
-      q_off_s[threadIdx.x] = off;
       lse_s[threadIdx.x] = lse;
     }
     __syncthreads();
-    load_rows_to_smem(q_s, ld, q, q_off_s, kRowBlock, d);
+    load_rows(q_s, q, q_off_s, kRowTile, d, kLog2e * rsqrtf(float(d)));
     __syncthreads();
-    float x[4] = {0.f, 0.f, 0.f, 0.f};
-    for (int e = 0; e < d; ++e) {
-      const float qe = q_s[i * ld + e];
-#pragma unroll
-      for (int m = 0; m < 4; ++m) x[m] = fmaf(qe, k_s[(j + 8 * m) * ld + e], x[m]);
-    }
-    const bool row_ok = row0 + i < R;
-    const float lse = lse_s[i];
+    float x[2][4];
+    dots(q_s, k_s, d, x);
+    const float lse0 = lse_s[2 * i], lse1 = lse_s[2 * i + 1];
+    const bool ok0 = row0 + 2 * i < R, ok1 = row0 + 2 * i + 1 < R;  // rows past the last add nothing
 #pragma unroll
     for (int m = 0; m < 4; ++m) {
-      float p = (row_ok && tt + j + 8 * m < N) ? exp2f(x[m] * scale - lse) : 0.f;
-      float p2 = p * p;
-      // sum over the 4 rows of this warp that share token lane j
-      p += __shfl_xor_sync(0xffffffffu, p, 8);
-      p += __shfl_xor_sync(0xffffffffu, p, 16);
-      acc[m] += p;
-      if (pa2) {
-        p2 += __shfl_xor_sync(0xffffffffu, p2, 8);
-        p2 += __shfl_xor_sync(0xffffffffu, p2, 16);
-        acc2[m] += p2;
-      }
+      const float p0 = ok0 ? exp2f(x[0][m] - lse0) : 0.f, p1 = ok1 ? exp2f(x[1][m] - lse1) : 0.f;
+      acc[m] += p0 + p1;
+      if (pa2) acc2[m] += fmaf(p0, p0, p1 * p1);
     }
   }
-  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-  if (lane < 8) {
+  // sum over the 16 row pairs, in order
+  auto reduce = [&](const float (&a)[4], float* out) {
+    __syncthreads();
 #pragma unroll
-    for (int m = 0; m < 4; ++m) {
-      red_s[warp][lane + 8 * m] = acc[m];
-      red2_s[warp][lane + 8 * m] = acc2[m];
+    for (int m = 0; m < 4; ++m) red_s[i][j + 16 * m] = a[m];
+    __syncthreads();
+    if (threadIdx.x < kKeyTile && tt + threadIdx.x < N) {
+      float sum = 0.f;
+#pragma unroll
+      for (int w = 0; w < kRowTile / 2; ++w) sum += red_s[w][threadIdx.x];
+      out[out0 + threadIdx.x] = sum;
     }
-  }
-  __syncthreads();
-  if (threadIdx.x < kTokTile && tt + threadIdx.x < N) {
-    float sum = 0.f;
-#pragma unroll
-    for (int w = 0; w < kThreads / 32; ++w) sum += red_s[w][threadIdx.x];
-    pa[int64_t(blockIdx.y) * kv.n_tot + t0 + tt + threadIdx.x] = sum;
-    if (pa2) {
-      float sum2 = 0.f;
-#pragma unroll
-      for (int w = 0; w < kThreads / 32; ++w) sum2 += red2_s[w][threadIdx.x];
-      pa2[int64_t(blockIdx.y) * kv.n_tot + t0 + tt + threadIdx.x] = sum2;
-    }
-  }
-}
-
-// ss[li][g][tg] = sum over e of V[l][g][t][e]^2 for every KV head g; one warp per token.
-template <typename T>
-__global__ void __launch_bounds__(256) value_sumsq_kernel(KvDev kv, BatchDev b, LayerList layers,
-                                                          float* ss) {
-  const int r = blockIdx.y, li = blockIdx.z, l = layers.ids[li];
-  const int t0 = b.tok_off[r], N = b.tok_off[r + 1] - t0;
-  const int t = blockIdx.x * 8 + threadIdx.x / 32, lane = threadIdx.x % 32;
-  if (t >= N) return;
-  const T* vb = static_cast<const T*>(kv.v);
-  for (int g = 0; g < kv.Hkv; ++g) {
-    const float acc = warp_row_sumsq(vb + kv.row(l, g, r, int64_t(t0) + t, t), kv.d, lane);
-    if (lane == 0) ss[(int64_t(li) * kv.Hkv + g) * kv.n_tot + t0 + t] = acc;
-  }
+  };
+  reduce(acc, pa);
+  if (pa2) reduce(acc2, pa2);
 }
 
 }  // namespace
 
-cudaError_t launch_value_sumsq(const KvDev& kv, const BatchDev& b, const LayerList& layers,
-                               int max_tokens, float* ss, cudaStream_t stream) {
-  const dim3 grid((max_tokens + 7) / 8, b.R, layers.n);
-  if (grid.x == 0 || layers.n == 0) return cudaSuccess;
-  if (kv.dtype == CONDUIT_BF16)
-    value_sumsq_kernel<__nv_bfloat16><<<grid, 256, 0, stream>>>(kv, b, layers, ss);
-  else
-    value_sumsq_kernel<float><<<grid, 256, 0, stream>>>(kv, b, layers, ss);
-  count_launches(1);
-  return cudaGetLastError();
+// Chunks of keys pass 1 takes: enough that its blocks (32 rows of a slab by one
+// chunk) fill the GPU about twice over, whole key tiles each.
+int score_simt_chunks(const KvDev& kv, int n_layers, int rows, int max_tokens) {
+  const int64_t blocks = std::max<int64_t>(1, int64_t(n_layers) * kv.Hkv * ((rows + kRowTile - 1) / kRowTile));
+  const int tiles = std::max(1, (max_tokens + kKeyTile - 1) / kKeyTile);
+  return int(std::min<int64_t>(tiles, (320 + blocks - 1) / blocks));
 }
 
 cudaError_t launch_score_simt(const KvDev& kv, const BatchDev& b, const void* q, int32_t q_tot,
-                              const LayerList& layers, int max_rows, int max_tokens,
-                              float2* stats, float* pa, float* pa2, const float* extra_lse,
-                              cudaStream_t stream) {
+                              const LayerList& layers, int max_rows, int max_tokens, int chunks, float2* stats,
+                              float* pa, float* pa2, const float* extra_lse, float* ss, cudaStream_t stream) {
   if (layers.n == 0 || max_rows == 0 || max_tokens == 0) return cudaSuccess;
-  const size_t smem = size_t(kRowBlock + kTokTile) * (kv.d + 1) * sizeof(float);
-  const dim3 g1((max_rows + kRowBlock - 1) / kRowBlock, layers.n * kv.Hkv, b.R);
-  const dim3 g2((max_tokens + kTokTile - 1) / kTokTile, layers.n * kv.Hkv, b.R);
-  cudaError_t err;
-  if (kv.dtype == CONDUIT_BF16) {
-    auto* f1 = rowstats_kernel<__nv_bfloat16>;
-    auto* f2 = colsum_kernel<__nv_bfloat16>;
-    if ((err = cudaFuncSetAttribute(f1, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)))) return err;
-    if ((err = cudaFuncSetAttribute(f2, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)))) return err;
-    const auto* qq = static_cast<const __nv_bfloat16*>(q);
-    f1<<<g1, kThreads, smem, stream>>>(kv, b, qq, q_tot, layers, stats);
+  const int smem = (kRowTile + kKeyTile) * row_stride(kv.d) * int(sizeof(float));
+  const int tiles = (max_tokens + kKeyTile - 1) / kKeyTile;
+  const int chunk_keys = (tiles + chunks - 1) / chunks * kKeyTile;
+  chunks = (max_tokens + chunk_keys - 1) / chunk_keys;
+  const dim3 g1(unsigned((max_rows + kRowTile - 1) / kRowTile) * chunks, layers.n * kv.Hkv, b.R);
+  const dim3 g2(tiles, layers.n * kv.Hkv, b.R);
+  auto go = [&](auto* f1, auto* f2, auto* qq) -> cudaError_t {
+    cudaError_t err;
+    if ((err = cudaFuncSetAttribute(f1, cudaFuncAttributeMaxDynamicSharedMemorySize, smem))) return err;
+    if ((err = cudaFuncSetAttribute(f2, cudaFuncAttributeMaxDynamicSharedMemorySize, smem))) return err;
+    f1<<<g1, kThreads, smem, stream>>>(kv, b, qq, q_tot, layers, chunk_keys, chunks, stats);
     if ((err = cudaGetLastError())) return err;
-    f2<<<g2, kThreads, smem, stream>>>(kv, b, qq, q_tot, layers, stats, pa, pa2, extra_lse);
-  } else {
-    auto* f1 = rowstats_kernel<float>;
-    auto* f2 = colsum_kernel<float>;
-    if ((err = cudaFuncSetAttribute(f1, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)))) return err;
-    if ((err = cudaFuncSetAttribute(f2, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)))) return err;
-    const auto* qq = static_cast<const float*>(q);
-    f1<<<g1, kThreads, smem, stream>>>(kv, b, qq, q_tot, layers, stats);
-    if ((err = cudaGetLastError())) return err;
-    f2<<<g2, kThreads, smem, stream>>>(kv, b, qq, q_tot, layers, stats, pa, pa2, extra_lse);
-  }
+    f2<<<g2, kThreads, smem, stream>>>(kv, b, qq, q_tot, layers, chunk_keys, chunks, stats, pa, pa2, extra_lse, ss);
+    return cudaGetLastError();
+  };
+  const cudaError_t err =
+      kv.dtype == CONDUIT_BF16
+          ? go(rowstats_kernel<__nv_bfloat16>, colsum_kernel<__nv_bfloat16>, static_cast<const __nv_bfloat16*>(q))
+          : go(rowstats_kernel<float>, colsum_kernel<float>, static_cast<const float*>(q));
+  if (err) return err;
   count_launches(2);
-  return cudaGetLastError();
+  return cudaSuccess;
 }
 
 }  // namespace conduit

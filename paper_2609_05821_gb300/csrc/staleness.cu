@@ -314,7 +314,7 @@ cudaError_t launch_staleness_iso(const KvDev& kv, const BatchDev& b, const int32
     count_launches(1);
     if ((err_c = cudaGetLastError())) return err_c;
     if (q_tot > 0) {
-      err_c = launch_refresh_simt(kx, b, pos, b.q_off, q_tot, rows, out, stream);
+      err_c = launch_refresh_simt(kx, b, pos, b.q_off, q_off_host, q_tot, rows, out, stream);
       if (err_c) return err_c;
       const dim3 grid(kv.L, b.R);
       if (bf16)
