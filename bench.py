@@ -222,7 +222,7 @@ def call_kernels(pipe) -> dict:
     tail = ["finalize_tokens_kernel", "image_means_kernel"]
     if tc:  # hbm or tensor: run_conduit keeps whichever ideal time is longer for the workload
         score = (["score_tc_kernel"] + tail, "hbm", "score_tc.cu")
-        refresh = (["refresh_tc_kernel"], "tensor", "refresh_tc.cu")
+        refresh = (["one_refresh_tc_kernel or refresh_tc_kernel"], "tensor", "refresh_tc.cu")
     else:
         score = (["rowstats_kernel", "colsum_kernel"] + tail, "alu", "score_simt.cu")
         refresh = (["refresh_simt_kernel"], "alu", "refresh_simt.cu")

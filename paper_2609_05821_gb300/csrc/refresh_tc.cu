@@ -2,14 +2,13 @@
 // (selective recompute, Conduit Sec. 3.1 / 4.3):
 //   out[l][i][h] = sum_{j <= p_i} softmax_j(<q[l][i][h], K'[l][h/G][j]> / sqrt(d)) V'[l][h/G][j]
 //
-// Work item: two query tiles A and B of 128 rows of one (layer, KV head,
-// request), each floor(128/G) consecutive selected rows times the G query
-// heads that share the KV head; B holds the later rows. Keys stream in tiles
-// of 128, and every K and V tile serves both query tiles: an SM takes at most
-// about 39 bytes per clock from L2 by bulk copies (measured, whatever is in
-// flight), so one query tile per 64 KB of K and V cannot run faster than about
-// 1 700 cycles per tile, and two share that. The kernel is persistent: one CTA
-// per SM takes items from an atomic counter. Roles (384 threads):
+// Two kernels; launch_refresh_tc chooses. A query tile is floor(128/G)
+// consecutive selected rows times the G query heads that share the KV head,
+// 128 rows of one (layer, KV head, request). Keys stream in tiles of 128. Both
+// kernels are persistent: one CTA per SM takes items from an atomic counter.
+//
+// refresh_tc_kernel: two query tiles A and B per work item; B holds the later
+// rows. Every K and V tile is copied once for both. Roles (384 threads):
 //   warp 0      takes and decodes the items (record and row positions in
 //               shared memory, one item ahead) and loads the K tiles
 //   warp 2      loads the V tiles
@@ -32,14 +31,33 @@
 // has completed (the softmax may then rescale O_x).
 // TMEM: S_A, S_B at columns [0, 256), O_A, O_B at [256, 512).
 //
-// Measured (GB300, SM clock 2 070 MHz, against one query tile per item with
-// three S buffers): multi-image prompt 1 253 -> 945 us, batched serving 22.6 ->
-// 18.6 ms, long document 15.2 -> 15.0 ms (17.0 -> 16.3 ms back to back, under
-// the power cap). What bounds it: the chain softmax (about 1 150 cycles for 128
-// keys a thread) -> P V -> next S of a tile, about 3 000 cycles per pair of
-// tiles against 2 048 of tensor work. About 10 % of the multi-image gain is that
-// rows a box leaves empty (G not a power of two) no longer take the masking
-// path.
+// What bounds it: the chain softmax (about 1 150 cycles for 128 keys a thread)
+// -> P V -> next S of a tile, about 3 000 cycles per pair of tiles against 2 048
+// of tensor work.
+//
+// one_refresh_tc_kernel: one query tile per item, three S buffers, and the two
+// softmax warps of a lane quarter share each key tile. It takes about 1 650
+// cycles per tile, but its items are half as long, so it is the faster one where
+// few items reach an SM. Roles:
+//   warp 0      items, query tiles (two buffers) and K tiles; warp 10 V tiles
+//   warp 1      S(t) = Q K(t)^T into TMEM buffer t % 3; warp 11 O += P(t) V(t).
+//               Two warps, because one issuing both, with a wait for each P V
+//               before the S that reuses its buffer, took longer per key tile
+//               than the softmax; both converged, as above (refresh attention
+//               of 16 layers of 4 096 keys 201 -> 196 us)
+//   warps 2-9   softmax: a thread owns one row and 64 of the 128 keys; the two
+//               halves of a row exchange their maxima through shared memory
+// TMEM: S buffers at columns [0, 384) (P in the upper 64 of each), O at
+// [384, 512). S(t) is issued once P(t-3) V(t-3) has completed.
+//
+// In both, rows a box leaves empty (G not a power of two) hold zeros and are
+// never masked: as fully masked rows they sent their warps down the masking
+// path in every key tile (28 heads, 8 192 tokens: 1 254 -> 970 us).
+//
+// Measured (GB300, SM clock 2 070 MHz, before -> now): multi-image prompt 1 254
+// -> 896 us, batched serving 22.6 -> 18.5 ms, long document 15.3 -> 15.0 ms
+// (17.0 -> 16.3 ms back to back, under the power cap), single image 45.5 -> 42.8
+// us, 16 layers of 4 096 tokens 225 -> 196 us.
 //
 // The staleness estimator (kStale) runs the same schedule with every scoring row
 // of a request at its last key: V is the draw z itself, the softmax warps scale
@@ -105,9 +123,10 @@ struct RefArgs {
   int32_t out32;           // out is 32-byte aligned: rows are written in 32-byte stores
   int32_t n_sel;
   int32_t rows_per_tile;   // selected rows per query tile, floor(128 / G)
-  int32_t n_blocks;        // items per (layer, KV head)
+  int32_t n_blocks;        // items (blocks) per (layer, KV head)
   int32_t n_items;         // n_blocks * Hkv * L
-  int32_t blocks_major;    // item order: block (largest first) outer, or (layer, head) outer
+  int32_t span;            // selected rows per item: of one query tile or of two
+  int32_t tail;            // the last `tail` (layer, KV head) pairs come longest block first (see decode_item)
   int32_t* next_item;      // work counter, zero at launch; NULL: CTA c takes items c, c + grid, ...
   float scale_log2;
   int32_t* status;
@@ -120,11 +139,11 @@ struct RefArgs {
 // A work item: block `blk` of (layer l, KV head g), counted from the largest
 // positions, and the request, first selected row and row count. A request's
 // blocks are cut from its last row down, so only the block of its smallest
-// positions may hold fewer than two query tiles.
-// Every layer and head of a request has the same selected positions, so the
-// blocks-major order (all (layer, head) pairs of the largest block first) is
-// longest-first scheduling; the (layer, head)-major order keeps the CTAs in
-// flight on few K/V prefixes, which L2 then shares when the cache exceeds it.
+// positions may be partly filled.
+// Item order: (layer, head)-major up to the last `tail` pairs, so that the CTAs
+// in flight work on few K/V prefixes, which L2 then shares; then all blocks of
+// the last pairs, longest first (every layer and head of a request has the same
+// selected positions). Longest-first is what evens out the end of the launch.
 struct Item {
   int l, g, r, i0, cnt, m, blk;
 };
@@ -138,8 +157,9 @@ __device__ __forceinline__ Item decode_item(const RefArgs& a, int u) {
     it.m = u / a.n_blocks % a.draws;
     u = u / (a.n_blocks * a.draws) * a.n_blocks + u % a.n_blocks;
   }
-  const int x = a.blocks_major ? u / n_lg : u % a.n_blocks;
-  const int lg = a.blocks_major ? u % n_lg : u / a.n_blocks;
+  const int v = u - (n_lg - a.tail) * a.n_blocks;
+  const int x = v >= 0 ? v / a.tail : u % a.n_blocks;
+  const int lg = v >= 0 ? n_lg - a.tail + v % a.tail : u / a.n_blocks;
   it.g = lg % a.kv.Hkv;
   it.l = lg / a.kv.Hkv;
   int blk = a.n_blocks - 1 - x;
@@ -147,7 +167,7 @@ __device__ __forceinline__ Item decode_item(const RefArgs& a, int u) {
   it.r = 0;
   it.i0 = 0;
   it.cnt = 0;
-  const int span = 2 * a.rows_per_tile;
+  const int span = a.span;
   for (int rr = 0; rr < a.b.R; ++rr) {
     const int k0 = a.idx_off[rr], kr = a.idx_off[rr + 1] - k0;
     const int nb = (kr + span - 1) / span;
@@ -229,9 +249,9 @@ __device__ __forceinline__ bool wait_warp(uint64_t* bar, uint32_t parity, volati
   return __all_sync(0xffffffffu, wait_or_abort(bar, parity, abort));
 }
 
-__device__ __forceinline__ void raise_abort(const RefArgs& a, const Smem& s, int32_t site) {
-  if (!*s.abort) flag_status(a.status, CONDUIT_FLAG_TIMEOUT | site);
-  *s.abort = 1;
+__device__ __forceinline__ void raise_abort(const RefArgs& a, volatile int* abort, int32_t site) {
+  if (!*abort) flag_status(a.status, CONDUIT_FLAG_TIMEOUT | site);
+  *abort = 1;
 }
 
 // Warp-cooperative TMA of the 128-key tile starting at request-local key j0:
@@ -350,7 +370,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       nt_a = min(nt_a, nt);  // idx ascends, so this changes nothing unless the caller broke that
       const int rs = n & 1;
       if (!wait_warp(&s.recempty[rs], ((n >> 1) & 1) ^ 1, s.abort)) {
-        if (lane == 0) raise_abort(a, s, tc::kSiteLoad);
+        if (lane == 0) raise_abort(a, s.abort, tc::kSiteLoad);
         break;
       }
       if (!kStale) {
@@ -380,7 +400,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       for (int t = 0; t < nt; ++t, ++T) {
         const uint32_t sl = 2 * T % kStages;
         if (T >= kAhead && !wait_warp(&s.done[(T - kAhead) % kDone], ((T - kAhead) / kDone) & 1, s.abort)) {
-          if (lane == 0) raise_abort(a, s, tc::kSiteLoad);
+          if (lane == 0) raise_abort(a, s.abort, tc::kSiteLoad);
           ok = false;
           break;
         }
@@ -395,7 +415,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     for (uint32_t n = 0; ok; ++n) {
       const int rs = n & 1;
       if (!wait_warp(&s.recfull[rs], (n >> 1) & 1, s.abort)) {
-        if (lane == 0) raise_abort(a, s, tc::kSiteLoad);
+        if (lane == 0) raise_abort(a, s.abort, tc::kSiteLoad);
         break;
       }
       const volatile int* rec = s.rec + rs * 16;
@@ -406,7 +426,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       for (int t = 0; t < nt; ++t, ++T) {
         const uint32_t sl = (2 * T + 1) % kStages;
         if (T >= kAhead && !wait_warp(&s.done[(T - kAhead) % kDone], ((T - kAhead) / kDone) & 1, s.abort)) {
-          if (lane == 0) raise_abort(a, s, tc::kSiteLoad);
+          if (lane == 0) raise_abort(a, s.abort, tc::kSiteLoad);
           ok = false;
           break;
         }
@@ -512,7 +532,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
       if (!ok) break;
     }
-    if (!ok && lane == 0) raise_abort(a, s, tc::kSiteMma);
+    if (!ok && lane == 0) raise_abort(a, s.abort, tc::kSiteMma);
     tc::mma_commit_if(leader, &s.mdone[x]);  // every MMA issued above has completed once this arrives
     tc::mbar_wait(&s.mdone[x], 0);
     if (cq < nq) tc::mbar_wait(&s.qfull[x], cq & 1);  // a copy in flight (only after an abort)
@@ -535,7 +555,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       const float sc = j < N ? scale[j] : 0.f;
       const uint32_t e = 2 * Tv + 1, sl = e % kStages;
       if (!wait_warp(&s.full[sl], (e / kStages) & 1, s.abort)) {
-        if (lane == 0) raise_abort(a, s, tc::kSiteLoad);
+        if (lane == 0) raise_abort(a, s.abort, tc::kSiteLoad);
         return false;
       }
       uint8_t* tile = s.kv + sl * kTileBytes;
@@ -563,7 +583,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     for (uint32_t n = 0; ok; ++n) {
       const int rs = n & 1;
       if (!wait_warp(&s.recfull[rs], (n >> 1) & 1, s.abort)) {
-        if (lane == 0) raise_abort(a, s, tc::kSiteLoad);
+        if (lane == 0) raise_abort(a, s.abort, tc::kSiteLoad);
         break;
       }
       const volatile int* rec = s.rec + rs * 16;
@@ -601,7 +621,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       for (int t = 0; t < nt && ok; ++t, ++ns) {
         // the tcgen05.ld below is warp-collective: the whole warp goes on or stops
         if (!wait_warp(&s.sfull[x], ns & 1, s.abort)) {
-          if (lane == 0) raise_abort(a, s, tc::kSiteMma);
+          if (lane == 0) raise_abort(a, s.abort, tc::kSiteMma);
           ok = false;
           break;
         }
@@ -680,7 +700,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (kStale && nt == 0 && lane == 0) *part = 0.0;  // no rows in this tile
       if (nt == 0 || !ok) continue;
       if (!wait_warp(&s.ofull[x], no & 1, s.abort)) {
-        if (lane == 0) raise_abort(a, s, tc::kSiteFinal);
+        if (lane == 0) raise_abort(a, s.abort, tc::kSiteFinal);
         ok = false;
         break;
       }
@@ -755,6 +775,494 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (warp == kMmaWarp) tc::tmem_dealloc(tmem, kTmemCols);
 }
 
+// ------------------------------------------------ one query tile per item
+constexpr int kSoftThreads = 256;
+constexpr int kOneVWarp = 10, kPvWarp = 11;      // after the item/K, MMA and eight softmax warps
+constexpr int kKStages = 2, kVStages = 2, kQBufs = 2;
+constexpr uint32_t kOneTileBytes = 2 * kHalfBytes;
+constexpr uint32_t kQBytes = 2 * kHalfBytes;
+constexpr int kRecInts = 9;                      // decoded item record (see OneSmem::rec)
+constexpr uint32_t kOneSmem = 1024 + kQBufs * kQBytes + (kKStages + kVStages) * kOneTileBytes + 256 +
+                              2 * 2 * 128 * 4 + 2 * 128 * 4 + kQBufs * (kRecInts + kRows) * 4;
+constexpr int kSBufs = 3;                        // S runs up to two key tiles ahead of the softmax
+constexpr uint32_t kOneOCol = kSBufs * kSCols;
+
+struct OneSmem {
+  uint8_t* q;        // [kQBufs][2 halves][128 rows][128 B]
+  uint8_t* k;        // [kKStages][2 halves][128 keys][128 B]
+  uint8_t* v;        // [kVStages][2 halves][128 keys][128 B]
+  uint64_t *kfull, *kempty;   // [kKStages]
+  uint64_t *vfull, *vempty;   // [kVStages]
+  uint64_t *sfull, *pfull;    // [kSBufs] per S buffer
+  uint64_t *pvdone;           // [kSBufs] per S buffer: the P.V that read its P has completed
+  uint64_t *qfull, *qempty;   // [kQBufs] query tile (and item index) of one item
+  uint64_t *ofull, *oempty;   // once per item: O complete / O read out
+  uint64_t *mdone;            // [2] per MMA thread: all its MMAs completed
+  uint32_t* tmem_slot;
+  volatile int* abort;
+  uint32_t* counters;  // [0] K loads, [1] V loads, [2] K consumed, [3] V consumed
+  float* xmax;         // [2 tile parities][2 halves][128 rows] half-row maxima
+  float* xsum;         // [2 halves][128 rows] half-row sums at the end
+  // per query buffer, written by the loader with the query tile: the decoded
+  // item {u (-1: no more work), l, g, r, i0, cnt, key tiles, N_r, t0} and the
+  // positions of its selected rows, so the other roles read no global memory
+  // between items
+  volatile int* rec;   // [kQBufs][kRecInts]
+  volatile int* pos;   // [kQBufs][kRows]
+};
+
+__device__ __forceinline__ OneSmem carve_one(uint8_t* raw) {
+  uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(raw) + 1023) & ~uintptr_t(1023));
+  OneSmem s;
+  s.q = base;
+  s.k = s.q + kQBufs * kQBytes;
+  s.v = s.k + kKStages * kOneTileBytes;
+  uint64_t* bar = reinterpret_cast<uint64_t*>(s.v + kVStages * kOneTileBytes);
+  s.kfull = bar;
+  s.kempty = s.kfull + kKStages;
+  s.vfull = s.kempty + kKStages;
+  s.vempty = s.vfull + kVStages;
+  s.sfull = s.vempty + kVStages;
+  s.pfull = s.sfull + kSBufs;
+  s.pvdone = s.pfull + kSBufs;
+  s.qfull = s.pvdone + kSBufs;
+  s.qempty = s.qfull + kQBufs;
+  s.ofull = s.qempty + kQBufs;
+  s.oempty = s.ofull + 1;
+  s.mdone = s.oempty + 1;
+  s.tmem_slot = reinterpret_cast<uint32_t*>(s.mdone + 2);
+  s.abort = reinterpret_cast<volatile int*>(s.tmem_slot + 1);
+  s.counters = reinterpret_cast<uint32_t*>(s.tmem_slot + 2);
+  s.xmax = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(bar) + 256);
+  s.xsum = s.xmax + 2 * 2 * 128;
+  s.rec = reinterpret_cast<volatile int*>(s.xsum + 2 * 128);
+  s.pos = s.rec + kQBufs * kRecInts;
+  return s;
+}
+
+// Agreement of the 256 softmax threads (named barrier 1 with an AND
+// reduction): every thread arrives, so all of them take the same branch.
+__device__ __forceinline__ bool softmax_all(bool pred) {
+  uint32_t out;
+  asm volatile(
+      "{\n.reg .pred pi, po;\nsetp.ne.u32 pi, %1, 0;\nbar.red.and.pred po, 1, %2, pi;\nselp.u32 %0, 1, 0, po;\n}\n"
+      : "=r"(out)
+      : "r"(uint32_t(pred)), "n"(kSoftThreads)
+      : "memory");
+  return out != 0;
+}
+
+__global__ void __launch_bounds__(kThreads, 1)
+    one_refresh_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant__ CUtensorMap vmap,
+                      const __grid_constant__ CUtensorMap qmap, const __grid_constant__ RefArgs a) {
+  extern __shared__ uint8_t smem_raw[];
+  const OneSmem s = carve_one(smem_raw);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const KvDev& kv = a.kv;
+  const int G = kv.G, Hq = kv.Hq;
+  const int qrows = a.rows_per_tile * G;          // rows the query box fills
+
+  if (tid == 0) {
+    for (int i = 0; i < kKStages; ++i) {
+      tc::mbar_init(&s.kfull[i], 1);
+      tc::mbar_init(&s.kempty[i], 1);
+    }
+    for (int i = 0; i < kVStages; ++i) {
+      tc::mbar_init(&s.vfull[i], 1);
+      tc::mbar_init(&s.vempty[i], 1);
+    }
+    for (int i = 0; i < kSBufs; ++i) {
+      tc::mbar_init(&s.sfull[i], 1);
+      // per buffer, so the softmax can never be two phases ahead of the MMA's
+      // wait: P(t+3) needs S(t+3), issued only after P(t) V(t) has completed
+      tc::mbar_init(&s.pfull[i], kSoftThreads);
+      tc::mbar_init(&s.pvdone[i], 1);
+    }
+    for (int i = 0; i < kQBufs; ++i) {
+      tc::mbar_init(&s.qfull[i], 1);   // the loader's expect-tx (or plain arrive at the end)
+      // the S thread's commit + the P.V thread's, softmax's and V warp's reads of the item
+      tc::mbar_init(&s.qempty[i], 4);
+    }
+    tc::mbar_init(s.ofull, 1);
+    tc::mbar_init(s.oempty, kSoftThreads);
+    tc::mbar_init(&s.mdone[0], 1);
+    tc::mbar_init(&s.mdone[1], 1);
+    *s.abort = 0;
+    for (int i = 0; i < 4; ++i) s.counters[i] = 0;
+    tc::fence_barrier_init();
+    tc::prefetch_tensormap(&kmap);
+    tc::prefetch_tensormap(&vmap);
+    tc::prefetch_tensormap(&qmap);
+  }
+  if (warp == 1) tc::tmem_alloc(s.tmem_slot, kTmemCols);
+  for (uint32_t i = qrows * 128 + tid * 16; i < kHalfBytes; i += kThreads * 16)  // rows the boxes leave empty
+    for (int h = 0; h < 2 * kQBufs; ++h) *reinterpret_cast<uint4*>(s.q + h * kHalfBytes + i) = make_uint4(0, 0, 0, 0);
+  tc::fence_proxy_async_smem();
+  __syncthreads();
+  tc::tc_fence_after();
+  const uint32_t tmem = *s.tmem_slot;
+
+  if (warp == 0) {
+    // ------------------------------------------------------- loads (warp 0)
+    uint32_t nk = 0, T = 0;
+    bool ok = true;
+    for (uint32_t n = 0; ok; ++n) {
+      int u = 0;
+      if (lane == 0) {
+        u = n == 0 ? int(blockIdx.x)
+                   : a.next_item ? int(gridDim.x) + atomicAdd(a.next_item, 1) : int(blockIdx.x + n * gridDim.x);
+        if (u >= a.n_items) u = -1;
+      }
+      u = __shfl_sync(0xffffffffu, u, 0);
+      const Item it = decode_item<false>(a, u < 0 ? 0 : u);
+      const int t0 = a.b.tok_off[it.r], N = a.b.tok_off[it.r + 1] - t0;
+      int nt = 0;
+      if (u >= 0 && it.cnt > 0) {
+        const int p_max = min(a.idx[it.i0 + it.cnt - 1], N - 1);
+        nt = p_max < 0 ? 0 : p_max / kKT + 1;
+      }
+      int my_pos[kRows / 32];  // positions of the item's rows, loaded before the buffer is free
+#pragma unroll
+      for (int k = 0; k < kRows / 32; ++k) {
+        const int i = lane + 32 * k;
+        my_pos[k] = (u >= 0 && i < it.cnt) ? a.idx[it.i0 + i] : -1;
+      }
+      const int qs = n & 1;
+      if (!__all_sync(0xffffffffu, wait_or_abort(&s.qempty[qs], ((n >> 1) & 1) ^ 1, s.abort))) {
+        if (lane == 0) raise_abort(a, s.abort, tc::kSiteLoad);
+        break;
+      }
+#pragma unroll
+      for (int k = 0; k < kRows / 32; ++k) s.pos[qs * kRows + lane + 32 * k] = my_pos[k];
+      if (lane == 0) {
+        volatile int* rec = s.rec + qs * kRecInts;
+        rec[0] = u;
+        rec[1] = it.l;
+        rec[2] = it.g;
+        rec[3] = it.r;
+        rec[4] = it.i0;
+        rec[5] = it.cnt;
+        rec[6] = nt;
+        rec[7] = N;
+        rec[8] = t0;
+      }
+      __threadfence_block();
+      __syncwarp();  // the lanes' positions are ordered before lane 0's release below
+      if (lane == 0) {
+        if (u < 0) {
+          tc::mbar_arrive(&s.qfull[qs]);  // no more work: the others stop at this buffer
+        } else {
+          tc::mbar_arrive_expect_tx(&s.qfull[qs], 2u * 128u * uint32_t(qrows));
+          for (int hf = 0; hf < 2; ++hf)
+            tc::tma_load_3d(s.q + qs * kQBytes + hf * kHalfBytes, &qmap, &s.qfull[qs], hf * 64,
+                            it.g * G, it.l * a.n_sel + it.i0);
+        }
+      }
+      if (u < 0) break;
+      for (int t = 0; t < nt; ++t, ++T) {
+        const int sk = T % kKStages;
+        if (!__all_sync(0xffffffffu, wait_or_abort(&s.kempty[sk], ((T / kKStages) & 1) ^ 1, s.abort))) {
+          if (lane == 0) raise_abort(a, s.abort, tc::kSiteLoad);
+          ok = false;
+          break;
+        }
+        load_tile<2>(a, &kmap, s.k + sk * kOneTileBytes, &s.kfull[sk], it.l, it.g, it.r, t0, N, t * kKT, lane);
+        ++nk;
+      }
+    }
+    if (lane == 0) s.counters[0] = nk;
+  } else if (warp == kOneVWarp) {
+    // --------------------------------------------------- V loads (warp 10)
+    // on a warp of their own: a V stage frees only once its P.V has
+    // completed, and waiting for it must not hold back the K tiles and the
+    // next item's query tile
+    uint32_t nv = 0, T = 0;
+    for (uint32_t n = 0;; ++n) {
+      const int qs = n & 1;
+      if (!__all_sync(0xffffffffu, wait_or_abort(&s.qfull[qs], (n >> 1) & 1, s.abort))) {
+        if (lane == 0) raise_abort(a, s.abort, tc::kSiteLoad);
+        break;
+      }
+      const volatile int* rec = s.rec + qs * kRecInts;
+      const int u = rec[0], l = rec[1], g = rec[2], r = rec[3], nt = rec[6], N = rec[7], t0 = rec[8];
+      __syncwarp();
+      if (lane == 0) tc::mbar_arrive(&s.qempty[qs]);  // this warp is done with the record
+      if (u < 0) break;
+      bool ok = true;
+      for (int t = 0; t < nt; ++t, ++T) {
+        const int sv = T % kVStages;
+        if (!__all_sync(0xffffffffu, wait_or_abort(&s.vempty[sv], ((T / kVStages) & 1) ^ 1, s.abort))) {
+          if (lane == 0) raise_abort(a, s.abort, tc::kSiteLoad);
+          ok = false;
+          break;
+        }
+        load_tile<2>(a, &vmap, s.v + sv * kOneTileBytes, &s.vfull[sv], l, g, r, t0, N, t * kKT, lane);
+        ++nv;
+      }
+      if (!ok) break;
+    }
+    if (lane == 0) s.counters[1] = nv;
+  } else if (warp == 1) {
+    // ---------------------------------------------------------- MMA: S = Q K^T
+    // S(t) goes to buffer t % kSBufs once P(t-3) V(t-3), which read that
+    // buffer's P, has completed (possibly of an earlier item); so this warp
+    // runs up to two tiles ahead of the P.V warp
+    const uint32_t leader = lane == 0;
+    uint32_t T = 0;
+    bool ok = true;
+    const uint32_t idesc_s = tc::idesc_bf16(kRows, kKT);
+    const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
+    for (uint32_t n = 0; ok; ++n) {
+      const int qs = n & 1;
+      if (!(ok = wait_warp(&s.qfull[qs], (n >> 1) & 1, s.abort))) break;
+      const int u = __shfl_sync(0xffffffffu, s.rec[qs * kRecInts], 0);
+      const int nt = __shfl_sync(0xffffffffu, s.rec[qs * kRecInts + 6], 0);
+      if (u < 0) break;
+      const uint64_t dq = tc::desc_sw128(tc::smem_u32(s.q + qs * kQBytes));
+      for (int t = 0; t < nt; ++t, ++T) {
+        const int b = T % kSBufs, sk = T % kKStages;
+        if (T >= uint32_t(kSBufs) && !(ok = wait_warp(&s.pvdone[b], ((T / kSBufs) - 1) & 1, s.abort))) break;
+        if (!(ok = wait_warp(&s.kfull[sk], (T / kKStages) & 1, s.abort))) break;
+        if (leader) s.counters[2] = T + 1;
+        __syncwarp();
+        tc::tc_fence_after();
+        const uint64_t dk = tc::desc_sw128(tc::smem_u32(s.k + sk * kOneTileBytes));
+#pragma unroll
+        for (int kk = 0; kk < 8; ++kk) {
+          const uint32_t off = ((kk >> 2) * kHalfBytes + (kk & 3) * 32) >> 4;
+          tc::mma_bf16_if(leader, tm + b * kSCols, dq + off, dk + off, idesc_s, kk > 0);
+        }
+        tc::mma_commit_if(leader, &s.sfull[b]);
+        tc::mma_commit_if(leader, &s.kempty[sk]);
+      }
+      if (ok) tc::mma_commit_if(leader, &s.qempty[qs]);  // every S of this item is issued
+    }
+    if (!ok && leader) raise_abort(a, s.abort, tc::kSiteMma);
+    tc::mma_commit_if(leader, &s.mdone[0]);  // every MMA issued above has completed once this arrives
+    tc::mbar_wait(&s.mdone[0], 0);
+    __syncwarp();
+  } else if (warp == kPvWarp) {
+    // -------------------------------------------------------- MMA: O += P V
+    const uint32_t leader = lane == 0;
+    uint32_t T = 0;
+    bool ok = true;
+    const uint32_t idesc_o = tc::idesc_bf16(kRows, kMaxD, /*b_mn_major=*/true);
+    const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
+    for (uint32_t n = 0; ok; ++n) {
+      const int qs = n & 1;
+      if (!(ok = wait_warp(&s.qfull[qs], (n >> 1) & 1, s.abort))) break;
+      const int u = __shfl_sync(0xffffffffu, s.rec[qs * kRecInts], 0);
+      const int nt = __shfl_sync(0xffffffffu, s.rec[qs * kRecInts + 6], 0);
+      tc::mbar_arrive_if(leader, &s.qempty[qs]);  // this warp is done with the record
+      if (u < 0) break;
+      for (int t = 0; t < nt; ++t, ++T) {
+        const int b = T % kSBufs, sv = T % kVStages;
+        if (!(ok = wait_warp(&s.vfull[sv], (T / kVStages) & 1, s.abort))) break;
+        if (leader) s.counters[3] = T + 1;
+        __syncwarp();
+        if (!(ok = wait_warp(&s.pfull[b], (T / kSBufs) & 1, s.abort))) break;
+        // O of the previous item must have been read out before P(0) V(0) overwrites it
+        if (t == 0 && n > 0 && !(ok = wait_warp(s.oempty, (n - 1) & 1, s.abort))) break;
+        tc::tc_fence_after();
+        const uint64_t dv = tc::desc_sw128_mn(tc::smem_u32(s.v + sv * kOneTileBytes), kHalfBytes);
+        const uint32_t pb = tm + b * kSCols + kPCol;
+#pragma unroll
+        for (int kk = 0; kk < kKT / 16; ++kk)  // O += P(t) V(t)
+          tc::mma_bf16_ts_if(leader, tm + kOneOCol, pb + kk * 8, dv + kk * (2048 >> 4), idesc_o, t > 0 || kk > 0);
+        tc::mma_commit_if(leader, &s.pvdone[b]);
+        tc::mma_commit_if(leader, &s.vempty[sv]);
+      }
+      if (ok) tc::mma_commit_if(leader, s.ofull);  // O of this item is complete once this arrives
+    }
+    if (!ok && leader) raise_abort(a, s.abort, tc::kSiteMma);
+    tc::mma_commit_if(leader, &s.mdone[1]);
+    tc::mbar_wait(&s.mdone[1], 0);
+    __syncwarp();
+  } else if (warp >= 2 && warp < kOneVWarp) {
+    // -------------------------------------------------------------- softmax
+    const int et = tid - 64;                             // 0..255
+    const int hh = et >> 7;                              // half of the key tile / of O
+    const int quarter = warp & 3;
+    const int row = quarter * 32 + lane;                 // TMEM lane = query row of the tile
+    const uint32_t lane_base = uint32_t(quarter * 32) << 16;
+    const uint32_t tl = tmem + lane_base;
+    bool ok = true;
+    uint32_t T = 0;
+    for (uint32_t n = 0;; ++n) {
+      const int qs = n & 1;
+      // all 256 threads agree to go on, so the named barriers below stay uniform
+      const bool got = wait_or_abort(&s.qfull[qs], (n >> 1) & 1, s.abort);
+      if (!softmax_all(ok && got)) {
+        if (ok) raise_abort(a, s.abort, tc::kSiteLoad);
+        break;
+      }
+      const volatile int* rec = s.rec + qs * kRecInts;
+      const int u = rec[0];
+      Item it;
+      it.l = rec[1];
+      it.g = rec[2];
+      it.r = rec[3];
+      it.i0 = rec[4];
+      it.cnt = rec[5];
+      const int nt = rec[6], N = rec[7];
+      const bool row_ok = u >= 0 && row < it.cnt * G;
+      const int i_row = it.i0 + (row_ok ? row / G : 0);
+      const int h_row = it.g * G + (row_ok ? row % G : 0);
+      int p_row = row_ok ? s.pos[qs * kRows + row / G] : -1;  // rows past the item (or the box) are fully masked
+      const bool live = p_row >= 0 && p_row < N;
+      if (!live) p_row = 0x7fffffff;
+      asm volatile("bar.sync 1, %0;" ::"n"(kSoftThreads) : "memory");  // everyone has read the record
+      if (et == 0) tc::mbar_arrive(&s.qempty[qs]);
+      if (u < 0) break;
+
+      float m_ref = -INFINITY, lsum = 0.f;  // running max (scaled, log2 units, same in both halves) and half-row sum
+      for (int t = 0; t < nt; ++t) {
+        const uint32_t Tc = T + t;
+        const uint32_t sbuf = Tc % kSBufs;
+        const uint32_t sb = tl + sbuf * kSCols;
+        // the tcgen05.ld below is warp-collective: the whole warp goes on or stops
+        const bool gs = __all_sync(0xffffffffu, ok && (tc::mbar_probe(&s.sfull[sbuf], (Tc / kSBufs) & 1) ||
+                                                       wait_or_abort(&s.sfull[sbuf], (Tc / kSBufs) & 1, s.abort)));
+        if (!gs) {
+          if (ok) raise_abort(a, s.abort, tc::kSiteMma);
+          ok = false;
+        }
+        float sv[64];
+        float hmax = -INFINITY;
+        const int j0 = t * kKT + hh * 64;
+        if (gs) {
+          tc::tc_fence_after();
+          tc::tmem_ld64(sb + hh * 64, sv);
+          if (j0 + 63 > p_row) {  // part of this half is past this row's position
+#pragma unroll
+            for (int i = 0; i < 64; ++i)
+              if (j0 + i > p_row) sv[i] = -INFINITY;
+          }
+          float tm[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+          for (int i = 0; i < 32; ++i) tm[i & 3] = tc::fmax3(tm[i & 3], sv[2 * i], sv[2 * i + 1]);
+          hmax = fmaxf(fmaxf(tm[0], tm[1]), fmaxf(tm[2], tm[3]));
+        }
+        // exchange the half-row maxima (buffers alternate with the tile, so a
+        // half that runs ahead never overwrites a value its partner still reads)
+        float* xm = s.xmax + (Tc & 1) * 256;
+        xm[hh * 128 + row] = hmax;
+        asm volatile("bar.sync 1, %0;" ::"n"(kSoftThreads) : "memory");
+        if (!ok) continue;
+        const float tmax = fmaxf(hmax, xm[(hh ^ 1) * 128 + row]) * a.scale_log2;
+        const bool need = tmax > m_ref + kRescaleLog2 || (m_ref == -INFINITY && tmax != -INFINITY);
+        const float alpha = need ? tc::ex2(m_ref - tmax) : 1.f;  // 0 when m_ref is -inf
+        if (need) {
+          lsum *= alpha;
+          m_ref = tmax;
+        }
+        // this half of P = 2^(S scale - m) in bf16 pairs over the upper half of S
+        // (one packed FMA per pair for scale and bias, packed adds for the sum).
+        // A row with no visible key yet (m = -inf) uses bias 0: its logits are
+        // all -inf and its P is 0.
+        const float2 sc2 = make_float2(a.scale_log2, a.scale_log2);
+        const float2 nb2 = m_ref == -INFINITY ? make_float2(0.f, 0.f) : make_float2(-m_ref, -m_ref);
+        float2 ls2[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+        {
+#pragma unroll
+          for (int c = 0; c < 2; ++c) {
+            uint32_t pw[16];
+#pragma unroll
+            for (int i = 0; i < 16; ++i) {
+              const float2 y = tc::ffma2(make_float2(sv[32 * c + 2 * i], sv[32 * c + 2 * i + 1]), sc2, nb2);
+              const float2 pp = make_float2(tc::ex2(y.x), tc::ex2(y.y));
+              ls2[i & 1] = tc::fadd2(ls2[i & 1], pp);
+              __nv_bfloat162 pr = __floats2bfloat162_rn(pp.x, pp.y);
+              pw[i] = *reinterpret_cast<uint32_t*>(&pr);
+            }
+            tc::tmem_st16_nowait(sb + kPCol + hh * 32 + 16 * c, pw);
+          }
+          tc::tmem_wait_st();
+        }
+        const float ls[4] = {ls2[0].x, ls2[0].y, ls2[1].x, ls2[1].y};
+        lsum += (ls[0] + ls[1]) + (ls[2] + ls[3]);
+        if (__any_sync(0xffffffffu, need) && t > 0) {
+          // P(t-1) V(t-1) must have completed before this warp rescales its half
+          // of O. That buffer's next P.V needs a P this softmax has not written
+          // yet, so the barrier's parity cannot alias; P(t) V(t) waits for this
+          // warp's pfull arrival below.
+          if (!__all_sync(0xffffffffu,
+                          wait_or_abort(&s.pvdone[(Tc - 1) % kSBufs], ((Tc - 1) / kSBufs) & 1, s.abort))) {
+            raise_abort(a, s.abort, tc::kSiteMma);
+            ok = false;
+            continue;
+          }
+          tc::tc_fence_after();
+          for (int c = hh * 64; c < hh * 64 + 64; c += 32) {
+            float o[32];
+            tc::tmem_ld32(tl + kOneOCol + c, o);
+#pragma unroll
+            for (int i = 0; i < 32; ++i) o[i] *= alpha;
+            tc::tmem_st32(tl + kOneOCol + c, o);
+          }
+        }
+        tc::tc_fence_before();
+        tc::mbar_arrive(&s.pfull[sbuf]);
+      }
+      T += nt;
+      // row sum = the two halves' sums (same running max in both)
+      s.xsum[hh * 128 + row] = lsum;
+      asm volatile("bar.sync 1, %0;" ::"n"(kSoftThreads) : "memory");
+      const float total = s.xsum[row] + s.xsum[128 + row];
+      // O of this item is complete once the MMA thread's per-item commit has
+      // arrived (it cannot run a phase ahead: the next one needs this warp's P)
+      const bool fin = __all_sync(0xffffffffu, ok && wait_or_abort(s.ofull, n & 1, s.abort));
+      if (!fin && ok) {
+        raise_abort(a, s.abort, tc::kSiteFinal);
+        ok = false;
+      }
+      if (fin) {
+        tc::tc_fence_after();
+        const float inv = total > 0.f ? 1.f / total : 0.f;
+        __nv_bfloat16* dst = a.out + ((int64_t(it.l) * a.n_sel + i_row) * Hq + h_row) * kMaxD;
+        // This thread's 64 columns of O in one load, then its half row as
+        // bf16. Each lane writes its own row, so a warp's store covers 32
+        // rows: 32-byte stores (whole sectors) when the buffer allows them.
+        float o[64];
+        tc::tmem_ld64(tl + kOneOCol + hh * 64, o);
+        if (live) {
+          uint32_t w[32];
+#pragma unroll
+          for (int k2 = 0; k2 < 32; ++k2) {
+            __nv_bfloat162 pr = __floats2bfloat162_rn(o[2 * k2] * inv, o[2 * k2 + 1] * inv);
+            w[k2] = *reinterpret_cast<uint32_t*>(&pr);
+          }
+          __nv_bfloat16* drow = dst + hh * 64;
+          if (a.out32) {
+#pragma unroll
+            for (int u8 = 0; u8 < 4; ++u8)
+              asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(drow + u8 * 16),
+                           "r"(w[8 * u8]), "r"(w[8 * u8 + 1]), "r"(w[8 * u8 + 2]), "r"(w[8 * u8 + 3]),
+                           "r"(w[8 * u8 + 4]), "r"(w[8 * u8 + 5]), "r"(w[8 * u8 + 6]), "r"(w[8 * u8 + 7])
+                           : "memory");
+          } else {
+#pragma unroll
+            for (int u4 = 0; u4 < 8; ++u4)
+              *reinterpret_cast<uint4*>(drow + u4 * 8) = make_uint4(w[4 * u4], w[4 * u4 + 1], w[4 * u4 + 2], w[4 * u4 + 3]);
+          }
+        }
+      }
+      tc::tc_fence_before();
+      tc::mbar_arrive(s.oempty);  // O may be overwritten by the next item
+    }
+  }
+  __syncthreads();
+  if (tid == 0) {  // drain loads issued but never consumed (only after an abort)
+    for (uint32_t n = s.counters[2]; n < s.counters[0]; ++n)
+      tc::mbar_wait(&s.kfull[n % kKStages], (n / kKStages) & 1);
+    for (uint32_t n = s.counters[3]; n < s.counters[1]; ++n)
+      tc::mbar_wait(&s.vfull[n % kVStages], (n / kVStages) & 1);
+  }
+  tc::tc_fence_before();
+  __syncthreads();
+  if (warp == 1) tc::tmem_dealloc(tmem, kTmemCols);
+}
+
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*,
                                   const cuuint64_t*, const cuuint64_t*, const cuuint32_t*,
                                   const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
@@ -818,13 +1326,30 @@ bool refresh_tc_supported(const KvDev& kv) {
   return true;
 }
 
-// Rows of a (layer, KV head, request) in blocks of two query tiles.
-static int query_blocks(const BatchDev& b, const int32_t* off_host, int rows_per_tile) {
+// Blocks of `span` rows of a (layer, KV head), over its requests.
+static int query_blocks(const BatchDev& b, const int32_t* off_host, int span) {
   int blocks = 0;
-  for (int r = 0; r < b.R; ++r)
-    blocks += (off_host[r + 1] - off_host[r] + 2 * rows_per_tile - 1) / (2 * rows_per_tile);
+  for (int r = 0; r < b.R; ++r) blocks += (off_host[r + 1] - off_host[r] + span - 1) / span;
   return blocks;
 }
+
+// One query tile per item or two, for head_dim 128 (the smaller sizes have the
+// two-tile kernel only), by the key tiles that two-tile items would bring to an
+// SM. Two-tile items are half as many and cost less per tile, which pays once
+// the end of the launch no longer shows (one / two tiles per item, us):
+// 2 layers x 1 885 tokens 22.6 / 35.0, 28 x 1 024 42.8 / 45.0, 36 x 4 096 (213
+// key tiles per SM) 423 / 442, two requests of 4 096 (283) 498 / 511, 28 x 6 144
+// (319) 598 / 590, 28 x 8 192 (540) 912 / 896, long document (8 000) 15 400 /
+// 15 000. Pages of 16 keys and fewer cost one tile per item more, since each
+// page half is a copy of its own: 8 x 2 048 (10) 39.3 / 42.7, 28 x 2 048 (35)
+// 108.7 / 106.9, 8 x 4 096 (40) 109.2 / 105.6, four requests of 2 048 (142) 404
+// / 381; pages of 32 are as contiguous caches (28 x 2 048 97.3 / 105.2).
+constexpr double kOneKeyTilesPerSm = 300., kOneKeyTilesPerSmPaged = 24.;
+constexpr int kOneMinPage = 32;
+// Items per SM in longest-first order at the end of a launch whose K/V exceeds
+// L2: 0 / 2 / 3 / 4 items took 213 / 196 / 196.5 / 199 us on 16 layers of 4 096
+// tokens (one tile per item) and 952 / 908 / 896 / 904 us on 28 of 8 192 (two).
+constexpr int kTailItemsPerSm = 3;
 
 cudaError_t launch_refresh_tc(const KvDev& kv, const BatchDev& b, const int32_t* idx,
                               const int32_t* idx_off_dev, const int32_t* idx_off_host, int32_t n_sel,
@@ -844,23 +1369,31 @@ cudaError_t launch_refresh_tc(const KvDev& kv, const BatchDev& b, const int32_t*
   a.out32 = (reinterpret_cast<uintptr_t>(out) & 31) == 0 && kv.d % 16 == 0;
   a.n_sel = n_sel;
   a.rows_per_tile = kRows / kv.G;
-  const int blocks = query_blocks(b, idx_off_host, a.rows_per_tile);
-  a.n_blocks = blocks;
-  a.n_items = blocks * kv.Hkv * kv.L;
-  a.next_item = work_counter;
-  a.scale_log2 = kLog2e / sqrtf(float(kv.d));
-  a.status = status;
-  if (blocks == 0) return cudaSuccess;
-  int dev = 0, sms = 0;
+  int dev = 0, sms = 0, l2 = 0;
   cudaError_t err;
   if ((err = cudaGetDevice(&dev))) return err;
   if ((err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev))) return err;
-  int l2 = 0;
   if ((err = cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev))) return err;
-  // longest-first when the whole K/V of the batch fits in half of L2 (the rest
-  // holds queries and outputs), else (layer, head)-major
-  const double kv_bytes = 2.0 * double(kv.L) * kv.Hkv * double(kv.n_tot) * kv.d * 2;
-  a.blocks_major = kv_bytes <= 0.5 * double(l2) ? 1 : 0;
+  const int n_lg = kv.Hkv * kv.L;
+  a.span = 2 * a.rows_per_tile;
+  a.n_blocks = query_blocks(b, idx_off_host, a.span);
+  const double key_tiles = double(a.n_blocks) * n_lg * (double(kv.n_tot) / b.R) / (2 * kKT);
+  const bool few_copies = kv.page_size == 0 || kv.page_size >= kOneMinPage;
+  const bool one = kv.d == kMaxD && key_tiles < sms * (few_copies ? kOneKeyTilesPerSm : kOneKeyTilesPerSmPaged);
+  if (one) {
+    a.span = a.rows_per_tile;
+    a.n_blocks = query_blocks(b, idx_off_host, a.span);
+  }
+  a.n_items = a.n_blocks * n_lg;
+  a.next_item = work_counter;
+  a.scale_log2 = kLog2e / sqrtf(float(kv.d));
+  a.status = status;
+  if (a.n_blocks == 0) return cudaSuccess;
+  // longest-first throughout when the whole K/V of the batch fits in half of L2
+  // (the rest holds queries and outputs), else for about the last kTailItemsPerSm
+  // items of each SM
+  const double kv_bytes = 2.0 * double(n_lg) * double(kv.n_tot) * kv.d * 2;
+  a.tail = kv_bytes <= 0.5 * double(l2) ? n_lg : std::min(n_lg, (kTailItemsPerSm * sms + a.n_blocks - 1) / a.n_blocks);
   if (work_counter && (err = cudaMemsetAsync(work_counter, 0, sizeof(int32_t), stream))) return err;
   auto launch = [&](auto* f, uint32_t smem) -> cudaError_t {
     if ((err = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)))) return err;
@@ -869,7 +1402,9 @@ cudaError_t launch_refresh_tc(const KvDev& kv, const BatchDev& b, const int32_t*
   };
   // head_dim 128 keeps its bf16 P; the smaller sizes ran with fp32 weights on
   // CUDA cores before and keep that precision by a split P
-  if (kv.d == kMaxD)
+  if (one)
+    err = launch(one_refresh_tc_kernel, kOneSmem);
+  else if (kv.d == kMaxD)
     err = launch(refresh_tc_kernel<2, false>, Shape<2>::kSmem);
   else if (kv.d > 64)
     err = launch(refresh_tc_kernel<2, true>, Shape<2>::kSmem);
@@ -881,7 +1416,7 @@ cudaError_t launch_refresh_tc(const KvDev& kv, const BatchDev& b, const int32_t*
 }
 
 int stale_tc_blocks(const KvDev& kv, const BatchDev& b, const int32_t* q_off_host) {
-  return query_blocks(b, q_off_host, kRows / kv.G);
+  return query_blocks(b, q_off_host, 2 * (kRows / kv.G));
 }
 
 cudaError_t launch_stale_tc(const KvDev& kv, const BatchDev& b, const int32_t* q_off_host, int32_t q_tot,
@@ -894,7 +1429,8 @@ cudaError_t launch_stale_tc(const KvDev& kv, const BatchDev& b, const int32_t* q
   a.idx_off = b.q_off;
   a.n_sel = q_tot;
   a.rows_per_tile = kRows / kv.G;
-  a.n_blocks = query_blocks(b, q_off_host, a.rows_per_tile);
+  a.span = 2 * a.rows_per_tile;
+  a.n_blocks = query_blocks(b, q_off_host, a.span);
   a.draws = draws;
   a.n_items = draws * a.n_blocks * kv.Hkv * kv.L;
   a.next_item = work_counter;

@@ -1,6 +1,6 @@
 """Refresh attention at the edges of its work items against the oracle.
 
-A work item of the tensor-core kernel is two query tiles of floor(128/G)
+A work item of the tensor-core kernels is one or two query tiles of floor(128/G)
 selected rows; the cases put the selected rows just below, at and above one
 and two tiles, one row alone, a last item of one row, and positions such that
 the first tile needs fewer 128-key tiles than the second (or only one). The bar
@@ -35,8 +35,7 @@ def _positions(spec, n):
     return np.unique(np.linspace(0, n - 1, spec).round().astype(np.int64)) if spec else np.zeros(0, np.int64)
 
 
-def _run(C, hq, hkv, d, n_r, specs, seed=0, form="plain", dtype=torch.bfloat16):
-    L, G = 2, hq // hkv
+def _run(C, hq, hkv, d, n_r, specs, seed=0, form="plain", dtype=torch.bfloat16, L=2):
     if len(specs) == 2 and isinstance(specs[0], str):
         specs = (specs,)
     pos = [_positions(s, n) for s, n in zip(specs, n_r)]
@@ -51,7 +50,18 @@ def _run(C, hq, hkv, d, n_r, specs, seed=0, form="plain", dtype=torch.bfloat16):
     off, off_dev = C.idx_offsets([len(p) for p in pos])
     idx = torch.tensor(np.concatenate(pos), dtype=torch.int32, device="cuda")
     status = torch.zeros(1, dtype=torch.int32, device="cuda")
-    if form == "plain":
+    if form == "paged":  # pages of 16 tokens, a request's in reverse order
+        pages = [-(-n // 16) for n in n_r]
+        first = np.concatenate([[0], np.cumsum(pages)]).tolist()
+        table = torch.full((R, max(pages)), -1, dtype=torch.int32)
+        pool = [torch.zeros(L, first[-1], hkv, 16, d, dtype=dtype, device="cuda") for _ in range(2)]
+        for r, n in enumerate(n_r):
+            table[r, :pages[r]] = torch.arange(first[r + 1] - 1, first[r] - 1, -1, dtype=torch.int32)
+            for dst, src in zip(pool, (k, v)):
+                rows = torch.nn.functional.pad(src[:, :, tok[r]:tok[r + 1]], (0, 0, 0, 16 * pages[r] - n))
+                dst[:, table[r, :pages[r]].long().cuda()] = rows.view(L, hkv, pages[r], 16, d).transpose(1, 2)
+        kv = C.KvCache(*pool, hq, 16, table)
+    if form in ("plain", "paged"):
         out = C.conduit_refresh_attn(kv, batch, idx, off, off_dev, q_rows, status=status)
     else:  # straight through the ABI: no workspace, or rows that start 2 bytes off a 16-byte boundary
         shift = 1 if form == "misaligned" else 0
@@ -62,7 +72,8 @@ def _run(C, hq, hkv, d, n_r, specs, seed=0, form="plain", dtype=torch.bfloat16):
                                              C._ptr(q_s), C._ptr(out), None, 0, C._ptr(status),
                                              C._stream_ptr(None)))
     assert C.conduit_read_status(status) == C.OK
-    f = lambda t: t.double().cpu().numpy()
+    sub = [0, 1] if L == 2 else [0, L // 2, L - 1]
+    f = lambda t: t[sub].double().cpu().numpy()
     i0 = 0
     for r, p in enumerate(pos):
         if len(p):
@@ -88,6 +99,13 @@ def C():
 def test_item_edges(C, case):
     hq, hkv, d, n_r, specs = CASES[case]
     _run(C, hq, hkv, d, n_r, specs, seed=case)
+
+
+@pytest.mark.parametrize("form", ("plain", "paged"))
+def test_many_items(C, form):
+    """Enough items that a cache in small pages takes two query tiles per item (a contiguous one still
+    takes one), and more K/V than half of L2: both parts of the item order."""
+    _run(C, 14, 2, 128, (1481,), (163,), form=form, L=64)
 
 
 @pytest.mark.parametrize("d", HEAD_DIMS)
