@@ -6,8 +6,12 @@
 // Keys stream through shared memory in tiles of 64 with an online softmax
 // (running max and sum per row) in the log2 domain, up to the tile's last
 // position; every K and V row is read once per tile rather than once per row.
-// What bounds it on the smallest calls is the chain of tiles: fp32, 50 rows of 25
-// selected tokens, 256 keys of 64 dims: 87 us with one warp per row, 40 us now.
+// What bounds it on the smallest calls is the chain of tiles, so where the row
+// tiles leave SMs idle a cluster of up to eight CTAs takes the key tiles of one row
+// tile in turn, and each then merges a part of the rows over the cluster's (max,
+// sum, partial output) through distributed shared memory, in CTA order. fp32, 50
+// rows of 25 selected tokens, 256 keys of 64 dims: 87 us with one warp per row, 40
+// us with one CTA per row tile, 15.5 us with four.
 #include <algorithm>
 
 #include "simt_tile.cuh"
@@ -17,11 +21,13 @@ namespace {
 
 using namespace simt;
 
+constexpr int kMaxSplits = 8;  // CTAs of a cluster
+
 // kDimVecs: float4 accumulators per row and thread, ceil(d / 64)
 template <typename T, int kDimVecs>
 __global__ void __launch_bounds__(kThreads) refresh_simt_kernel(KvDev kv, BatchDev b, const int32_t* idx,
                                                                 const int32_t* idx_off, int32_t n_sel,
-                                                                const T* q_rows, T* out) {
+                                                                const T* q_rows, T* out, int splits) {
   extern __shared__ __align__(16) float sm[];
   const int d = kv.d, G = kv.G, ld = row_stride(d);
   float* q_s = sm;                         // [32][d + 4]
@@ -31,8 +37,10 @@ __global__ void __launch_bounds__(kThreads) refresh_simt_kernel(KvDev kv, BatchD
   constexpr int kPStride = kRowTile + 2;
   __shared__ int64_t q_off_s[kRowTile], k_off_s[kKeyTile];
   __shared__ int pos_s[kRowTile];
+  __shared__ float2 mz_s[kRowTile];        // (max, sum) of this CTA's keys, for its cluster
 
-  int tile = blockIdx.x, r = 0;  // the tile's request and first row
+  const int part = blockIdx.x % splits;    // rank in the cluster
+  int tile = blockIdx.x / splits, r = 0;  // the tile's request and first row
   for (; r < b.R; ++r) {
     const int tiles = int((int64_t(idx_off[r + 1] - idx_off[r]) * G + kRowTile - 1) / kRowTile);
     if (tile < tiles) break;
@@ -73,7 +81,7 @@ __global__ void __launch_bounds__(kThreads) refresh_simt_kernel(KvDev kv, BatchD
   const T* kb = static_cast<const T*>(kv.k);
   const T* vb = static_cast<const T*>(kv.v);
 
-  for (int j0 = 0; j0 <= p_max; j0 += kKeyTile) {
+  for (int j0 = part * kKeyTile; j0 <= p_max; j0 += splits * kKeyTile) {
     __syncthreads();
     if (threadIdx.x < kKeyTile) {
       const int t = j0 + threadIdx.x;
@@ -145,6 +153,41 @@ __global__ void __launch_bounds__(kThreads) refresh_simt_kernel(KvDev kv, BatchD
     else
       add_keys(true);
   }
+  if (splits > 1) {
+    __syncthreads();  // k_s is free
+#pragma unroll
+    for (int a = 0; a < 2; ++a) {
+      if (j == 0) mz_s[2 * i + a] = make_float2(m_run[a], z_run[a]);
+#pragma unroll
+      for (int v = 0; v < kDimVecs; ++v) {
+        const int e = 4 * j + 64 * v;
+        if (e < d) *reinterpret_cast<float4*>(k_s + (2 * i + a) * ld + e) = acc[a][v];
+      }
+    }
+    cluster_barrier();
+    const int rows_part = kRowTile / splits, vecs = d / 4;
+    for (int x = threadIdx.x; x < rows_part * vecs; x += kThreads) {
+      const int row = part * rows_part + x / vecs, e = x % vecs * 4;
+      if (pos_s[row] < 0) continue;
+      float m = -INFINITY, z = 0.f;
+      for (int c = 0; c < splits; ++c) m = fmaxf(m, cluster_ld(&mz_s[row].x, c));
+      const float ref = m == -INFINITY ? 0.f : m;
+      float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+      for (int c = 0; c < splits; ++c) {
+        const float w = exp2f(cluster_ld(&mz_s[row].x, c) - ref);
+        const float4 y = cluster_ld4(k_s + row * ld + e, c);
+        z = fmaf(cluster_ld(&mz_s[row].y, c), w, z);
+        o = make_float4(fmaf(y.x, w, o.x), fmaf(y.y, w, o.y), fmaf(y.z, w, o.z), fmaf(y.w, w, o.w));
+      }
+      T* dst = out + q_off_s[row] + e;
+      dst[0] = from_float<T>(o.x / z);
+      dst[1] = from_float<T>(o.y / z);
+      dst[2] = from_float<T>(o.z / z);
+      dst[3] = from_float<T>(o.w / z);
+    }
+    cluster_barrier();  // no CTA leaves while another may still read its part
+    return;
+  }
 #pragma unroll
   for (int a = 0; a < 2; ++a) {
     if (p_row[a] < 0) continue;
@@ -165,15 +208,25 @@ __global__ void __launch_bounds__(kThreads) refresh_simt_kernel(KvDev kv, BatchD
 
 template <typename T>
 cudaError_t launch(const KvDev& kv, const BatchDev& b, const int32_t* idx, const int32_t* idx_off_dev,
-                   unsigned tiles, int32_t n_sel, const void* q_rows, void* out, cudaStream_t stream) {
+                   unsigned tiles, int splits, int32_t n_sel, const void* q_rows, void* out, cudaStream_t stream) {
   const int ld = row_stride(kv.d);
   const int smem = int(sizeof(float)) * ((kRowTile + 2 * kKeyTile) * ld + kKeyTile * (kRowTile + 2));
   auto go = [&](auto* f) -> cudaError_t {
     cudaError_t err = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (err) return err;
-    f<<<dim3(tiles, kv.Hkv, kv.L), kThreads, smem, stream>>>(kv, b, idx, idx_off_dev, n_sel,
-                                                             static_cast<const T*>(q_rows), static_cast<T*>(out));
-    return cudaGetLastError();
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = splits;
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cfg.gridDim = dim3(tiles * splits, kv.Hkv, kv.L);
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, f, kv, b, idx, idx_off_dev, n_sel, static_cast<const T*>(q_rows),
+                              static_cast<T*>(out), splits);
   };
   return kv.d <= 64 ? go(refresh_simt_kernel<T, 1>)
          : kv.d <= 128 ? go(refresh_simt_kernel<T, 2>) : go(refresh_simt_kernel<T, 4>);
@@ -188,10 +241,18 @@ cudaError_t launch_refresh_simt(const KvDev& kv, const BatchDev& b, const int32_
   int64_t tiles = 0;
   for (int r = 0; r < b.R; ++r)
     tiles += (int64_t(idx_off_host[r + 1] - idx_off_host[r]) * kv.G + kRowTile - 1) / kRowTile;
-  const cudaError_t err =
-      kv.dtype == CONDUIT_BF16
-          ? launch<__nv_bfloat16>(kv, b, idx, idx_off_dev, unsigned(tiles), n_sel, q_rows, out, stream)
-          : launch<float>(kv, b, idx, idx_off_dev, unsigned(tiles), n_sel, q_rows, out, stream);
+  if (tiles == 0) return cudaSuccess;
+  int dev = 0, sms = 0;
+  cudaError_t err;
+  if ((err = cudaGetDevice(&dev))) return err;
+  if ((err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev))) return err;
+  // the largest split that keeps one CTA per SM and a key tile for each
+  const int64_t ctas = tiles * kv.Hkv * kv.L, key_tiles = (kv.n_tot + kKeyTile - 1) / kKeyTile;
+  int splits = kMaxSplits;
+  while (splits > 1 && (ctas * splits > sms || key_tiles < splits)) splits /= 2;
+  err = kv.dtype == CONDUIT_BF16
+            ? launch<__nv_bfloat16>(kv, b, idx, idx_off_dev, unsigned(tiles), splits, n_sel, q_rows, out, stream)
+            : launch<float>(kv, b, idx, idx_off_dev, unsigned(tiles), splits, n_sel, q_rows, out, stream);
   if (err) return err;
   count_launches(1);
   return cudaSuccess;

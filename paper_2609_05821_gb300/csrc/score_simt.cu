@@ -125,13 +125,23 @@ __global__ void __launch_bounds__(kThreads) colsum_kernel(KvDev kv, BatchDev b, 
   const int64_t out0 = int64_t(blockIdx.y) * kv.n_tot + t0 + tt;
 
   key_offsets(kv, l, g, r, t0, N, tt, k_off_s);
+  row_offsets(kv, l, g, q0, nq, q_tot, 0, q_off_s);
   __syncthreads();
   load_rows(k_s, static_cast<const T*>(kv.k), k_off_s, kKeyTile, d, 1.f);
+  load_rows(q_s, q, q_off_s, kRowTile, d, kLog2e * rsqrtf(float(d)));
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-  if (ss != nullptr) {
-    for (int t = warp; t < kKeyTile && tt + t < N; t += kThreads / 32) {
-      const float acc = warp_row_sumsq(static_cast<const T*>(kv.v) + k_off_s[t], d, lane);
-      if (lane == 0) ss[out0 + t] = acc;
+  if (ss != nullptr) {  // the eight rows of a warp are read before the first is written
+    constexpr int kTok = kKeyTile / (kThreads / 32);
+    float sq[kTok];
+#pragma unroll
+    for (int n = 0; n < kTok; ++n) {
+      const int64_t o = k_off_s[warp + n * (kThreads / 32)];
+      sq[n] = o >= 0 ? warp_row_sumsq(static_cast<const T*>(kv.v) + o, d, lane) : 0.f;
+    }
+#pragma unroll
+    for (int n = 0; n < kTok; ++n) {
+      const int t = warp + n * (kThreads / 32);
+      if (lane == 0 && tt + t < N) ss[out0 + t] = sq[n];
     }
   }
 
@@ -139,8 +149,12 @@ __global__ void __launch_bounds__(kThreads) colsum_kernel(KvDev kv, BatchDev b, 
   const int n_chunks = (N + chunk_keys - 1) / chunk_keys;
   float acc[4] = {0.f, 0.f, 0.f, 0.f}, acc2[4] = {0.f, 0.f, 0.f, 0.f};
   for (int row0 = 0; row0 < R; row0 += kRowTile) {
-    __syncthreads();
-    row_offsets(kv, l, g, q0, nq, q_tot, row0, q_off_s);
+    if (row0 > 0) {
+      __syncthreads();
+      row_offsets(kv, l, g, q0, nq, q_tot, row0, q_off_s);
+      __syncthreads();
+      load_rows(q_s, q, q_off_s, kRowTile, d, kLog2e * rsqrtf(float(d)));
+    }
     if (threadIdx.x < kRowTile) {
       const int rr = row0 + threadIdx.x;
       float lse = 0.f;
@@ -159,8 +173,6 @@ __global__ void __launch_bounds__(kThreads) colsum_kernel(KvDev kv, BatchDev b, 
       }
       lse_s[threadIdx.x] = lse;
     }
-    __syncthreads();
-    load_rows(q_s, q, q_off_s, kRowTile, d, kLog2e * rsqrtf(float(d)));
     __syncthreads();
     float x[2][4];
     dots(q_s, k_s, d, x);

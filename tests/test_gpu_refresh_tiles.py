@@ -152,6 +152,8 @@ def test_cuda_core_tiles(C, dtype, d):
     for specs in ((44, 17), (("head", 11), ("tail", 11)), (1, 0)):
         plain = _run(C, 6, 2, d, (300, 141), specs, seed=d, dtype=dtype)
         assert torch.equal(_run(C, 6, 2, d, (300, 141), specs, seed=d, form="misaligned", dtype=dtype), plain)
+    for specs in ((9,), (("head", 1),), (44,)):   # clusters of eight CTAs: keys for all, for one, two row tiles
+        _run(C, 6, 2, d, (700,), specs, seed=d, dtype=dtype)
     test_scores_of_head_dims(C, d, dtype)
 
 
