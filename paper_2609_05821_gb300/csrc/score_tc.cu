@@ -382,7 +382,10 @@ __device__ __forceinline__ float col_sum_sq(const float (&v)[NC], const float* n
   return (ac[0].x + ac[0].y) + (ac[1].x + ac[1].y);
 }
 
-template <int kHalves>
+// kPair: launched in clusters of two. A kernel of its own for one CTA per unit,
+// without the exchange: batched serving 4 869 -> 4 757 us with its tail, 112 units
+// of 64 tiles and 63 rows 132.8 -> 131.5 us.
+template <int kHalves, bool kPair>
 __global__ void __launch_bounds__(kThreads, 1)
     score_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant__ CUtensorMap vmap,
                     const __grid_constant__ TcArgs a) {
@@ -392,7 +395,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   const Smem s = carve<kHalves>(smem_raw);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   // the CTAs (one, or a cluster of two) that share a unit
-  const int rank = int(cluster_rank()), ctas = int(cluster_size());
+  const int rank = kPair ? int(cluster_rank()) : 0, ctas = kPair ? int(cluster_size()) : 1;
   const int unit0 = int(blockIdx.x) / ctas, unit_step = int(gridDim.x) / ctas;
   if (tc::smem_u32(smem_raw) & 1023u) {  // the swizzled tiles need 1024-byte atoms
     if (tid == 0) flag_status(a.status, CONDUIT_FLAG_TIMEOUT | tc::kSiteLoad);
@@ -847,10 +850,16 @@ cudaError_t launch_score_tc(const KvDev& kv, const BatchDev& b, const int32_t* q
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
     cfg.attrs = &attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = ctas > 1;
     return cudaLaunchKernelEx(&cfg, f, kmap, vmap, a);
   };
-  err = kv.d <= 64 ? launch(score_tc_kernel<1>, Shape<1>::kSmemBytes) : launch(score_tc_kernel<2>, Shape<2>::kSmemBytes);
+  const bool pair = ctas > 1;
+  if (kv.d <= 64)
+    err = pair ? launch(score_tc_kernel<1, true>, Shape<1>::kSmemBytes)
+               : launch(score_tc_kernel<1, false>, Shape<1>::kSmemBytes);
+  else
+    err = pair ? launch(score_tc_kernel<2, true>, Shape<2>::kSmemBytes)
+               : launch(score_tc_kernel<2, false>, Shape<2>::kSmemBytes);
   if (err) return err;
   count_launches(1);
   return cudaSuccess;
