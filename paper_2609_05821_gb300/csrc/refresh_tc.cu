@@ -38,7 +38,7 @@
 // one_refresh_tc_kernel: one query tile per item, three S buffers, and the two
 // softmax warps of a lane quarter share each key tile. It takes about 1 650
 // cycles per tile, but its items are half as long, so it is the faster one where
-// few items reach an SM. Roles:
+// few items reach an SM, and for the head sizes below 128 throughout. Roles:
 //   warp 0      items, query tiles (two buffers) and K tiles; warp 10 V tiles
 //   warp 1      S(t) = Q K(t)^T into TMEM buffer t % 3; warp 11 O += P(t) V(t).
 //               Two warps, because one issuing both, with a wait for each P V
@@ -55,9 +55,9 @@
 // path in every key tile (28 heads, 8 192 tokens: 1 254 -> 970 us).
 //
 // Measured (GB300, SM clock 2 070 MHz, before -> now): multi-image prompt 1 254
-// -> 896 us, batched serving 22.6 -> 18.5 ms, long document 15.3 -> 15.0 ms
-// (17.0 -> 16.3 ms back to back, under the power cap), single image 45.5 -> 42.8
-// us, 16 layers of 4 096 tokens 225 -> 196 us.
+// -> 891 us, batched serving 22.6 -> 18.5 ms, long document 15.3 -> 15.0 ms
+// (19.0 -> 18.0 ms back to back, under the power cap), single image 45.3 -> 42.5
+// us, 16 layers of 4 096 tokens 225 -> 196 us, 2 layers of 1 885 25.2 -> 20.6 us.
 //
 // The staleness estimator (kStale) runs the same schedule with every scoring row
 // of a request at its last key: V is the draw z itself, the softmax warps scale
@@ -852,6 +852,7 @@ __device__ __forceinline__ bool softmax_all(bool pred) {
   return out != 0;
 }
 
+template <int kHalves, bool kSplit>
 __global__ void __launch_bounds__(kThreads, 1)
     one_refresh_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant__ CUtensorMap vmap,
                       const __grid_constant__ CUtensorMap qmap, const __grid_constant__ RefArgs a) {
@@ -859,7 +860,9 @@ __global__ void __launch_bounds__(kThreads, 1)
   const OneSmem s = carve_one(smem_raw);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const KvDev& kv = a.kv;
+  constexpr int kDP = 64 * kHalves, kOW = kDP / 2;  // kOW: columns of O of a softmax thread
   const int G = kv.G, Hq = kv.Hq;
+  const int d = kHalves == 2 && !kSplit ? kMaxD : kv.d;
   const int qrows = a.rows_per_tile * G;          // rows the query box fills
 
   if (tid == 0) {
@@ -952,8 +955,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (u < 0) {
           tc::mbar_arrive(&s.qfull[qs]);  // no more work: the others stop at this buffer
         } else {
-          tc::mbar_arrive_expect_tx(&s.qfull[qs], 2u * 128u * uint32_t(qrows));
-          for (int hf = 0; hf < 2; ++hf)
+          tc::mbar_arrive_expect_tx(&s.qfull[qs], uint32_t(kHalves) * 128u * uint32_t(qrows));
+          for (int hf = 0; hf < kHalves; ++hf)
             tc::tma_load_3d(s.q + qs * kQBytes + hf * kHalfBytes, &qmap, &s.qfull[qs], hf * 64,
                             it.g * G, it.l * a.n_sel + it.i0);
         }
@@ -966,7 +969,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           ok = false;
           break;
         }
-        load_tile<2>(a, &kmap, s.k + sk * kOneTileBytes, &s.kfull[sk], it.l, it.g, it.r, t0, N, t * kKT, lane);
+        load_tile<kHalves>(a, &kmap, s.k + sk * kOneTileBytes, &s.kfull[sk], it.l, it.g, it.r, t0, N, t * kKT, lane);
         ++nk;
       }
     }
@@ -996,7 +999,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           ok = false;
           break;
         }
-        load_tile<2>(a, &vmap, s.v + sv * kOneTileBytes, &s.vfull[sv], l, g, r, t0, N, t * kKT, lane);
+        load_tile<kHalves>(a, &vmap, s.v + sv * kOneTileBytes, &s.vfull[sv], l, g, r, t0, N, t * kKT, lane);
         ++nv;
       }
       if (!ok) break;
@@ -1027,10 +1030,11 @@ __global__ void __launch_bounds__(kThreads, 1)
         __syncwarp();
         tc::tc_fence_after();
         const uint64_t dk = tc::desc_sw128(tc::smem_u32(s.k + sk * kOneTileBytes));
+        const int ksteps = kSplit ? (d + 15) / 16 : kDP / 16;
 #pragma unroll
-        for (int kk = 0; kk < 8; ++kk) {
+        for (int kk = 0; kk < kDP / 16; ++kk) {
           const uint32_t off = ((kk >> 2) * kHalfBytes + (kk & 3) * 32) >> 4;
-          tc::mma_bf16_if(leader, tm + b * kSCols, dq + off, dk + off, idesc_s, kk > 0);
+          if (kk < ksteps) tc::mma_bf16_if(leader, tm + b * kSCols, dq + off, dk + off, idesc_s, kk > 0);
         }
         tc::mma_commit_if(leader, &s.sfull[b]);
         tc::mma_commit_if(leader, &s.kempty[sk]);
@@ -1046,7 +1050,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const uint32_t leader = lane == 0;
     uint32_t T = 0;
     bool ok = true;
-    const uint32_t idesc_o = tc::idesc_bf16(kRows, kMaxD, /*b_mn_major=*/true);
+    const uint32_t idesc_o = tc::idesc_bf16(kRows, kDP, /*b_mn_major=*/true);
     const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
     for (uint32_t n = 0; ok; ++n) {
       const int qs = n & 1;
@@ -1065,10 +1069,15 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (t == 0 && n > 0 && !(ok = wait_warp(s.oempty, (n - 1) & 1, s.abort))) break;
         tc::tc_fence_after();
         const uint64_t dv = tc::desc_sw128_mn(tc::smem_u32(s.v + sv * kOneTileBytes), kHalfBytes);
-        const uint32_t pb = tm + b * kSCols + kPCol;
+        const uint32_t pb = tm + b * kSCols;
 #pragma unroll
         for (int kk = 0; kk < kKT / 16; ++kk)  // O += P(t) V(t)
-          tc::mma_bf16_ts_if(leader, tm + kOneOCol, pb + kk * 8, dv + kk * (2048 >> 4), idesc_o, t > 0 || kk > 0);
+          tc::mma_bf16_ts_if(leader, tm + kOneOCol, pb + kPCol + kk * 8, dv + kk * (2048 >> 4), idesc_o, t > 0 || kk > 0);
+        if (kSplit) {
+#pragma unroll
+          for (int kk = 0; kk < kKT / 16; ++kk)
+            tc::mma_bf16_ts_if(leader, tm + kOneOCol, pb + kPLoCol + kk * 8, dv + kk * (2048 >> 4), idesc_o, true);
+        }
         tc::mma_commit_if(leader, &s.pvdone[b]);
         tc::mma_commit_if(leader, &s.vempty[sv]);
       }
@@ -1159,14 +1168,15 @@ __global__ void __launch_bounds__(kThreads, 1)
         // this half of P = 2^(S scale - m) in bf16 pairs over the upper half of S
         // (one packed FMA per pair for scale and bias, packed adds for the sum).
         // A row with no visible key yet (m = -inf) uses bias 0: its logits are
-        // all -inf and its P is 0.
+        // all -inf and its P is 0. Both halves of S have been read (the barrier
+        // above), so either thread may write over the other's half.
         const float2 sc2 = make_float2(a.scale_log2, a.scale_log2);
         const float2 nb2 = m_ref == -INFINITY ? make_float2(0.f, 0.f) : make_float2(-m_ref, -m_ref);
         float2 ls2[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
         {
 #pragma unroll
           for (int c = 0; c < 2; ++c) {
-            uint32_t pw[16];
+            uint32_t pw[16], lo[16];
 #pragma unroll
             for (int i = 0; i < 16; ++i) {
               const float2 y = tc::ffma2(make_float2(sv[32 * c + 2 * i], sv[32 * c + 2 * i + 1]), sc2, nb2);
@@ -1174,8 +1184,14 @@ __global__ void __launch_bounds__(kThreads, 1)
               ls2[i & 1] = tc::fadd2(ls2[i & 1], pp);
               __nv_bfloat162 pr = __floats2bfloat162_rn(pp.x, pp.y);
               pw[i] = *reinterpret_cast<uint32_t*>(&pr);
+              if (kSplit) {
+                const float2 hi = __bfloat1622float2(pr);
+                pr = __floats2bfloat162_rn(pp.x - hi.x, pp.y - hi.y);
+                lo[i] = *reinterpret_cast<uint32_t*>(&pr);
+              }
             }
             tc::tmem_st16_nowait(sb + kPCol + hh * 32 + 16 * c, pw);
+            if (kSplit) tc::tmem_st16_nowait(sb + kPLoCol + hh * 32 + 16 * c, lo);
           }
           tc::tmem_wait_st();
         }
@@ -1193,7 +1209,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             continue;
           }
           tc::tc_fence_after();
-          for (int c = hh * 64; c < hh * 64 + 64; c += 32) {
+          for (int c = hh * kOW; c < hh * kOW + kOW; c += 32) {
             float o[32];
             tc::tmem_ld32(tl + kOneOCol + c, o);
 #pragma unroll
@@ -1219,31 +1235,34 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (fin) {
         tc::tc_fence_after();
         const float inv = total > 0.f ? 1.f / total : 0.f;
-        __nv_bfloat16* dst = a.out + ((int64_t(it.l) * a.n_sel + i_row) * Hq + h_row) * kMaxD;
-        // This thread's 64 columns of O in one load, then its half row as
-        // bf16. Each lane writes its own row, so a warp's store covers 32
-        // rows: 32-byte stores (whole sectors) when the buffer allows them.
-        float o[64];
-        tc::tmem_ld64(tl + kOneOCol + hh * 64, o);
-        if (live) {
-          uint32_t w[32];
+        __nv_bfloat16* dst = a.out + ((int64_t(it.l) * a.n_sel + i_row) * Hq + h_row) * d;
+        // This thread's columns of O, 32 at a time, as bf16. Each lane writes its own
+        // row, so a warp's store covers 32 rows: 32-byte stores (whole sectors)
+        // when the buffer allows them.
 #pragma unroll
-          for (int k2 = 0; k2 < 32; ++k2) {
+        for (int c = hh * kOW; c < hh * kOW + kOW; c += 32) {
+          float o[32];
+          tc::tmem_ld32(tl + kOneOCol + c, o);
+          if (!live) continue;
+          uint32_t w[16];
+#pragma unroll
+          for (int k2 = 0; k2 < 16; ++k2) {
             __nv_bfloat162 pr = __floats2bfloat162_rn(o[2 * k2] * inv, o[2 * k2 + 1] * inv);
             w[k2] = *reinterpret_cast<uint32_t*>(&pr);
           }
-          __nv_bfloat16* drow = dst + hh * 64;
           if (a.out32) {
 #pragma unroll
-            for (int u8 = 0; u8 < 4; ++u8)
-              asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(drow + u8 * 16),
-                           "r"(w[8 * u8]), "r"(w[8 * u8 + 1]), "r"(w[8 * u8 + 2]), "r"(w[8 * u8 + 3]),
-                           "r"(w[8 * u8 + 4]), "r"(w[8 * u8 + 5]), "r"(w[8 * u8 + 6]), "r"(w[8 * u8 + 7])
-                           : "memory");
+            for (int u8 = 0; u8 < 2; ++u8)
+              if (c + u8 * 16 < d)
+                asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst + c + u8 * 16),
+                             "r"(w[8 * u8]), "r"(w[8 * u8 + 1]), "r"(w[8 * u8 + 2]), "r"(w[8 * u8 + 3]),
+                             "r"(w[8 * u8 + 4]), "r"(w[8 * u8 + 5]), "r"(w[8 * u8 + 6]), "r"(w[8 * u8 + 7])
+                             : "memory");
           } else {
 #pragma unroll
-            for (int u4 = 0; u4 < 8; ++u4)
-              *reinterpret_cast<uint4*>(drow + u4 * 8) = make_uint4(w[4 * u4], w[4 * u4 + 1], w[4 * u4 + 2], w[4 * u4 + 3]);
+            for (int u4 = 0; u4 < 4; ++u4)
+              if (c + u4 * 8 < d)
+                *reinterpret_cast<uint4*>(dst + c + u4 * 8) = make_uint4(w[4 * u4], w[4 * u4 + 1], w[4 * u4 + 2], w[4 * u4 + 3]);
           }
         }
       }
@@ -1333,8 +1352,11 @@ static int query_blocks(const BatchDev& b, const int32_t* off_host, int span) {
   return blocks;
 }
 
-// One query tile per item or two, for head_dim 128 (the smaller sizes have the
-// two-tile kernel only), by the key tiles that two-tile items would bring to an
+// One query tile per item or two. The split P of the smaller head sizes makes a
+// tile's softmax and P V longer, and one tile per item is faster throughout (24
+// layers, 14/2 heads of 64 dims: 2 916 tokens 93 us / 107 with two, 24 576 tokens
+// 4 636 / 4 747; 16 layers, 32/8 heads of 96 dims, 16 384 tokens 3 229 / 3 855).
+// For head_dim 128 it goes by the key tiles that two-tile items would bring to an
 // SM. Two-tile items are half as many and cost less per tile, which pays once
 // the end of the launch no longer shows (one / two tiles per item, us):
 // 2 layers x 1 885 tokens 22.6 / 35.0, 28 x 1 024 42.8 / 45.0, 36 x 4 096 (213
@@ -1350,6 +1372,12 @@ constexpr int kOneMinPage = 32;
 // L2: 0 / 2 / 3 / 4 items took 213 / 196 / 196.5 / 199 us on 16 layers of 4 096
 // tokens (one tile per item) and 952 / 908 / 896 / 904 us on 28 of 8 192 (two).
 constexpr int kTailItemsPerSm = 3;
+// Up to this many one-tile items per SM come in a fixed order (they are then
+// longest first throughout): a counter costs its reset and an atomic per item, and
+// evens out more items than that. Fixed / counter, us: 2 layers of 1 885 tokens (96
+// items) 20.5 / 22.6, 28 of 600 (448) 26.7 / 28.3, three requests of 1 024 (576)
+// 38.5 / 38.9, 28 of 1 024 (672) 44.5 / 43.0, 14 of 2 000 (672) 58.0 / 54.6.
+constexpr int kDealtItemsPerSm = 3;
 
 cudaError_t launch_refresh_tc(const KvDev& kv, const BatchDev& b, const int32_t* idx,
                               const int32_t* idx_off_dev, const int32_t* idx_off_host, int32_t n_sel,
@@ -1379,13 +1407,13 @@ cudaError_t launch_refresh_tc(const KvDev& kv, const BatchDev& b, const int32_t*
   a.n_blocks = query_blocks(b, idx_off_host, a.span);
   const double key_tiles = double(a.n_blocks) * n_lg * (double(kv.n_tot) / b.R) / (2 * kKT);
   const bool few_copies = kv.page_size == 0 || kv.page_size >= kOneMinPage;
-  const bool one = kv.d == kMaxD && key_tiles < sms * (few_copies ? kOneKeyTilesPerSm : kOneKeyTilesPerSmPaged);
+  const bool one = kv.d != kMaxD || key_tiles < sms * (few_copies ? kOneKeyTilesPerSm : kOneKeyTilesPerSmPaged);
   if (one) {
     a.span = a.rows_per_tile;
     a.n_blocks = query_blocks(b, idx_off_host, a.span);
   }
   a.n_items = a.n_blocks * n_lg;
-  a.next_item = work_counter;
+  a.next_item = a.n_items <= (one ? kDealtItemsPerSm * sms : sms) ? nullptr : work_counter;
   a.scale_log2 = kLog2e / sqrtf(float(kv.d));
   a.status = status;
   if (a.n_blocks == 0) return cudaSuccess;
@@ -1394,7 +1422,7 @@ cudaError_t launch_refresh_tc(const KvDev& kv, const BatchDev& b, const int32_t*
   // items of each SM
   const double kv_bytes = 2.0 * double(n_lg) * double(kv.n_tot) * kv.d * 2;
   a.tail = kv_bytes <= 0.5 * double(l2) ? n_lg : std::min(n_lg, (kTailItemsPerSm * sms + a.n_blocks - 1) / a.n_blocks);
-  if (work_counter && (err = cudaMemsetAsync(work_counter, 0, sizeof(int32_t), stream))) return err;
+  if (a.next_item && (err = cudaMemsetAsync(work_counter, 0, sizeof(int32_t), stream))) return err;
   auto launch = [&](auto* f, uint32_t smem) -> cudaError_t {
     if ((err = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)))) return err;
     f<<<std::min(a.n_items, sms), kThreads, smem, stream>>>(kmap, vmap, qmap, a);
@@ -1402,14 +1430,14 @@ cudaError_t launch_refresh_tc(const KvDev& kv, const BatchDev& b, const int32_t*
   };
   // head_dim 128 keeps its bf16 P; the smaller sizes ran with fp32 weights on
   // CUDA cores before and keep that precision by a split P
-  if (one)
-    err = launch(one_refresh_tc_kernel, kOneSmem);
-  else if (kv.d == kMaxD)
+  if (!one)
     err = launch(refresh_tc_kernel<2, false>, Shape<2>::kSmem);
+  else if (kv.d == kMaxD)
+    err = launch(one_refresh_tc_kernel<2, false>, kOneSmem);
   else if (kv.d > 64)
-    err = launch(refresh_tc_kernel<2, true>, Shape<2>::kSmem);
+    err = launch(one_refresh_tc_kernel<2, true>, kOneSmem);
   else
-    err = launch(refresh_tc_kernel<1, true>, Shape<1>::kSmem);
+    err = launch(one_refresh_tc_kernel<1, true>, kOneSmem);
   if (err) return err;
   count_launches(1);
   return cudaSuccess;

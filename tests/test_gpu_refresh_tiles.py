@@ -101,11 +101,12 @@ def test_item_edges(C, case):
     _run(C, hq, hkv, d, n_r, specs, seed=case)
 
 
-@pytest.mark.parametrize("form", ("plain", "paged"))
-def test_many_items(C, form):
-    """Enough items that a cache in small pages takes two query tiles per item (a contiguous one still
-    takes one), and more K/V than half of L2: both parts of the item order."""
-    _run(C, 14, 2, 128, (1481,), (163,), form=form, L=64)
+@pytest.mark.parametrize("form,d", [("plain", 128), ("paged", 128), ("plain", 96), ("plain", 40)])
+def test_many_items(C, form, d):
+    """Enough items for the work counter (fewer are dealt out in a fixed order), and that a cache in small
+    pages takes two query tiles per item (a contiguous one takes one); at 96 and 128 dims more K/V than half
+    of L2, so both parts of the item order."""
+    _run(C, 14, 2, d, (1481,), (163,), form=form, L=64)
 
 
 @pytest.mark.parametrize("d", HEAD_DIMS)
