@@ -550,10 +550,19 @@ __global__ void __launch_bounds__(kThreads, 1)
     uint32_t Tv = 0;                                     // (kStale) the CTA's V tiles
     // (kStale) this query tile's share of scaling V tile t of the item: thread j
     // scales its half of row j by the key's deviation
-    auto scale_v = [&](const float* scale, int t, int N) {
+    // `ahead`: this stream has not seen an S of the tile before. Then K(T - kAhead),
+    // which had V(T)'s slot before it, may still be on its way, and the wait for the
+    // slot's phase would take its unfinished phase for the one after it; so wait
+    // first, as the loader does, until that tile is done.
+    auto scale_v = [&](const float* scale, int t, int N, bool ahead) {
       const int j = t * kKT + row;
       const float sc = j < N ? scale[j] : 0.f;
       const uint32_t e = 2 * Tv + 1, sl = e % kStages;
+      if (ahead && Tv >= uint32_t(kAhead) &&
+          !wait_warp(&s.done[(Tv - kAhead) % kDone], ((Tv - kAhead) / kDone) & 1, s.abort)) {
+        if (lane == 0) raise_abort(a, s.abort, tc::kSiteLoad);
+        return false;
+      }
       if (!wait_warp(&s.full[sl], (e / kStages) & 1, s.abort)) {
         if (lane == 0) raise_abort(a, s.abort, tc::kSiteLoad);
         return false;
@@ -615,7 +624,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (kStale) {
         key_scale = a.key_scale + (int64_t(l) * kv.Hkv + g) * kv.n_tot + t0;
         // V(0), or every V tile when no rows of the item are in this query tile
-        for (int t = 0; t < (nt == 0 ? nt_all : 1) && ok; ++t) ok = scale_v(key_scale, t, N);
+        for (int t = 0; t < (nt == 0 ? nt_all : 1) && ok; ++t) ok = scale_v(key_scale, t, N, true);
       }
       float m_ref = -INFINITY, lsum = 0.f;  // running max (scaled, log2 units) and row sum
       for (int t = 0; t < nt && ok; ++t, ++ns) {
@@ -691,7 +700,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         // S_B(t) was the last to read K(t) and, in issue order, comes after both
         // P V of the tile before: their slots may be loaded again
         tc::mbar_arrive_if(releases, &s.done[ns % kDone]);
-        if (kStale && t + 1 < nt && !scale_v(key_scale, t + 1, N)) {
+        if (kStale && t + 1 < nt && !scale_v(key_scale, t + 1, N, false)) {
           ok = false;
           break;
         }

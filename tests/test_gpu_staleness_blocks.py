@@ -1,0 +1,39 @@
+"""Staleness with blocks of queries that leave the first query tile empty: paged and contiguous agree bit for bit.
+
+With G = 7 a work item holds 2 x 18 queries; 37 to 54 of them leave a last block whose first tile has no rows.
+Its softmax warps scale value tiles ahead of any logits, while the copies of a paged K (one per page half) land
+late. Short requests make many such items follow one another.
+"""
+
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("d", (128, 96, 64))
+def test_paged_equals_contiguous(d):
+    from paper_2609_05821_gb300 import _build
+    _build.build()
+    from paper_2609_05821_gb300 import conduit as C
+    L, hq, hkv, R, M, page = 11, 28, 4, 16, 2, 16
+    n_r = [16 * (12 + r) for r in range(R)]
+    nq = [37 + r for r in range(R)]
+    cum = lambda x: [sum(x[:i]) for i in range(len(x) + 1)]
+    tok, qo = cum(n_r), cum(nq)
+    rng = torch.Generator(device="cuda").manual_seed(d)
+    draw = lambda *shape: torch.randn(shape, generator=rng, device="cuda").bfloat16()
+    k, v, q, z = draw(L, hkv, tok[-1], d), draw(L, hkv, tok[-1], d), draw(L, hq, qo[-1], d), draw(M, L, hkv, tok[-1], d)
+    pages = tok[-1] // page
+    order = torch.randperm(pages, generator=rng, device="cuda")
+    pool = lambda t: t.view(L, hkv, pages, page, d).transpose(1, 2)[:, torch.argsort(order)].contiguous()
+    table = torch.full((R, max(n_r) // page), -1, dtype=torch.int32)
+    for r in range(R):
+        table[r, :n_r[r] // page] = order[tok[r] // page:tok[r + 1] // page].cpu().int()
+    batch = C.Batch(tok, tok, list(range(R + 1)), qo, device="cuda")
+    mask = (torch.rand(tok[-1], generator=rng, device="cuda") < 0.1).to(torch.uint8)
+    run = lambda kv: C.conduit_staleness_iso(kv, batch, q, mask, z, 0.5)[0]
+    want = run(C.KvCache(k, v, hq))
+    paged = C.KvCache(pool(k), pool(v), hq, page, table)
+    for _ in range(20):
+        assert torch.equal(run(paged), want)
