@@ -177,16 +177,15 @@ conduit_status read_opts(const conduit_score_opts* o, ScoreMode* m) {
 }
 
 // Without value partials (vmode != 0) there is no ss region; the RMS
-// statistic adds a pa2 region of the size of pa. `least`: the layout that takes
-// the least scratch, on the CUDA cores with one key chunk where head_dim is not 128.
+// statistic adds a pa2 region of the size of pa.
 ScoreLayout score_layout(const conduit_kv* kv, const conduit_batch* b, int n_layers,
-                         const ScoreMode& mode, bool least = false) {
+                         const ScoreMode& mode) {
   const bool normed = mode.vmode != 0;
   const int R = b->num_requests;
   const size_t n_tot = size_t(b->tok_off[R]);
   const size_t q_tot = size_t(b->q_off[R]);
   ScoreLayout s{};
-  s.tc = score_tc_supported(make_kv(kv, b)) && (!least || kv->head_dim == 128);
+  s.tc = score_tc_supported(make_kv(kv, b));
   s.rg_max = 1;
   s.parts = s.tc ? 2 : 1;
   if (s.tc) {
@@ -204,7 +203,7 @@ ScoreLayout score_layout(const conduit_kv* kv, const conduit_batch* b, int n_lay
       max_tok = std::max(max_tok, b->tok_off[r + 1] - b->tok_off[r]);
       rows += kv->num_q_heads / kv->num_kv_heads * (b->q_off[r + 1] - b->q_off[r]);
     }
-    s.chunks = least ? 1 : score_simt_chunks(make_kv(kv, b), n_layers, rows, max_tok);
+    s.chunks = score_simt_chunks(make_kv(kv, b), n_layers, rows, max_tok);
     off += align_up(size_t(total_rows) * s.chunks * sizeof(float2));
   }
   const size_t pa_bytes =
@@ -287,10 +286,9 @@ struct FusedLayout {
   size_t arrivals, keys, total;
 };
 
-FusedLayout fused_layout(const conduit_kv* kv, const conduit_batch* b, int n_layers, const ScoreMode& mode,
-                         bool least = false) {
+FusedLayout fused_layout(const conduit_kv* kv, const conduit_batch* b, int n_layers, const ScoreMode& mode) {
   FusedLayout f;
-  f.score = score_layout(kv, b, n_layers, mode, least);
+  f.score = score_layout(kv, b, n_layers, mode);
   f.arrivals = f.score.total;
   f.keys = f.arrivals + align_up(size_t(b->num_requests) * sizeof(int32_t));
   f.total = f.keys + align_up(size_t(b->tok_off[b->num_requests]) * sizeof(uint32_t));
@@ -317,10 +315,7 @@ conduit_status score_impl(const conduit_kv* kv, const conduit_batch* batch, cons
   if ((st = make_layers(kv, layers, n_layers, &ll))) return st;
   const bool normed = mode.vmode != 0;
   if (mode.vmode == 1 && (st = check_norm_cache(kv, mode.vnorm))) return st;
-  FusedLayout flay = fused_layout(kv, batch, ll.n, mode);
-  // a workspace below the size query's answer that still holds the least layout is taken
-  if (workspace && workspace_bytes < (tail ? flay.total : flay.score.total))
-    flay = fused_layout(kv, batch, ll.n, mode, /*least=*/true);
+  const FusedLayout flay = fused_layout(kv, batch, ll.n, mode);
   const ScoreLayout& lay = flay.score;
   if ((st = check_workspace(workspace, workspace_bytes, tail ? flay.total : lay.total))) return st;
 

@@ -169,21 +169,3 @@ def test_values_past_a_position_add_nothing(C):
     v[:, :, 50] = float("inf")
     got = C.conduit_refresh_attn(C.KvCache(k, v, 1), batch, idx, off, off_dev, q_rows)
     assert torch.equal(got[:, 0], clean[:, 0]) and not torch.isfinite(got[:, 1]).any()
-
-
-@pytest.mark.parametrize("dtype,d", [(torch.float32, 64), (torch.bfloat16, 64)])
-def test_scores_in_the_least_workspace(C, dtype, d):
-    """A workspace for one key chunk on the CUDA cores, less than the size query asks for, is taken."""
-    L, hq, hkv, n, nq = 2, 6, 2, 700, 90
-    up = lambda x: (x + 255) // 256 * 256
-    least = up(8 * L * hq * nq) + 2 * up(4 * L * hkv * n) + up(4 * n)   # statistics, column sums, value sums, A
-    rng = torch.Generator(device="cuda").manual_seed(d)
-    draw = lambda *shape: torch.randn(shape, generator=rng, device="cuda").to(dtype)
-    kv = C.KvCache(draw(L, hkv, n, d), draw(L, hkv, n, d), hq)
-    q, batch = draw(L, hq, nq, d), C.Batch([0, n], [0, 300, n], [0, 2], [0, nq], device="cuda")
-    assert C.conduit_score_workspace_size(kv, batch) > least
-    ws = torch.empty(least, dtype=torch.uint8, device="cuda")
-    for a, b in zip(C.conduit_score(kv, batch, q, workspace=ws), C.conduit_score(kv, batch, q)):
-        assert torch.allclose(a, b, rtol=1e-5)   # the same sums in fp32, in another order
-    with pytest.raises(C.ConduitError):
-        C.conduit_score(kv, batch, q, workspace=ws[:-256])
