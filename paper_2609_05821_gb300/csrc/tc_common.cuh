@@ -196,20 +196,6 @@ __device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t a_desc, uint6
       : "memory");
 }
 
-// D[tmem] (+)= A[tmem] * B[smem]: A (M x 16, bf16 pairs packed in 8 columns
-// of each lane) is read from tensor memory.
-__device__ __forceinline__ void mma_bf16_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc,
-                                            uint32_t idesc, bool accumulate) {
-  asm volatile(
-      "{\n"
-      ".reg .pred p;\n"
-      "setp.ne.b32 p, %4, 0;\n"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n"
-      "}\n" ::"r"(d_tmem),
-      "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate ? 1u : 0u)
-      : "memory");
-}
-
 // Arrive on *bar once every MMA issued so far by this thread has completed.
 __device__ __forceinline__ void mma_commit(uint64_t* bar) {
   asm volatile(
@@ -223,7 +209,8 @@ __device__ __forceinline__ void mma_commit(uint64_t* bar) {
 // operands live in uniform registers, so that the issue of an MMA costs less
 // than its 64 tensor cycles even beside busy warps (a loop run by one lane of
 // a diverged warp took 83 cycles per 128x128x16 MMA beside eight softmax warps,
-// this form 64).
+// this form 64). With _ts, A (M x 16, bf16 pairs packed in 8 columns of each lane)
+// is read from tensor memory.
 __device__ __forceinline__ void mma_bf16_if(uint32_t leader, uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc,
                                             uint32_t idesc, bool accumulate) {
   asm volatile(
