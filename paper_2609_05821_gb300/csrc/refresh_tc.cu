@@ -98,7 +98,8 @@ template <int kHalves>
 struct Shape {
   static constexpr uint32_t kTileBytes = kHalves * kHalfBytes;
   // K and V tiles in one ring, K(0) V(0) K(1) V(1) ...: tile T may be loaded
-  // once tile T - kAhead is done, and fewer than kDone tiles are undecided
+  // once tile T - kAhead is done (by both streams), and fewer than kDone tiles
+  // are undecided
   static constexpr int kStages = kHalves == 1 ? 9 : 5;
   static constexpr int kAhead = (kStages - 1) / 2;
   static constexpr int kDone = 2 * kAhead;
@@ -187,7 +188,7 @@ struct Smem {
   uint8_t* q;        // [2 tiles][halves][128 rows][128 B]
   uint8_t* kv;       // [kStages][halves][128 keys][128 B]: K tile t of the CTA in slot 2t mod kStages, V in 2t + 1
   uint64_t* full;             // [kStages]
-  uint64_t* done;             // [kDone] tile T of the CTA: K(T) and V(T - 1) have been used
+  uint64_t* done;             // [kDone] tile T of the CTA: both streams have used K(T) and V(T - 1)
   uint64_t *sfull, *pfull;    // [2] per query tile: S computed / P written
   uint64_t *ofull;            // [2] per query tile, once per item that has rows in it: O complete
   uint64_t* qfull;            // [2] per query tile
@@ -307,7 +308,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 
   if (tid == 0) {
     for (int i = 0; i < kStages; ++i) tc::mbar_init(&s.full[i], 1);
-    for (int i = 0; i < kDone; ++i) tc::mbar_init(&s.done[i], 1);
+    for (int i = 0; i < kDone; ++i) tc::mbar_init(&s.done[i], 2);    // A's MMAs, B's softmax
     for (int i = 0; i < kDone; ++i) tc::mbar_init(&s.scaled[i], 8);  // the softmax warps
     for (int i = 0; i < 2; ++i) {
       tc::mbar_init(&s.sfull[i], 1);
@@ -447,7 +448,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     // --------------------------- query tile and MMAs of one stream (warps 1, 3)
     // the whole warp walks the schedule on uniform values, one lane issues
     const int x = __shfl_sync(0xffffffffu, warp == kMmaWarp ? 0 : 1, 0);
-    const uint32_t leader = lane == 0;
+    const uint32_t leader = lane == 0, frees = x == 0 ? leader : 0u;
     uint32_t T = 0, turn = 0, np = 0, nq = 0, cq = 0;  // tiles, turns, P tiles, query tiles loaded / consumed
     const uint32_t idesc_s = tc::idesc_bf16(kRows, kKT);
     const uint32_t idesc_o = tc::idesc_bf16(kRows, kDP, /*b_mn_major=*/true);
@@ -528,7 +529,12 @@ __global__ void __launch_bounds__(kThreads, 1)
         } else {
           tc::mbar_arrive_if(leader, &s.turn[x ^ 1]);
         }
-        if (more) ++T;
+        if (more) {
+          // A's share of done[T]: S_A(T) and P_A(T - 1) V(T - 1) have completed, or
+          // A's last MMAs where it has no rows left
+          tc::mma_commit_if(frees, &s.done[T % kDone]);
+          ++T;
+        }
       }
       if (!ok) break;
     }
@@ -697,8 +703,9 @@ __global__ void __launch_bounds__(kThreads, 1)
         tc::tc_fence_before();
         __syncwarp();
         tc::mbar_arrive_if(leader, &s.pfull[x]);
-        // S_B(t) was the last to read K(t) and, in issue order, comes after both
-        // P V of the tile before: their slots may be loaded again
+        // B's share of done: S_B(t) has completed and, in warp 3's issue order, so has
+        // P_B(t-1) V(t-1). Warp 1 commits A's, which this says nothing of: its last
+        // MMAs of a turn may be issued after the turn has passed to B.
         tc::mbar_arrive_if(releases, &s.done[ns % kDone]);
         if (kStale && t + 1 < nt && !scale_v(key_scale, t + 1, N, false)) {
           ok = false;
