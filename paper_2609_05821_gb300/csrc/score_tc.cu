@@ -153,7 +153,7 @@ struct Smem {
   uint64_t* vempty;    // [kVBufs]
   uint64_t* tfull;     // [2]
   uint64_t* tempty;    // [2]
-  uint64_t* qready;    // [1]
+  uint64_t* qready;    // [1] the rows of a unit that has tiles are staged
   uint64_t* mdone;     // [1]
   uint64_t* peer;      // [2] the peer CTA has written its row statistics of a unit (by unit parity)
   uint32_t* tmem_slot;
@@ -481,7 +481,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int ksteps = (a.kv.d + 15) / 16;  // 16-dim steps that are not all padding
     for (int u = unit0; u < a.n_units && ok; u += unit_step) {
       Unit w;
-      if (!decode_unit(a, u, w, rank, ctas)) continue;
+      if (!decode_unit(a, u, w, rank, ctas) || w.tiles == 0) continue;
       if (!wait_or_abort(s.qready, useq & 1, s.abort)) {
         if (!*s.abort) raise_abort(a, s, tc::kSiteMma);
         break;
@@ -559,10 +559,15 @@ __global__ void __launch_bounds__(kThreads, 1)
       Unit w;
       if (!decode_unit(a, u, w, rank, ctas)) continue;
       const int nrb = (w.rows + 127) / 128;
-      if (ok && !*s.abort) stage_rows<kHalves>(a, w, s.q, nrb * 128, et);
-      tc::fence_proxy_async_smem();
-      epi_barrier();
-      if (et == 0) tc::mbar_arrive(s.qready);
+      if (w.tiles > 0) {
+        // A CTA of a pair has no tiles in a unit of one tile. Nothing then waits for
+        // the MMA thread, so an arrival there could come a phase before that thread
+        // has seen the last one: neither role counts such a unit's rows.
+        if (ok && !*s.abort) stage_rows<kHalves>(a, w, s.q, nrb * 128, et);
+        tc::fence_proxy_async_smem();
+        epi_barrier();
+        if (et == 0) tc::mbar_arrive(s.qready);
+      }
       // pass A share: row block rb (with one row block the second warp group
       // only does value norms) and this thread's half of each V row
       const bool do_rows = nrb == 2 || h == 0;
@@ -783,6 +788,13 @@ static int ctas_per_unit(int units, int tiles, int sms) {
   const int64_t two = int64_t((units + pairs - 1) / pairs) * ((tiles + 1) / 2 + 4);
   return two * 20 < one * 19 ? 2 : 1;
 }
+
+#ifdef CONDUIT_TEST_HOOKS
+// Test builds only: the CTAs that share a unit of such a launch.
+extern "C" int32_t conduit_test_score_ctas(int32_t units, int32_t tiles, int32_t sms) {
+  return ctas_per_unit(units, tiles, sms);
+}
+#endif
 
 cudaError_t launch_score_tc(const KvDev& kv, const BatchDev& b, const int32_t* q_off_host, int max_tokens,
                             const void* q, int32_t q_tot, const LayerList& layers, int rg_max,

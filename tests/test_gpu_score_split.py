@@ -7,6 +7,8 @@ of a few tiles. The bar is the 1e-3 of tests/parity.py for bf16 scores; the spli
 itself only adds a rounding of each row's log2-sum-exp, so 1e-5 is asked for.
 """
 
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -22,6 +24,13 @@ def C():
     _build.build()
     from paper_2609_05821_gb300 import conduit
     return conduit
+
+
+def _ctas(units, tiles):
+    """CTAs per unit of a scoring launch, from the test build of the library."""
+    from paper_2609_05821_gb300 import _build
+    lib = ctypes.CDLL(_build.build_test_hooks())
+    return lib.conduit_test_score_ctas(units, tiles, torch.cuda.get_device_properties(0).multi_processor_count)
 
 
 @pytest.mark.parametrize("n,nq,d,extra", [(3713, 4, 128, False), (3713, 40, 128, True), (2049, 3, 64, False),
@@ -47,3 +56,38 @@ def test_split_units(C, n, nq, d, extra):
     status = torch.zeros(1, dtype=torch.int32, device="cuda")
     s, _, _ = C.conduit_score(kv, batch, q, status=status)
     assert torch.isnan(s).all() and C.conduit_read_status(status) == C.ERR_NONFINITE
+
+
+@pytest.mark.parametrize("d,kw", [(128, {}), (64, {}), (128, {"statistic": "rms"}), (128, {"value_norm": "side_cache"})])
+def test_short_requests_in_a_split_batch(C, d, kw):
+    """Requests of one key tile in a split launch: one CTA of the pair has no tiles of them, several times in a row.
+
+    Every request gets what it gets alone, up to the rounding of the split (1e-5)."""
+    L, hq, hkv = 4, 8, 4
+    n_r = [1, 128, 4000] + [1 + 17 * i % 128 for i in range(11)]   # 14 requests, 224 units: three per pair of CTAs
+    assert _ctas(L * hkv * len(n_r), 32) == 2
+    nq = [1 + 7 * r % 40 for r in range(len(n_r))]
+    cum = lambda x: [sum(x[:i]) for i in range(len(x) + 1)]
+    tok, qo = cum(n_r), cum(nq)
+    gen = torch.Generator(device="cuda").manual_seed(d)
+    draw = lambda *shape: torch.randn(shape, generator=gen, device="cuda").bfloat16()
+    k, v, q = draw(L, hkv, tok[-1], d), draw(L, hkv, tok[-1], d), draw(L, hq, qo[-1], d)
+
+    def score(kv, batch, q):
+        vn = C.conduit_value_norms(kv, batch) if kw.get("value_norm") == "side_cache" else None
+        status = torch.zeros(1, dtype=torch.int32, device="cuda")
+        out = C.conduit_score_ex(kv, batch, q, vnorm=vn, status=status, **kw)
+        assert C.conduit_read_status(status) == C.OK
+        return out
+
+    batch = C.Batch(tok, tok, list(range(len(n_r) + 1)), qo, device="cuda")
+    got = score(C.KvCache(k, v, hq), batch, q)
+    for _ in range(5):
+        assert all(torch.equal(a, b) for a, b in zip(got, score(C.KvCache(k, v, hq), batch, q)))
+    for r, n in enumerate(n_r):
+        t, qs = slice(tok[r], tok[r + 1]), slice(qo[r], qo[r + 1])
+        alone = C.Batch([0, n], [0, n], [0, 1], [0, nq[r]], device="cuda")
+        cut = lambda x, s: x[:, :, s].contiguous()
+        want = score(C.KvCache(cut(k, t), cut(v, t), hq), alone, cut(q, qs))
+        for a, b in zip((got[0][t], got[1][t], got[2][r:r + 1]), want):
+            assert torch.all((a - b).abs() <= 1e-5 * b.abs() + 1e-7 * b.abs().max()), (r, n)
