@@ -35,7 +35,8 @@ def _positions(spec, n):
     return np.unique(np.linspace(0, n - 1, spec).round().astype(np.int64)) if spec else np.zeros(0, np.int64)
 
 
-def _run(C, hq, hkv, d, n_r, specs, seed=0, form="plain", dtype=torch.bfloat16, L=2):
+def _run(C, hq, hkv, d, n_r, specs, seed=0, form="plain", dtype=torch.bfloat16, L=2, unused=0.0):
+    """`unused`: what a page's rows without a token hold."""
     if len(specs) == 2 and isinstance(specs[0], str):
         specs = (specs,)
     pos = [_positions(s, n) for s, n in zip(specs, n_r)]
@@ -54,11 +55,11 @@ def _run(C, hq, hkv, d, n_r, specs, seed=0, form="plain", dtype=torch.bfloat16, 
         pages = [-(-n // 16) for n in n_r]
         first = np.concatenate([[0], np.cumsum(pages)]).tolist()
         table = torch.full((R, max(pages)), -1, dtype=torch.int32)
-        pool = [torch.zeros(L, first[-1], hkv, 16, d, dtype=dtype, device="cuda") for _ in range(2)]
+        pool = [torch.full((L, first[-1], hkv, 16, d), unused, dtype=dtype, device="cuda") for _ in range(2)]
         for r, n in enumerate(n_r):
             table[r, :pages[r]] = torch.arange(first[r + 1] - 1, first[r] - 1, -1, dtype=torch.int32)
             for dst, src in zip(pool, (k, v)):
-                rows = torch.nn.functional.pad(src[:, :, tok[r]:tok[r + 1]], (0, 0, 0, 16 * pages[r] - n))
+                rows = torch.nn.functional.pad(src[:, :, tok[r]:tok[r + 1]], (0, 0, 0, 16 * pages[r] - n), value=unused)
                 dst[:, table[r, :pages[r]].long().cuda()] = rows.view(L, hkv, pages[r], 16, d).transpose(1, 2)
         kv = C.KvCache(*pool, hq, 16, table)
     if form in ("plain", "paged"):
@@ -156,6 +157,28 @@ def test_cuda_core_tiles(C, dtype, d):
     for specs in ((9,), (("head", 1),), (44,)):   # clusters of eight CTAs: keys for all, for one, two row tiles
         _run(C, 6, 2, d, (700,), specs, seed=d, dtype=dtype)
     test_scores_of_head_dims(C, d, dtype)
+
+
+@pytest.mark.parametrize("d,L", [(40, 2), (64, 2), (96, 2), (128, 2), (128, 64)])
+def test_rows_without_a_token_are_not_read(C, d, L):
+    """NaN and Inf in the unused rows of a request's last page, and at the head of the next request's rows.
+
+    At 128 dims 64 layers in small pages take two query tiles per item, two layers one."""
+    n_r, specs = (1481, 300), (163, ("tail", 30))
+    plain = _run(C, 14, 2, d, n_r, specs, form="paged", L=L)
+    for unused in (float("nan"), float("inf")):
+        assert torch.equal(_run(C, 14, 2, d, n_r, specs, form="paged", L=L, unused=unused), plain)
+    gen = torch.Generator(device="cuda").manual_seed(d)
+    draw = lambda *shape: torch.randn(shape, generator=gen, device="cuda").bfloat16()
+    k, v, q_rows = draw(L, 2, 700, d), draw(L, 2, 700, d), draw(L, 75, 14, d)
+    tok = [0, 300, 700]
+    batch = C.Batch(tok, tok, [0, 1, 2], [0, 1, 2], device="cuda")
+    off, off_dev = C.idx_offsets([75, 0])
+    idx = torch.arange(3, 300, 4, dtype=torch.int32, device="cuda")[:75]
+    clean = C.conduit_refresh_attn(C.KvCache(k, v, 14), batch, idx, off, off_dev, q_rows)
+    assert torch.isfinite(clean).all()
+    k[:, :, 300:], v[:, :, 300:] = float("nan"), float("inf")
+    assert torch.equal(C.conduit_refresh_attn(C.KvCache(k, v, 14), batch, idx, off, off_dev, q_rows), clean)
 
 
 def test_values_past_a_position_add_nothing(C):

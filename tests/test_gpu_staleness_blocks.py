@@ -37,3 +37,19 @@ def test_paged_equals_contiguous(d):
     paged = C.KvCache(pool(k), pool(v), hq, page, table)
     for _ in range(20):
         assert torch.equal(run(paged), want)
+
+
+@pytest.mark.parametrize("d", (128, 96, 64))
+def test_draws_of_other_requests_are_not_read(d):
+    """Non-finite draws of a request change nothing in the one before it, whose last key tile they share."""
+    from paper_2609_05821_gb300 import conduit as C
+    L, hq, hkv, tok, qo = 2, 8, 2, [0, 200, 500], [0, 9, 20]
+    gen = torch.Generator(device="cuda").manual_seed(d)
+    draw = lambda *shape: torch.randn(shape, generator=gen, device="cuda").bfloat16()
+    k, v, q, z = draw(L, hkv, 500, d), draw(L, hkv, 500, d), draw(L, hq, 20, d), draw(2, L, hkv, 500, d)
+    batch = C.Batch(tok, tok, [0, 1, 2], qo, device="cuda")
+    mask = (torch.rand(500, generator=gen, device="cuda") < 0.1).to(torch.uint8)
+    clean = C.conduit_staleness_iso(C.KvCache(k, v, hq), batch, q, mask, z, 0.5)[0]
+    z[:, :, :, 200:] = float("nan")
+    got = C.conduit_staleness_iso(C.KvCache(k, v, hq), batch, q, mask, z, 0.5)[0]
+    assert got[0] == clean[0] and torch.isnan(got[1])
