@@ -135,6 +135,7 @@ struct RefArgs {
   int32_t draws;           // n_items = draws * n_blocks * Hkv * L
   const float* key_scale;  // [L][Hkv][n_tot]
   double* part;            // [draws][L * Hkv][n_blocks][2 query tiles][4 warps]
+  const __nv_bfloat16* q;  // the query rows, laid out as `out` (not kStale)
 };
 
 // A work item: block `blk` of (layer l, KV head g), counted from the largest
@@ -889,6 +890,69 @@ __device__ __forceinline__ OneSmem carve_one(uint8_t* raw) {
   return s;
 }
 
+// Output rows with values that are not finite although the row's maximum and sum are:
+// V holds such a value, in a key of the row or in a later one that shares a key tile
+// with the item's rows, where P is 0 but 0 x Inf or NaN is NaN. A warp computes the
+// rows of `lanes` again, key by key over the keys they see: columns col0 ... of each.
+// The cost is about 100 ns a key and row (64 dims; 112 at 96), so the 32 rows of a warp
+// take half a second at kRedoKeys keys: rows that see more, which would keep the other
+// roles waiting past their limit, stay as they are.
+constexpr int kRedoKeys = 1 << 17;
+template <int kCols>
+__device__ __noinline__ void redo_rows(const RefArgs& a, uint32_t lanes, int l, int g, int r, int t0, int p_row,
+                                       float m_ref, float inv, int64_t row_off, int col0, int lane) {
+  const KvDev& kv = a.kv;
+  const __nv_bfloat16* kb = static_cast<const __nv_bfloat16*>(kv.k);
+  const __nv_bfloat16* vb = static_cast<const __nv_bfloat16*>(kv.v);
+  __syncwarp();  // the rows' first values have been written
+  for (; lanes; lanes &= lanes - 1) {
+    const int src = __ffs(lanes) - 1;
+    const int p = __shfl_sync(0xffffffffu, p_row, src);
+    const float m = __shfl_sync(0xffffffffu, m_ref, src), w0 = __shfl_sync(0xffffffffu, inv, src);
+    const int64_t off = __shfl_sync(0xffffffffu, static_cast<long long>(row_off), src);
+    if (p >= kRedoKeys) continue;
+    float acc[kCols / 32] = {};
+    for (int j0 = 0; j0 <= p; j0 += 32) {
+      const int j = j0 + lane;
+      int64_t k_off = 0;
+      float w = 0.f;
+      if (j <= p) {
+        k_off = kv.row(l, g, r, int64_t(t0) + j, j);
+        float dot = 0.f;
+#pragma unroll 4
+        for (int c = 0; c < kv.d; c += 8) {
+          const uint4 qv = *reinterpret_cast<const uint4*>(a.q + off + c);
+          const uint4 kk = *reinterpret_cast<const uint4*>(kb + k_off + c);
+          const __nv_bfloat162* q2 = reinterpret_cast<const __nv_bfloat162*>(&qv);
+          const __nv_bfloat162* k2 = reinterpret_cast<const __nv_bfloat162*>(&kk);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const float2 x = __bfloat1622float2(q2[i]), y = __bfloat1622float2(k2[i]);
+            dot = fmaf(x.y, y.y, fmaf(x.x, y.x, dot));
+          }
+        }
+        w = exp2f(fmaf(dot, a.scale_log2, -m)) * w0;
+      }
+      const int n = min(32, p - j0 + 1);
+#pragma unroll 8
+      for (int jj = 0; jj < n; ++jj) {
+        const float wj = __shfl_sync(0xffffffffu, w, jj);
+        const int64_t v_off = __shfl_sync(0xffffffffu, static_cast<long long>(k_off), jj);
+#pragma unroll
+        for (int c = 0; c < kCols / 32; ++c) {
+          const int e = col0 + 32 * c + lane;
+          if (e < kv.d) acc[c] = fmaf(wj, __bfloat162float(vb[v_off + e]), acc[c]);
+        }
+      }
+    }
+#pragma unroll
+    for (int c = 0; c < kCols / 32; ++c) {
+      const int e = col0 + 32 * c + lane;
+      if (e < kv.d) a.out[off + e] = __float2bfloat16_rn(acc[c]);
+    }
+  }
+}
+
 // Agreement of the 256 softmax threads (named barrier 1 with an AND
 // reduction): every thread arrives, so all of them take the same branch.
 __device__ __forceinline__ bool softmax_all(bool pred) {
@@ -1191,7 +1255,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       it.r = rec[3];
       it.i0 = rec[4];
       it.cnt = rec[5];
-      const int nt = rec[6], N = rec[7];
+      const int nt = rec[6], N = rec[7], rec_t0 = rec[8];
       const bool row_ok = u >= 0 && row < it.cnt * G;
       const int i_row = it.i0 + (row_ok ? row / G : 0);
       const int h_row = it.g * G + (row_ok ? row % G : 0);
@@ -1313,7 +1377,9 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (fin) {
         tc::tc_fence_after();
         const float inv = total > 0.f ? 1.f / total : 0.f;
-        __nv_bfloat16* dst = a.out + ((int64_t(it.l) * a.n_sel + i_row) * Hq + h_row) * d;
+        const int64_t row_off = ((int64_t(it.l) * a.n_sel + i_row) * Hq + h_row) * d;
+        __nv_bfloat16* dst = a.out + row_off;
+        float zero = 0.f;  // NaN where a value is not finite
         // This thread's columns of O, 32 at a time, as bf16. Each lane writes its own
         // row, so a warp's store covers 32 rows: 32-byte stores (whole sectors)
         // when the buffer allows them.
@@ -1322,6 +1388,10 @@ __global__ void __launch_bounds__(kThreads, 1)
           float o[32];
           tc::tmem_ld32(tl + kOneOCol + c, o);
           if (!live) continue;
+          if (kSplit) {
+#pragma unroll
+            for (int i = 0; i < 32; ++i) zero = fmaf(o[i], 0.f, zero);
+          }
           uint32_t w[16];
 #pragma unroll
           for (int k2 = 0; k2 < 16; ++k2) {
@@ -1342,6 +1412,12 @@ __global__ void __launch_bounds__(kThreads, 1)
               if (c + u4 * 8 < d)
                 *reinterpret_cast<uint4*>(dst + c + u4 * 8) = make_uint4(w[4 * u4], w[4 * u4 + 1], w[4 * u4 + 2], w[4 * u4 + 3]);
           }
+        }
+        if (kSplit) {
+          // (a sum that is NaN comes from Q or K, and the row is NaN as it should be)
+          const uint32_t redo = __ballot_sync(0xffffffffu, live && total > 0.f && zero != 0.f);
+          if (redo)
+            redo_rows<kOW>(a, redo, it.l, it.g, it.r, rec_t0, p_row, m_ref, inv, row_off, hh * kOW, lane);
         }
       }
       tc::tc_fence_before();
@@ -1472,6 +1548,7 @@ cudaError_t launch_refresh_tc(const KvDev& kv, const BatchDev& b, const int32_t*
   a.idx = idx;
   a.idx_off = idx_off_dev;
   a.out = static_cast<__nv_bfloat16*>(out);
+  a.q = static_cast<const __nv_bfloat16*>(q_rows);
   a.out32 = (reinterpret_cast<uintptr_t>(out) & 31) == 0 && kv.d % 16 == 0;
   a.n_sel = n_sel;
   a.rows_per_tile = kRows / kv.G;

@@ -192,3 +192,36 @@ def test_values_past_a_position_add_nothing(C):
     v[:, :, 50] = float("inf")
     got = C.conduit_refresh_attn(C.KvCache(k, v, 1), batch, idx, off, off_dev, q_rows)
     assert torch.equal(got[:, 0], clean[:, 0]) and not torch.isfinite(got[:, 1]).any()
+
+
+@pytest.mark.parametrize("form", ["contiguous", "paged"])
+@pytest.mark.parametrize("d", [8, 40, 64, 72, 96, 120])
+def test_non_finite_values_reach_the_rows_that_see_them(C, d, form):
+    """bf16 head sizes below 128: Inf and NaN in V count from their own position on, as they do in the sum itself.
+
+    The other rows keep the module's bar, also where they share a key tile with such a value."""
+    n, hq, hkv, L = 300, 6, 2, 2
+    gen = torch.Generator(device="cuda").manual_seed(d)
+    draw = lambda *shape: torch.randn(shape, generator=gen, device="cuda").bfloat16()
+    k, v, q_rows = draw(L, hkv, n, d), draw(L, hkv, n, d), draw(L, n // 2, hq, d)
+    v[0, :, 50, :d // 2] = float("inf")
+    v[0, 0, 131, 3] = -float("inf")
+    v[0, 1, 200, d - 1] = float("nan")
+    kv = C.KvCache(k, v, hq)
+    if form == "paged":
+        pool = lambda t: torch.nn.functional.pad(t, (0, 0, 0, 4)).view(L, hkv, 19, 16, d).transpose(1, 2).contiguous()
+        kv = C.KvCache(pool(k), pool(v), hq, 16, torch.arange(19, dtype=torch.int32)[None])
+    batch = C.Batch([0, n], [0, n], [0, 1], [0, 1], device="cuda")
+    off, off_dev = C.idx_offsets([n // 2])
+    idx = torch.arange(1, n, 2, dtype=torch.int32, device="cuda")
+    got = C.conduit_refresh_attn(kv, batch, idx, off, off_dev, q_rows).double()
+    for i, p in enumerate(idx.tolist()):
+        for h in range(hq):
+            kk, vv = k[:, h // 3, :p + 1].double(), v[:, h // 3, :p + 1].double()
+            w = torch.softmax((kk @ q_rows[:, i, h].double()[:, :, None])[..., 0] / d ** 0.5, -1)
+            want = (w[:, :, None] * vv).sum(1)
+            x = got[:, i, h]
+            fine = torch.isfinite(want)
+            assert torch.equal(fine, torch.isfinite(x)) and torch.equal(torch.isnan(want), torch.isnan(x)), (p, h)
+            assert torch.equal(want[torch.isinf(want)], x[torch.isinf(want)]), (p, h)
+            assert torch.all((x - want).abs()[fine] <= 2e-2 + 2.0 ** -8 * want.abs()[fine]), (p, h)
