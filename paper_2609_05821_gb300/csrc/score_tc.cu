@@ -345,8 +345,8 @@ __device__ __forceinline__ void row_stats(float (&v)[NC], int valid, float scale
 
 // Sum over NC accumulator columns (scoring rows c0 ...) of 2^(S scale - lse_row),
 // given nlse = -lse. Columns past the row group carry nlse = -inf and add
-// exactly zero (the accumulator columns there hold finite values: TMEM is
-// zeroed at start).
+// exactly zero (the query rows there are zero, so they hold 0 for any token
+// whose key is finite).
 template <int NC>
 __device__ __forceinline__ float col_sum(const float (&v)[NC], const float* nlse, float scale) {
   const float2 sc2 = make_float2(scale, scale);
@@ -489,7 +489,10 @@ __global__ void __launch_bounds__(kThreads, 1)
       ++useq;
       tc::tc_fence_after();
       const int nrb = (w.rows + 127) / 128;
-      const int ncols = (w.rows + 15) & ~15;
+      // Pass B reads whole 32-column chunks, so its MMA writes them all: columns left
+      // from an earlier tile may hold a NaN of keys or of a request that are none of
+      // this unit's.
+      const int ncols = (w.rows + 31) & ~31;
       for (int i = 0; i < 2 * w.tiles; ++i) {
         const int st = kseq % kStages;
         if (!wait_or_abort(&s.kfull[st], (kseq / kStages) & 1, s.abort)) {
@@ -548,13 +551,6 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int64_t n_tot = a.kv.n_tot;
     uint32_t tseq = 0, vcons = 0, useq = 0;
     bool ok = true;
-    {  // zero this warp's TMEM lanes once, so unwritten accumulator columns hold finite values
-      uint32_t zero[64];
-#pragma unroll
-      for (int i = 0; i < 64; ++i) zero[i] = 0u;
-      for (int c = h * 256; c < h * 256 + 256; c += 64) tc::tmem_st64(tmem + lane_base + c, zero);
-      tc::tc_fence_before();
-    }
     for (int u = unit0; u < a.n_units; u += unit_step) {
       Unit w;
       if (!decode_unit(a, u, w, rank, ctas)) continue;

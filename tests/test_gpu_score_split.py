@@ -91,3 +91,32 @@ def test_short_requests_in_a_split_batch(C, d, kw):
         want = score(C.KvCache(cut(k, t), cut(v, t), hq), alone, cut(q, qs))
         for a, b in zip((got[0][t], got[1][t], got[2][r:r + 1]), want):
             assert torch.all((a - b).abs() <= 1e-5 * b.abs() + 1e-7 * b.abs().max()), (r, n)
+
+
+@pytest.mark.parametrize("form", ["contiguous", "paged"])
+@pytest.mark.parametrize("d,nq", [(128, 10), (64, 10), (40, 3), (96, 36), (128, 72)])
+def test_keys_of_no_token_reach_no_score(C, d, nq, form):
+    """NaN in the next request's keys and values, or in a page's unused rows, leaves a request's scores as they are.
+
+    40, 12, 144 and 288 scoring rows: the last 32-column chunk of a row group is partly filled."""
+    L, hq, hkv, tok = 2, 8, 2, [0, 168, 460]
+    gen = torch.Generator(device="cuda").manual_seed(d)
+    draw = lambda *shape: torch.randn(shape, generator=gen, device="cuda").bfloat16()
+    k, v, q = draw(L, hkv, 460, d), draw(L, hkv, 460, d), draw(L, hq, nq + 5, d)
+    batch = C.Batch(tok, tok, [0, 1, 2], [0, nq, nq + 5], device="cuda")
+    if form == "paged":   # request 0: pages 0 .. 10, the last with 8 unused rows; request 1: pages 11 .. 29
+        table = torch.full((2, 19), -1, dtype=torch.int32)
+        table[0, :11], table[1, :19] = torch.arange(11), torch.arange(11, 30)
+        def cache(x, unused):
+            pool = torch.full((L, hkv, 480, d), unused, dtype=x.dtype, device="cuda")
+            pool[:, :, :168], pool[:, :, 176:468] = x[:, :, :168], x[:, :, 168:]
+            return pool.view(L, hkv, 30, 16, d).transpose(1, 2).contiguous()
+        score = lambda unused: C.conduit_score(C.KvCache(cache(k, unused), cache(v, unused), hq, 16, table), batch, q)
+        clean, got, end = score(0.0), score(float("nan")), 460
+    else:
+        clean = C.conduit_score(C.KvCache(k, v, hq), batch, q)
+        k[:, :, 168:], v[:, :, 168:] = float("nan"), float("nan")
+        got, end = C.conduit_score(C.KvCache(k, v, hq), batch, q), 168
+    assert torch.isfinite(clean[0]).all()
+    for a, b, n in zip(got, clean, (end, end, 2 if form == "paged" else 1)):
+        assert torch.equal(a[:n], b[:n])
