@@ -204,7 +204,7 @@ ScoreLayout score_layout(const conduit_kv* kv, const conduit_batch* b, int n_lay
       rows += kv->num_q_heads / kv->num_kv_heads * (b->q_off[r + 1] - b->q_off[r]);
     }
     s.chunks = score_simt_chunks(make_kv(kv, b), n_layers, rows, max_tok);
-    off += align_up(size_t(total_rows) * s.chunks * sizeof(float2));
+    off += align_up(score_simt_stats(total_rows, max_tok) * sizeof(float2));
   }
   const size_t pa_bytes =
       align_up(size_t(n_layers) * kv->num_kv_heads * s.rg_max * s.parts * n_tot * sizeof(float));

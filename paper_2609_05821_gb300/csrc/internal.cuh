@@ -132,7 +132,10 @@ void count_launches(int n);
 // log-sum-exp of each scoring row over keys outside the visual span) and ss (value
 // sums of squares) may be NULL. stats holds (max, sum) of every scoring row for up
 // to `chunks` = score_simt_chunks(...) chunks of keys.
+// `rows` counts one layer and KV head there, all of them in score_simt_stats, the
+// entries a workspace holds for `stats`.
 int score_simt_chunks(const KvDev& kv, int n_layers, int rows, int max_tokens);
+size_t score_simt_stats(int64_t rows, int max_tokens);
 cudaError_t launch_score_simt(const KvDev& kv, const BatchDev& b, const void* q, int32_t q_tot,
                               const LayerList& layers, int max_rows, int max_tokens, int chunks, float2* stats,
                               float* pa, float* pa2, const float* extra_lse, float* ss, cudaStream_t stream);

@@ -206,10 +206,21 @@ __global__ void __launch_bounds__(kThreads) colsum_kernel(KvDev kv, BatchDev b, 
 
 // Chunks of keys pass 1 takes: enough that its blocks (32 rows of a slab by one
 // chunk) fill the GPU about twice over, whole key tiles each.
+constexpr int kFillBlocks = 320;
+static int key_tiles(int max_tokens) { return std::max(1, (max_tokens + kKeyTile - 1) / kKeyTile); }
+
 int score_simt_chunks(const KvDev& kv, int n_layers, int rows, int max_tokens) {
   const int64_t blocks = std::max<int64_t>(1, int64_t(n_layers) * kv.Hkv * ((rows + kRowTile - 1) / kRowTile));
-  const int tiles = std::max(1, (max_tokens + kKeyTile - 1) / kKeyTile);
-  return int(std::min<int64_t>(tiles, (320 + blocks - 1) / blocks));
+  return int(std::min<int64_t>(key_tiles(max_tokens), (kFillBlocks + blocks - 1) / blocks));
+}
+
+// Entries that hold every row's chunks. A larger call has fewer chunks, so rows x
+// chunks falls as often as it rises; a workspace must serve every call smaller than
+// the one it was sized for, so this takes what bounds it and never falls. Rows x
+// tiles is one bound. The other: with at least rows / 32 blocks, rows x ceil(320 /
+// blocks) is at most rows + 32 x 320.
+size_t score_simt_stats(int64_t rows, int max_tokens) {
+  return size_t(std::min(rows * key_tiles(max_tokens), rows + int64_t(kRowTile) * kFillBlocks));
 }
 
 cudaError_t launch_score_simt(const KvDev& kv, const BatchDev& b, const void* q, int32_t q_tot,

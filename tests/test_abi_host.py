@@ -363,3 +363,31 @@ def test_status_bits_are_the_header_values(C):
 def test_product_library_has_no_test_hooks(C):
     lib = ctypes.CDLL(C.LIB_PATH)
     assert not hasattr(lib, "conduit_test_withhold_v_tile")
+
+
+@pytest.mark.parametrize("dtype,d", [(torch.float32, 64), (torch.float32, 8), (torch.bfloat16, 256),
+                                     (torch.bfloat16, 128), (torch.bfloat16, 64)])
+def test_workspace_for_the_largest_call_serves_the_smaller_ones(C, dtype, d):
+    """The size queries never fall as queries, layers, tokens or requests are added."""
+    L, hkv, n = 8, 2, 2048
+    k = torch.zeros(L, hkv, 16, d, dtype=dtype)   # the queries read no cache row
+
+    def sizes(tokens, queries, layers, hq=8):
+        cum = lambda x: [sum(x[:i]) for i in range(len(x) + 1)]
+        tok, qo = cum(tokens), cum(queries)
+        batch = C.Batch(tok, tok, list(range(len(tokens) + 1)), qo, device="cpu")
+        kv = C.KvCache(k, k, hq)
+        return [C.conduit_score_workspace_size(kv, batch, layers),
+                C.conduit_score_ex_workspace_size(kv, batch, layers, C.score_opts(statistic="rms")),
+                C.conduit_score_with_norms_workspace_size(kv, batch, layers),
+                C.conduit_score_select_topk_workspace_size(kv, batch, layers)]
+
+    def grows(calls):
+        for small, large in zip(calls, calls[1:]):
+            assert all(a <= b for a, b in zip(sizes(*small), sizes(*large))), (small, large)
+
+    grows([([n], [q], 2) for q in range(1, 700)])
+    grows([([512], [64], layers) for layers in range(1, 9)])
+    grows([([m], [48], 2) for m in (1, 64, 65, 127, 128, 1000, 2048, 4096)])
+    grows([([512] * r, [28] * r, 8) for r in range(1, 12)])
+    grows([([m], [q], layers) for m, q, layers in ((100, 1, 1), (100, 36, 1), (512, 36, 4), (512, 312, 5), (900, 313, 8))])
