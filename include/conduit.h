@@ -443,10 +443,13 @@ conduit_status conduit_refresh_attn(const conduit_kv* kv, const conduit_batch* b
  *  M >= 1, kappa >= 0
  *  err        device double [R] E_r (written)
  *  err_layers device double [R][L] the per-layer terms of E_r, or NULL
- *  workspace  conduit_staleness_iso_workspace_size bytes (it holds one draw of
- *             xi in the cache's layout and the per-draw attention outputs)
- * Attention runs with the refresh kernels (bf16 P and outputs for bf16
- * caches); the reduction of ||O||^2 is in a fixed order.
+ *  workspace  conduit_staleness_iso_workspace_size bytes. bf16 caches with
+ *             head_dim 128: the keys' standard deviations and the partial sums
+ *             of every draw; others: one draw of xi in the cache's layout, the
+ *             queries and outputs of one draw's attention.
+ * Attention runs with the refresh kernels (for bf16 caches with bf16 xi and
+ * output rows, and bf16 P at head_dim 128); the reduction of ||O||^2 is in a
+ * fixed order.
  */
 conduit_status conduit_staleness_iso_workspace_size(const conduit_kv* kv, const conduit_batch* batch,
                                                    int32_t M, size_t* bytes);

@@ -185,6 +185,7 @@ struct StaleLayout {
 StaleLayout stale_layout(const KvDev& kv, const BatchDev& b, const int32_t* q_off_host, int M);
 // Work items per (layer, KV head, draw) and the launch of `draws` draws starting
 // at z: part gets [draws][L * Hkv][blocks][8] sums of ||O / rowsum||^2.
+bool stale_tc_supported(const KvDev& kv);
 int stale_tc_blocks(const KvDev& kv, const BatchDev& b, const int32_t* q_off_host);
 cudaError_t launch_stale_tc(const KvDev& kv, const BatchDev& b, const int32_t* q_off_host, int32_t q_tot,
                             const void* q, const void* z, int draws, const float* key_scale, double* part,

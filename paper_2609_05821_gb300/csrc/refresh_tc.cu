@@ -92,21 +92,15 @@ constexpr int kRecReaders = 11;                  // two MMA warps, V warp, eight
 constexpr uint32_t kBarBytes = 384;             // barriers, TMEM slot, abort flag, counters
 constexpr uint32_t kTailBytes = kBarBytes + 2 * (16 + 2 * kRows) * 4;
 
-// Head sizes: kHalves 64-dim halves of a row (one 128-byte swizzled row each;
-// a smaller head_dim is padded with zeros by the copies).
-template <int kHalves>
-struct Shape {
-  static constexpr uint32_t kTileBytes = kHalves * kHalfBytes;
-  // K and V tiles in one ring, K(0) V(0) K(1) V(1) ...: tile T may be loaded
-  // once tile T - kAhead is done (by both streams), and fewer than kDone tiles
-  // are undecided
-  static constexpr int kStages = kHalves == 1 ? 9 : 5;
-  static constexpr int kAhead = (kStages - 1) / 2;
-  static constexpr int kDone = 2 * kAhead;
-  static constexpr uint32_t kSmem = (2 + kStages) * kTileBytes + kTailBytes;
-  static_assert(kSmem <= 232448, "shared memory of one CTA");
-  static_assert((kStages + 2 * kDone + 6 + 4 + 4 + 2 + 1) * 8 + 32 <= kBarBytes, "barriers and counters");
-};
+constexpr uint32_t kTileBytes = 2 * kHalfBytes;  // a query, K or V tile of 128 dims
+// K and V tiles in one ring, K(0) V(0) K(1) V(1) ...: tile T may be loaded once tile
+// T - kAhead is done (by both streams), and fewer than kDone tiles are undecided.
+constexpr int kStages = 5;
+constexpr int kAhead = (kStages - 1) / 2;
+constexpr int kDone = 2 * kAhead;
+constexpr uint32_t kSmem = (2 + kStages) * kTileBytes + kTailBytes;
+static_assert(kSmem <= 232448, "shared memory of one CTA");
+static_assert((kStages + 2 * kDone + 6 + 4 + 4 + 2 + 1) * 8 + 32 <= kBarBytes, "barriers and counters");
 constexpr uint32_t kTmemCols = 512;
 constexpr uint32_t kSCols = 128;                 // one S buffer
 constexpr uint32_t kPCol = 64;                   // P (bf16 pairs) over the upper half of S ...
@@ -209,16 +203,14 @@ struct Smem {
   uint64_t* raw;       // [1] the copy of a V tile that ends past its request's keys
 };
 
-template <int kHalves>
 __device__ __forceinline__ Smem carve(uint8_t* base) {
-  using C = Shape<kHalves>;
   Smem s;
   s.q = base;
-  s.kv = s.q + 2 * C::kTileBytes;
-  uint64_t* bar = reinterpret_cast<uint64_t*>(s.kv + C::kStages * C::kTileBytes);
+  s.kv = s.q + 2 * kTileBytes;
+  uint64_t* bar = reinterpret_cast<uint64_t*>(s.kv + kStages * kTileBytes);
   s.full = bar;
-  s.done = s.full + C::kStages;
-  s.sfull = s.done + C::kDone;
+  s.done = s.full + kStages;
+  s.sfull = s.done + kDone;
   s.pfull = s.sfull + 2;
   s.ofull = s.pfull + 2;
   s.qfull = s.ofull + 2;
@@ -227,7 +219,7 @@ __device__ __forceinline__ Smem carve(uint8_t* base) {
   s.recempty = s.recfull + 2;
   s.mdone = s.recempty + 2;
   s.scaled = s.mdone + 2;
-  s.tmem_slot = reinterpret_cast<uint32_t*>(s.scaled + C::kDone);
+  s.tmem_slot = reinterpret_cast<uint32_t*>(s.scaled + kDone);
   s.abort = reinterpret_cast<volatile int*>(s.tmem_slot + 1);
   s.counters = reinterpret_cast<uint32_t*>(s.tmem_slot + 2);
   s.raw = reinterpret_cast<uint64_t*>(s.counters + 2);
@@ -301,21 +293,15 @@ __device__ __forceinline__ void clear_rows(uint8_t* tile, int first, int end, in
   __syncwarp();
 }
 
-// kSplit: P goes to the tensor cores as two bf16 tiles (value and rounding
-// error), which keeps it as precise as fp32 weights for a bf16 result.
-template <int kHalves, bool kSplit, bool kStale = false>
+template <bool kStale>
 __global__ void __launch_bounds__(kThreads, 1)
     refresh_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant__ CUtensorMap vmap,
                       const __grid_constant__ CUtensorMap qmap, const __grid_constant__ RefArgs a) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
-  using C = Shape<kHalves>;
-  constexpr int kStages = C::kStages, kAhead = C::kAhead, kDone = C::kDone, kDP = 64 * kHalves;
-  constexpr uint32_t kTileBytes = C::kTileBytes;
-  const Smem s = carve<kHalves>(smem_raw);
+  const Smem s = carve(smem_raw);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const KvDev& kv = a.kv;
   const int G = kv.G, Hq = kv.Hq;
-  const int d = kHalves == 2 && !kSplit ? kMaxD : kv.d;
   const int span = a.rows_per_tile;               // selected rows of a query tile
   if (tc::smem_u32(smem_raw) & 1023u) {           // the swizzled tiles need 1024-byte atoms
     if (tid == 0) flag_status(a.status, CONDUIT_FLAG_TIMEOUT | tc::kSiteLoad);
@@ -347,7 +333,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (warp == kMmaWarp) tc::tmem_alloc(s.tmem_slot, kTmemCols);
   // query rows the boxes never fill: zero, so their logits are finite
   for (uint32_t i = span * G * 128 + tid * 16; i < kHalfBytes; i += kThreads * 16)
-    for (int h = 0; h < 2 * kHalves; ++h) *reinterpret_cast<uint4*>(s.q + h * kHalfBytes + i) = make_uint4(0, 0, 0, 0);
+    for (int h = 0; h < 4; ++h) *reinterpret_cast<uint4*>(s.q + h * kHalfBytes + i) = make_uint4(0, 0, 0, 0);
   tc::fence_proxy_async_smem();
   __syncthreads();
   tc::tc_fence_after();
@@ -422,7 +408,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           ok = false;
           break;
         }
-        load_tile<kHalves>(a, &kmap, s.kv + sl * kTileBytes, &s.full[sl], it.l, it.g, it.r, t0, N, t * kKT, lane);
+        load_tile<2>(a, &kmap, s.kv + sl * kTileBytes, &s.full[sl], it.l, it.g, it.r, t0, N, t * kKT, lane);
       }
     }
     if (lane == 0) s.counters[0] = T;
@@ -453,13 +439,13 @@ __global__ void __launch_bounds__(kThreads, 1)
           const int64_t z_row = int64_t(m) * kv.L * kv.Hkv * kv.n_tot + row + t * kKT;
           if (lane == 0) tc::mbar_arrive_expect_tx(&s.full[sl], kTileBytes);
           __syncwarp();
-          if (lane < kHalves)
+          if (lane < 2)
             tc::tma_load_2d(s.kv + sl * kTileBytes + lane * kHalfBytes, &vmap, &s.full[sl], lane * 64, int32_t(z_row));
         } else if ((t + 1) * kKT <= N) {
-          load_tile<kHalves>(a, &vmap, s.kv + sl * kTileBytes, &s.full[sl], l, g, r, t0, N, t * kKT, lane);
+          load_tile<2>(a, &vmap, s.kv + sl * kTileBytes, &s.full[sl], l, g, r, t0, N, t * kKT, lane);
         } else {  // the copy arrives on a barrier of its own, and the tile is full once it has been cleared
           uint8_t* tile = s.kv + sl * kTileBytes;
-          load_tile<kHalves>(a, &vmap, tile, s.raw, l, g, r, t0, N, t * kKT, lane);
+          load_tile<2>(a, &vmap, tile, s.raw, l, g, r, t0, N, t * kKT, lane);
           if (!wait_warp(s.raw, n_raw & 1, s.abort)) {
             if (lane == 0) raise_abort(a, s.abort, tc::kSiteLoad);
             tc::mbar_wait(s.raw, n_raw & 1);  // the copy in flight
@@ -467,7 +453,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             break;
           }
           ++n_raw;
-          clear_rows<kHalves>(tile, N - t * kKT, kKT, lane);
+          clear_rows<2>(tile, N - t * kKT, kKT, lane);
           if (lane == 0) tc::mbar_arrive(&s.full[sl]);
         }
       }
@@ -480,18 +466,18 @@ __global__ void __launch_bounds__(kThreads, 1)
     const uint32_t leader = lane == 0, frees = x == 0 ? leader : 0u;
     uint32_t T = 0, turn = 0, np = 0, nq = 0, cq = 0;  // tiles, turns, P tiles, query tiles loaded / consumed
     const uint32_t idesc_s = tc::idesc_bf16(kRows, kKT);
-    const uint32_t idesc_o = tc::idesc_bf16(kRows, kDP, /*b_mn_major=*/true);
+    const uint32_t idesc_o = tc::idesc_bf16(kRows, kMaxD, /*b_mn_major=*/true);
     const uint32_t kv_addr = tc::smem_u32(s.kv);
     const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
-    const uint32_t s_col = tm + x * kSCols, o_col = tm + kOCol + x * kDP;
+    const uint32_t s_col = tm + x * kSCols, o_col = tm + kOCol + x * kMaxD;
     const uint64_t dq = tc::desc_sw128(tc::smem_u32(s.q) + x * kTileBytes);
     bool ok = true;
     auto load_q = [&](const volatile int* rec) {
       if (rec[0] < 0 || rec[7 + x] == 0) return;
       if (lane == 0) {
         uint8_t* dst = s.q + x * kTileBytes;
-        tc::mbar_arrive_expect_tx(&s.qfull[x], uint32_t(kHalves) * 128u * uint32_t(span * G));
-        for (int hf = 0; hf < kHalves; ++hf)
+        tc::mbar_arrive_expect_tx(&s.qfull[x], 256u * uint32_t(span * G));
+        for (int hf = 0; hf < 2; ++hf)
           if (kStale)
             tc::tma_load_3d(dst + hf * kHalfBytes, &qmap, &s.qfull[x], hf * 64, rec[4] + (x ? rec[5] : 0),
                             rec[1] * Hq + rec[2] * G);
@@ -539,20 +525,14 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
           for (int kk = 0; kk < kKT / 16; ++kk)  // O += P(t) V(t)
             tc::mma_bf16_ts_if(leader, o_col, s_col + kPCol + kk * 8, dv + kk * (2048 >> 4), idesc_o, t > 0 || kk > 0);
-          if (kSplit) {
-#pragma unroll
-            for (int kk = 0; kk < kKT / 16; ++kk)
-              tc::mma_bf16_ts_if(leader, o_col, s_col + kPLoCol + kk * 8, dv + kk * (2048 >> 4), idesc_o, true);
-          }
           if (t + 1 == nt_x) tc::mma_commit_if(leader, &s.ofull[x]);
         }
         if (t + 1 < nt_x) {
-          const int ksteps = kSplit ? (d + 15) / 16 : kDP / 16;
 #pragma unroll
-          for (int kk = 0; kk < kDP / 16; ++kk) {  // S(t + 1) = Q K(t + 1)^T
+          for (int kk = 0; kk < kMaxD / 16; ++kk) {  // S(t + 1) = Q K(t + 1)^T
             const uint32_t off = ((kk >> 2) * kHalfBytes + (kk & 3) * 32) >> 4;
-            if (kk == kDP / 16 - kPassEarly) tc::mbar_arrive_if(leader, &s.turn[x ^ 1]);
-            if (kk < ksteps) tc::mma_bf16_if(leader, s_col, dq + off, dk + off, idesc_s, kk > 0);
+            if (kk == kMaxD / 16 - kPassEarly) tc::mbar_arrive_if(leader, &s.turn[x ^ 1]);
+            tc::mma_bf16_if(leader, s_col, dq + off, dk + off, idesc_s, kk > 0);
           }
           tc::mma_commit_if(leader, &s.sfull[x]);
         } else {
@@ -580,7 +560,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int quarter = warp & 3;
     const int row = quarter * 32 + lane;                 // TMEM lane = query row of the tile
     const uint32_t tl = tmem + (uint32_t(quarter * 32) << 16);
-    const uint32_t sb = tl + x * kSCols, ob = tl + kOCol + x * kDP;
+    const uint32_t sb = tl + x * kSCols, ob = tl + kOCol + x * kMaxD;
     const uint32_t leader = lane == 0, releases = x == 1 && quarter == 0 && lane == 0;
     uint32_t Tv = 0;                                     // (kStale) the CTA's V tiles
     // (kStale) this query tile's share of scaling V tile t of the item: thread j
@@ -604,8 +584,8 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
       uint8_t* tile = s.kv + sl * kTileBytes;
 #pragma unroll
-      for (int i8 = 0; i8 < 4 * kHalves; ++i8) {
-        const int c = 4 * kHalves * x + i8;
+      for (int i8 = 0; i8 < 8; ++i8) {
+        const int c = 8 * x + i8;
         uint4* p = reinterpret_cast<uint4*>(tile + (c >> 3) * kHalfBytes + tc::sw128_offset(row, c & 7));
         uint4 v = *p;
         __nv_bfloat162* h = reinterpret_cast<__nv_bfloat162*>(&v);
@@ -618,7 +598,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
       if (j >= N) {  // another request's draws, and 0 x Inf or NaN is not 0
 #pragma unroll 1
-        for (int c = 4 * kHalves * x; c < 4 * kHalves * (x + 1); ++c)
+        for (int c = 8 * x; c < 8 * (x + 1); ++c)
           *reinterpret_cast<uint4*>(tile + (c >> 3) * kHalfBytes + tc::sw128_offset(row, c & 7)) = make_uint4(0, 0, 0, 0);
       }
       tc::fence_proxy_async_smem();
@@ -696,7 +676,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (__any_sync(0xffffffffu, need) && t > 0) {
           // S(t) is ready, so P(t-1) V(t-1) has completed; P(t) V(t) waits for
           // this warp's arrival below
-          for (int c = 0; c < kDP; c += 16) {
+          for (int c = 0; c < kMaxD; c += 16) {
             float o[16];
             tc::tmem_ld16(ob + c, o);
             uint32_t w[16];
@@ -708,29 +688,22 @@ __global__ void __launch_bounds__(kThreads, 1)
         // P = 2^(S scale - m) in bf16 pairs over S, which this warp has read (one
         // packed FMA per pair for scale and bias, packed adds for the sum). A row
         // with no visible key yet (m = -inf) uses bias 0: its logits are all
-        // -inf and its P is 0. With kSplit a second tile holds the rounding
-        // error of the first, so that P keeps 16 bits of mantissa.
+        // -inf and its P is 0.
         const float2 sc2 = make_float2(a.scale_log2, a.scale_log2);
         const float2 nb2 = m_ref == -INFINITY ? make_float2(0.f, 0.f) : make_float2(-m_ref, -m_ref);
         float2 ls2[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
 #pragma unroll
         for (int c = 0; c < kKT / 32; ++c) {
-          uint32_t pw[16], lo[16];
+          uint32_t pw[16];
 #pragma unroll
           for (int i = 0; i < 16; ++i) {
             const float2 y = tc::ffma2(make_float2(sv[32 * c + 2 * i], sv[32 * c + 2 * i + 1]), sc2, nb2);
             const float2 pp = make_float2(tc::ex2(y.x), tc::ex2(y.y));
             ls2[i & 1] = tc::fadd2(ls2[i & 1], pp);
-            __nv_bfloat162 pr = __floats2bfloat162_rn(pp.x, pp.y);
-            pw[i] = *reinterpret_cast<uint32_t*>(&pr);
-            if (kSplit) {
-              const float2 hi = __bfloat1622float2(pr);
-              pr = __floats2bfloat162_rn(pp.x - hi.x, pp.y - hi.y);
-              lo[i] = *reinterpret_cast<uint32_t*>(&pr);
-            }
+            const __nv_bfloat162 pr = __floats2bfloat162_rn(pp.x, pp.y);
+            pw[i] = *reinterpret_cast<const uint32_t*>(&pr);
           }
           tc::tmem_st16_nowait(sb + kPCol + 16 * c, pw);
-          if (kSplit) tc::tmem_st16_nowait(sb + kPLoCol + 16 * c, lo);
         }
         lsum += (ls2[0].x + ls2[0].y) + (ls2[1].x + ls2[1].y);
         tc::tmem_wait_st();
@@ -764,7 +737,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (kStale) {  // ||O / rowsum||^2 (in the cache's type) over the warp's rows, in a fixed order
         float ss[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-        for (int c = 0; c < kDP; c += 64) {
+        for (int c = 0; c < kMaxD; c += 64) {
           float o[64];
           tc::tmem_ld64(ob + c, o);
 #pragma unroll
@@ -780,9 +753,9 @@ __global__ void __launch_bounds__(kThreads, 1)
         tc::tc_fence_before();
         continue;
       }
-      __nv_bfloat16* dst = a.out + ((int64_t(l) * a.n_sel + i_row) * Hq + h_row) * d;
+      __nv_bfloat16* dst = a.out + ((int64_t(l) * a.n_sel + i_row) * Hq + h_row) * kMaxD;
 #pragma unroll
-      for (int c = 0; c < kDP; c += 64) {
+      for (int c = 0; c < kMaxD; c += 64) {
         float o[64];
         tc::tmem_ld64(ob + c, o);
         if (live) {
@@ -795,16 +768,14 @@ __global__ void __launch_bounds__(kThreads, 1)
           if (a.out32) {
 #pragma unroll
             for (int u8 = 0; u8 < 4; ++u8)
-              if (c + u8 * 16 < d)
-                asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst + c + u8 * 16),
-                             "r"(w[8 * u8]), "r"(w[8 * u8 + 1]), "r"(w[8 * u8 + 2]), "r"(w[8 * u8 + 3]),
-                             "r"(w[8 * u8 + 4]), "r"(w[8 * u8 + 5]), "r"(w[8 * u8 + 6]), "r"(w[8 * u8 + 7])
-                             : "memory");
+              asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst + c + u8 * 16),
+                           "r"(w[8 * u8]), "r"(w[8 * u8 + 1]), "r"(w[8 * u8 + 2]), "r"(w[8 * u8 + 3]),
+                           "r"(w[8 * u8 + 4]), "r"(w[8 * u8 + 5]), "r"(w[8 * u8 + 6]), "r"(w[8 * u8 + 7])
+                           : "memory");
           } else {
 #pragma unroll
             for (int u4 = 0; u4 < 8; ++u4)
-              if (c + u4 * 8 < d)
-                *reinterpret_cast<uint4*>(dst + c + u4 * 8) = make_uint4(w[4 * u4], w[4 * u4 + 1], w[4 * u4 + 2], w[4 * u4 + 3]);
+              *reinterpret_cast<uint4*>(dst + c + u4 * 8) = make_uint4(w[4 * u4], w[4 * u4 + 1], w[4 * u4 + 2], w[4 * u4 + 3]);
           }
         }
       }
@@ -965,6 +936,10 @@ __device__ __forceinline__ bool softmax_all(bool pred) {
   return out != 0;
 }
 
+// kHalves 64-dim halves of a row (one 128-byte swizzled row each; a smaller head_dim is
+// padded with zeros by the copies). kSplit: P goes to the tensor cores as two bf16
+// tiles (value and rounding error), which keeps it as precise as fp32 weights for a
+// bf16 result.
 template <int kHalves, bool kSplit>
 __global__ void __launch_bounds__(kThreads, 1)
     one_refresh_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant__ CUtensorMap vmap,
@@ -1586,7 +1561,7 @@ cudaError_t launch_refresh_tc(const KvDev& kv, const BatchDev& b, const int32_t*
   // head_dim 128 keeps its bf16 P; the smaller sizes ran with fp32 weights on
   // CUDA cores before and keep that precision by a split P
   if (!one)
-    err = launch(refresh_tc_kernel<2, false>, Shape<2>::kSmem);
+    err = launch(refresh_tc_kernel<false>, kSmem);
   else if (kv.d == kMaxD)
     err = launch(one_refresh_tc_kernel<2, false>, kOneSmem);
   else if (kv.d > 64)
@@ -1597,6 +1572,14 @@ cudaError_t launch_refresh_tc(const KvDev& kv, const BatchDev& b, const int32_t*
   count_launches(1);
   return cudaSuccess;
 }
+
+// At 128 dims, where the estimator has always run on tensor cores. They truncate each
+// of their sums, which a bf16 output row does not show and a sum of squared rows does;
+// with the split P of the smaller head sizes, twice as many sums, it came out low by
+// 3e-5 at 8 192 keys and 7e-5 at 16 384 (64 dims), more than the whole error of the
+// CUDA-core kernels (0.6e-5 and 1.7e-5 at 16 384). These take 15.7 ms for 0.7 (28
+// layers, 28/4 heads of 64 dims, 4 096 keys, five draws).
+bool stale_tc_supported(const KvDev& kv) { return kv.d == kMaxD && refresh_tc_supported(kv); }
 
 int stale_tc_blocks(const KvDev& kv, const BatchDev& b, const int32_t* q_off_host) {
   return query_blocks(b, q_off_host, 2 * (kRows / kv.G));
@@ -1646,12 +1629,7 @@ cudaError_t launch_stale_tc(const KvDev& kv, const BatchDev& b, const int32_t* q
     f<<<std::min(a.n_items, sms), kThreads, smem, stream>>>(kmap, zmap, qmap, a);
     return cudaGetLastError();
   };
-  if (kv.d == kMaxD)
-    err = launch(refresh_tc_kernel<2, false, true>, Shape<2>::kSmem);
-  else if (kv.d > 64)
-    err = launch(refresh_tc_kernel<2, true, true>, Shape<2>::kSmem);
-  else
-    err = launch(refresh_tc_kernel<1, true, true>, Shape<1>::kSmem);
+  err = launch(refresh_tc_kernel<true>, kSmem);
   if (err) return err;
   count_launches(1);
   return cudaSuccess;

@@ -5,7 +5,7 @@
 // sum_t alpha_{q,t} xi_t is the attention output of query row q over all the
 // request's visual keys with the values xi (zero for t in T), so each draw m
 // runs the refresh attention kernels with every scoring row at position
-// N_r - 1 over (K, xi^(m)). bf16 caches with head_dim up to 128 run all draws
+// N_r - 1 over (K, xi^(m)). bf16 caches with head_dim 128 run all draws
 // in one tensor-core launch (refresh_tc.cu) that reads the draws z and the
 // scoring queries as they are; for the other caches the kernels here build
 // xi^(m) in the cache's own layout, lay the scoring queries out as refresh rows,
@@ -204,7 +204,7 @@ StaleLayout stale_layout(const KvDev& kv, const BatchDev& b, const int32_t* q_of
                              : size_t(kv.L) * kv.num_pages * kv.Hkv * size_t(kv.page_size) * kv.d;
   s.xi_bytes = v_elems * esz;
   size_t off = 0;
-  s.tc = refresh_tc_supported(kv);
+  s.tc = stale_tc_supported(kv);
   if (s.tc) {  // the key scales, one partial per warp of every work item, the (request, layer) sums, the work counter
     s.n_blocks = stale_tc_blocks(kv, b, q_off_host);
     s.scale = off;

@@ -53,3 +53,24 @@ def test_draws_of_other_requests_are_not_read(d):
     z[:, :, :, 200:] = float("nan")
     got = C.conduit_staleness_iso(C.KvCache(k, v, hq), batch, q, mask, z, 0.5)[0]
     assert got[0] == clean[0] and torch.isnan(got[1])
+
+
+@pytest.mark.parametrize("d", (64, 96))
+def test_long_sums_have_no_bias(d):
+    """16 384 keys at head sizes below 128, against 64 bits from the same bf16 deviations, outputs rounded to bf16.
+
+    What remains are fp32 sums rounded to nearest, without a common sign, and the few outputs that round the other
+    way for them: below 1e-6 of the sum over 512 rows. Sums that truncate come out 7e-5 lower (64 dims)."""
+    from paper_2609_05821_gb300 import conduit as C
+    n, hq, nq, M, kappa = 16384, 8, 32, 2, 0.5
+    gen = torch.Generator(device="cuda").manual_seed(d)
+    draw = lambda *shape: torch.randn(shape, generator=gen, device="cuda").bfloat16()
+    k, v, q, z = draw(1, 1, n, d), draw(1, 1, n, d), draw(1, hq, nq, d), draw(M, 1, 1, n, d)
+    batch = C.Batch([0, n], [0, n], [0, 1], [0, nq], device="cuda")
+    mask = (torch.rand(n, generator=gen, device="cuda") < 0.1).to(torch.uint8)
+    got = float(C.conduit_staleness_iso(C.KvCache(k, v, hq), batch, q, mask, z, kappa)[0])
+    scale = kappa * (v[0, 0].float().square().sum(1) / d).sqrt() * (mask == 0)
+    p = torch.softmax(q[0].reshape(-1, d).double() @ k[0, 0].double().T / d ** 0.5, 1)
+    want = sum(float((p @ (scale[:, None] * z[m, 0, 0].float()).bfloat16().double()).bfloat16().double().square().sum())
+               for m in range(M)) / M
+    assert abs(got / want - 1) <= 5e-6, got / want - 1

@@ -91,7 +91,7 @@ def _unordered(items, stages, releasers):
     return bad
 
 
-@pytest.mark.parametrize("stages", (5, 9))
+@pytest.mark.parametrize("stages", (5,))
 @pytest.mark.parametrize("items", ITEMS)
 def test_copies_follow_the_reads_of_their_slot(items, stages):
     assert not _unordered(items, stages, _releasers())
