@@ -1,10 +1,11 @@
 """Scoring units split over a cluster of two CTAs against the oracle and one CTA.
 
 The library takes two CTAs per unit when that trims the last wave of units, so
-the cases have a little more than one wave of units on a 152-SM GPU: 160 units
-(20 layers x 8 KV heads) of an odd number of key tiles, the last one ragged, and
-of a few tiles. The bar is the 1e-3 of tests/parity.py for bf16 scores; the split
-itself only adds a rounding of each row's log2-sum-exp, so 1e-5 is asked for.
+the cases have a little more than one wave of units on a 152-SM GPU (160 units, 20
+layers x 8 KV heads) or half a wave (72), of odd and even numbers of key tiles,
+the last one ragged; each asserts that the launch is split. The bar is the 1e-3 of
+tests/parity.py for bf16 scores; the split itself only adds a rounding of each
+row's log2-sum-exp, so 1e-5 is asked for.
 """
 
 import ctypes
@@ -33,10 +34,11 @@ def _ctas(units, tiles):
     return lib.conduit_test_score_ctas(units, tiles, torch.cuda.get_device_properties(0).multi_processor_count)
 
 
-@pytest.mark.parametrize("n,nq,d,extra", [(3713, 4, 128, False), (3713, 40, 128, True), (2049, 3, 64, False),
-                                          (2900, 5, 128, False)])
-def test_split_units(C, n, nq, d, extra):
-    L, hq, hkv = 20, 16, 8
+@pytest.mark.parametrize("n,nq,d,extra,L", [(3713, 4, 128, False, 20), (3713, 40, 128, True, 20), (2900, 5, 128, False, 20),
+                                            (2900, 3, 64, False, 9), (2900, 40, 40, True, 9), (2049, 3, 64, False, 9)])
+def test_split_units(C, n, nq, d, extra, L):
+    hq, hkv = 16, 8
+    assert _ctas(L * hkv, -(-n // 128)) == 2
     gen = torch.Generator(device="cuda").manual_seed(n + nq)
     draw = lambda *shape: torch.randn(shape, generator=gen, device="cuda").bfloat16()
     k, v, q = draw(L, hkv, n, d), draw(L, hkv, n, d), draw(L, hq, nq, d)
