@@ -481,7 +481,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int ksteps = (a.kv.d + 15) / 16;  // 16-dim steps that are not all padding
     for (int u = unit0; u < a.n_units && ok; u += unit_step) {
       Unit w;
-      if (!decode_unit(a, u, w, rank, ctas) || w.tiles == 0) continue;
+      if (!decode_unit(a, u, w, rank, ctas) || (kPair && w.tiles == 0)) continue;
       if (!wait_or_abort(s.qready, useq & 1, s.abort)) {
         if (!*s.abort) raise_abort(a, s, tc::kSiteMma);
         break;
@@ -555,7 +555,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       Unit w;
       if (!decode_unit(a, u, w, rank, ctas)) continue;
       const int nrb = (w.rows + 127) / 128;
-      if (w.tiles > 0) {
+      if (!kPair || w.tiles > 0) {
         // A CTA of a pair has no tiles in a unit of one tile. Nothing then waits for
         // the MMA thread, so an arrival there could come a phase before that thread
         // has seen the last one: neither role counts such a unit's rows.
@@ -624,7 +624,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       {
         const int row = (do_rows ? rb : 1) * 128 + lrow;
         const bool has = do_rows && row < w.rows;
-        float lse = w.tiles > 0 ? m * a.scale_log2 + log2f(z) : -INFINITY;
+        float lse = !kPair || w.tiles > 0 ? m * a.scale_log2 + log2f(z) : -INFINITY;
         if (ctas > 1) {
           // The two CTAs hold each row's sum over their own keys: each writes
           // its into the other. (The buffers alternate by unit: the peer writes
