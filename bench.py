@@ -220,7 +220,8 @@ def call_kernels(pipe) -> dict:
     """
     tc = pipe.kv.k.dtype == torch.bfloat16 and pipe.kv.head_dim <= 128
     n_tot = int(pipe.batch.tok_off[-1])
-    tail = ["finalize_warps_kernel" if n_tot >= 98304 else "finalize_tokens_kernel", "image_means_kernel"]
+    warps = n_tot >= 98304 and n_tot * pipe.kv.num_layers >= 1500000
+    tail = ["finalize_warps_kernel" if warps else "finalize_tokens_kernel", "image_means_kernel"]
     if tc:  # hbm or tensor: run_conduit keeps whichever ideal time is longer for the workload
         score = (["score_tc_kernel"] + tail, "hbm", "score_tc.cu")
         refresh = (["one_refresh_tc_kernel or refresh_tc_kernel"], "tensor", "refresh_tc.cu")

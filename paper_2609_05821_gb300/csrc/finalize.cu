@@ -20,9 +20,11 @@ __global__ void __launch_bounds__(1024) finalize_tokens_kernel(TokenReduceArgs f
 // alone with all partials of a layer in flight: no barrier and no part of a warp's
 // life without loads, where a block of the kernel above spends most of its time
 // before its first and after its last load. It needs enough tokens for its warps to
-// cover the loads' latency: with the scoring, 8 192 tokens 251 us (blocks) / 288
-// (warps), 32 768 870 / 890, 65 536 949 / 946, batched serving (131 072) 4 752 /
-// 4 645, where the blocks take 235 us for 411 MB of partials.
+// cover the loads' latency, and layers enough that they matter. With the scoring, us
+// in blocks / warps: 28 layers, 28/4 heads 8 192 tokens 251 / 288, 32 768 870 / 890,
+// 65 536 1 008 / 1 004, 98 304 1 511 / 1 498, 131 072 2 028 / 1 995, batched serving
+// 4 752 / 4 645, where the blocks take 235 us for 411 MB of partials; 8 layers, 32/8
+// heads 98 304 816 / 820, 131 072 972 / 974.
 constexpr int kWarpsPerBlock = 4;
 
 __global__ void __launch_bounds__(32 * kWarpsPerBlock, 8) finalize_warps_kernel(TokenReduceArgs f,
@@ -102,7 +104,8 @@ __global__ void __launch_bounds__(kMeanThreads) image_means_kernel(const float* 
                    [] { __syncthreads(); });
 }
 
-constexpr int64_t kWarpTokens = 98304;  // finalize_warps_kernel from here on
+// finalize_warps_kernel from so many tokens, and tokens times layers, on
+constexpr int64_t kWarpTokens = 98304, kWarpWork = 1500000;
 
 }  // namespace
 
@@ -114,7 +117,7 @@ cudaError_t launch_finalize(const float* pa, const float* pa2, const float* ss, 
   const TokenReduceArgs f{pa, pa2, ss, vnorm, vmode, n_layers, Hkv, Hq, rg_max, group_rows, parts,
                           n_tot, s, attn_sum, status};
   const unsigned groups = unsigned((n_tot + kTokBlock - 1) / kTokBlock);
-  if (n_tot >= kWarpTokens)
+  if (n_tot >= kWarpTokens && n_tot * n_layers >= kWarpWork)
     finalize_warps_kernel<<<(groups + kWarpsPerBlock - 1) / kWarpsPerBlock, 32 * kWarpsPerBlock, 0, stream>>>(f, layers,
                                                                                                              b);
   else
