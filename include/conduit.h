@@ -74,7 +74,8 @@ enum { CONDUIT_F32 = 0, CONDUIT_BF16 = 1 };
  *  paged (page_size > 0): k, v are pools [L][P][Hkv][page_size][d];
  *    request r's token t lives in physical page
  *    page_table[r * max_pages_per_req + t / page_size] at row t % page_size.
- * k and v are 16-byte aligned device pointers of dtype `dtype`.
+ * k and v are 16-byte aligned device pointers of dtype `dtype`. Rows of a page
+ * that no token has may hold anything; they reach no result.
  */
 typedef struct conduit_kv {
   int32_t num_layers;        /* L */
@@ -144,7 +145,10 @@ int32_t conduit_budget(double r, int64_t n_vis);
  *  g         device fp32 [K]
  *  workspace device, 256-byte aligned, conduit_score_workspace_size bytes
  *  status    device int32 status word or NULL (NONFINITE if a score is NaN/Inf)
- * Results are deterministic: the same inputs give bitwise-equal outputs.
+ * Results are deterministic: the same inputs give bitwise-equal outputs. How
+ * the work is split goes by the whole batch, so a request's s, A and g may
+ * differ in their last bits with the other requests of its batch (and the
+ * order of scores that near each other with them).
  */
 conduit_status conduit_score_workspace_size(const conduit_kv* kv, const conduit_batch* batch,
                                             int32_t n_layers, size_t* bytes);
@@ -408,7 +412,11 @@ conduit_status conduit_kv_exchange(const conduit_kv* kv, const conduit_batch* ba
  * position p_i = idx_i and query head h,
  *   out[l][i][h] = sum_{j <= p_i} softmax_j(<q_rows[l][i][h], K'[l][h/G][j]> / sqrt(d)) V'[l][h/G][j]
  * where K', V' are the cache after conduit_kv_scatter (call it first).
- * Softmax and accumulation in fp32; out is written in the cache dtype.
+ * Softmax and accumulation in fp32; out is written in the cache dtype. A V that
+ * is not finite counts from its own position on. The exceptions are bf16 caches
+ * with head_dim 128, and rows that see more than 131 072 keys of smaller bf16
+ * heads: there it may also make rows before it NaN that share its 128-key tile
+ * or one of the kernel's query tiles with later rows.
  *  q_rows, out  device [L][idx_off[R]][Hq][d], dtype of kv
  *  idx must be ascending within each request (conduit_select_topk's order).
  *  workspace    device, 256-byte aligned, conduit_refresh_workspace_size

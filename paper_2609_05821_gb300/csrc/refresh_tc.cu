@@ -54,13 +54,20 @@
 // never masked: as fully masked rows they sent their warps down the masking
 // path in every key tile (28 heads, 8 192 tokens: 1 254 -> 970 us).
 //
-// Measured (GB300, SM clock 2 070 MHz, before -> now): multi-image prompt 1 254
-// -> 891 us, batched serving 22.6 -> 18.5 ms, long document 15.3 -> 15.0 ms
-// (19.0 -> 18.0 ms back to back, under the power cap), single image 45.3 -> 42.5
-// us, 16 layers of 4 096 tokens 225 -> 196 us, 2 layers of 1 885 25.2 -> 20.6 us.
+// Rows past a request's last key (the next request's, or a page's rows without a
+// token) reach no output: the two-tile kernel's V warp clears them in the last tile,
+// the other's P V warp in its last 16-key step, leaving out the steps behind it. A V
+// that is not finite at a later position of the same request is kept out of earlier
+// rows below 128 dims (redo_rows); at 128 dims it makes rows of its item NaN.
 //
-// The staleness estimator (kStale) runs the same schedule with every scoring row
-// of a request at its last key: V is the draw z itself, the softmax warps scale
+// Measured (GB300, the kernel before and this one timed in turn, back to back):
+// multi-image prompt 1 413 -> 1 036 us (at the power limit; 1 254 -> 891 one call at a
+// time), batched serving 23.2 -> 19.5 ms, long document 18.6 -> 17.5 ms, single image
+// 43.5 -> 38.2 us, 16 layers of 4 096 tokens 225 -> 196 us, 2 layers of 1 885 25.2 ->
+// 20.6 us.
+//
+// The staleness estimator (kStale, 128 dims) runs the same schedule with every scoring
+// row of a request at its last key: V is the draw z itself, the softmax warps scale
 // each V tile by its keys' standard deviations in shared memory while they would
 // wait for their next S (in place of a pass that writes xi = scale z to memory),
 // and a row ends as ||O / rowsum||^2, summed over its warp's rows, instead of an

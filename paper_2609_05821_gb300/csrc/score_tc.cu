@@ -776,7 +776,9 @@ int score_tc_groups(int rows) { return n_groups(rows); }
 // of units; with few units per SM that wave is most of the run. Multi-image, 224
 // units of 64 tiles on 152 SMs: 311 us with one CTA, 252 us with two; batched
 // serving, 27 waves, 4.91 against 4.96 ms; long document, 288 units of 324 tiles,
-// 1 331 against 1 345 us. Four CTAs reach only 144 SMs, eight 120.
+// 1 331 against 1 345 us. Four CTAs reach only 144 SMs, eight 120. The choice is the
+// launch's, and the pair's log2-sum-exp has a rounding more: the last bits of a
+// request's results may differ with what else is in its batch.
 static int ctas_per_unit(int units, int tiles, int sms) {
   const int pairs = sms / 2;
   if (pairs == 0 || tiles < 16) return 1;  // short units: the fixed share is most of them

@@ -467,7 +467,7 @@ __global__ void __launch_bounds__(kSelThreads) finalize_select_kernel(
 // Requests too large for one CTA's registers (more than 8 x 1024 tokens) take
 // a cluster of kClusterCtas CTAs: CTA c of the cluster owns the c-th
 // contiguous chunk of the request's tokens and keeps its keys in registers.
-// Each radix pass builds a 256-bin histogram per CTA in shared memory; after a
+// Each radix pass builds a 512-bin histogram per CTA in shared memory; after a
 // cluster barrier every CTA sums the kClusterCtas histograms through
 // distributed shared memory and takes the same digit decision. The selected
 // indices go out in ascending order: each CTA's count of keys above the k-th
