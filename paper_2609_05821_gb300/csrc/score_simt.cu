@@ -84,10 +84,11 @@ __global__ void __launch_bounds__(kThreads) rowstats_kernel(KvDev kv, BatchDev b
         tmax = fmaxf(tmax, x[a][m]);
       }
       const float m_new = fmaxf(m_run[a], lanes_max(tmax));
+      const float ref = m_new == -INFINITY ? 0.f : m_new;  // a chunk of masked keys: its sum is 0
       float psum = 0.f;
 #pragma unroll
-      for (int m = 0; m < 4; ++m) psum += exp2f(x[a][m] - m_new);
-      z_run[a] = z_run[a] * exp2f(m_run[a] - m_new) + lanes_sum(psum);
+      for (int m = 0; m < 4; ++m) psum += exp2f(x[a][m] - ref);
+      z_run[a] = z_run[a] * exp2f(m_run[a] - ref) + lanes_sum(psum);
       m_run[a] = m_new;
     }
   }

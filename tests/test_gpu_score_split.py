@@ -122,3 +122,27 @@ def test_keys_of_no_token_reach_no_score(C, d, nq, form):
     assert torch.isfinite(clean[0]).all()
     for a, b, n in zip(got, clean, (end, end, 2 if form == "paged" else 1)):
         assert torch.equal(a[:n], b[:n])
+
+
+@pytest.mark.parametrize("dtype,d", [(torch.float32, 64), (torch.float32, 128), (torch.float32, 256), (torch.bfloat16, 64),
+                                     (torch.bfloat16, 128), (torch.bfloat16, 136)])
+@pytest.mark.parametrize("lo,hi", [(70, 330), (0, 330), (200, 3000)])
+def test_masked_keys(C, dtype, d, lo, hi):
+    """Keys whose logits overflow to -inf get no weight, also where they fill a chunk of keys or a CTA's share of them."""
+    L, hq, hkv, n, nq = 1, 4, 2, 400 if hi < 400 else 3000, 5
+    gen = torch.Generator(device="cuda").manual_seed(d)
+    draw = lambda *shape: torch.randn(shape, generator=gen, device="cuda").to(dtype)
+    k, v, q = draw(L, hkv, n, d), draw(L, hkv, n, d), draw(L, hq, nq, d)
+    q[..., 0] = 32.0
+    k[..., 0] = 0.0
+    k[:, :, lo:hi, 0] = torch.finfo(dtype).min
+    batch = C.Batch([0, n], [0, n], [0, 1], [0, nq], device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    s, A, _ = C.conduit_score(C.KvCache(k, v, hq), batch, q, status=status)
+    assert C.conduit_read_status(status) == C.OK
+    x = torch.einsum("lhqd,lhtd->lhqt", q.double(), k.double().repeat_interleave(hq // hkv, 1)) / d ** 0.5
+    a = torch.softmax(x, -1).mean((1, 2))[0]
+    norm = v.double().square().sum((1, 3)).sqrt()[0]
+    assert torch.all(s[lo:hi] == 0) and torch.all(A[lo:hi] == 0)
+    for got, want in ((A, a), (s, a * norm)):
+        assert torch.all((got - want).abs() <= 1e-5 * want + 1e-7 * want.max())
