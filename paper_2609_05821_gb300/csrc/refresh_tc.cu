@@ -1358,7 +1358,8 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
       if (fin) {
         tc::tc_fence_after();
-        const float inv = total > 0.f ? 1.f / total : 0.f;
+        // no weight at all (every logit -inf): NaN below 128 dims, as on CUDA cores
+        const float inv = total > 0.f ? 1.f / total : kSplit ? NAN : 0.f;
         const int64_t row_off = ((int64_t(it.l) * a.n_sel + i_row) * Hq + h_row) * d;
         __nv_bfloat16* dst = a.out + row_off;
         float zero = 0.f;  // NaN where a value is not finite

@@ -225,3 +225,26 @@ def test_non_finite_values_reach_the_rows_that_see_them(C, d, form):
             assert torch.equal(fine, torch.isfinite(x)) and torch.equal(torch.isnan(want), torch.isnan(x)), (p, h)
             assert torch.equal(want[torch.isinf(want)], x[torch.isinf(want)]), (p, h)
             assert torch.all((x - want).abs()[fine] <= 2e-2 + 2.0 ** -8 * want.abs()[fine]), (p, h)
+
+
+@pytest.mark.parametrize("dtype,d", [(torch.float32, 64), (torch.float32, 128), (torch.bfloat16, 64), (torch.bfloat16, 96),
+                                     (torch.bfloat16, 136)])
+def test_masked_keys_get_no_weight(C, dtype, d):
+    """Keys whose logits overflow to -inf: a row that sees others gives them no weight, a row that sees no other is NaN."""
+    n, hq, hkv = 300, 4, 2
+    gen = torch.Generator(device="cuda").manual_seed(d)
+    draw = lambda *shape: torch.randn(shape, generator=gen, device="cuda").to(dtype)
+    k, v, q_rows = draw(1, hkv, n, d), draw(1, hkv, n, d), draw(1, 4, hq, d)
+    q_rows[..., 0], k[..., 0] = 32.0, 0.0
+    k[:, :, :40, 0] = k[:, :, 128:290, 0] = torch.finfo(dtype).min
+    batch = C.Batch([0, n], [0, n], [0, 1], [0, 1], device="cuda")
+    off, off_dev = C.idx_offsets([4])
+    idx = torch.tensor([20, 90, 270, 299], dtype=torch.int32, device="cuda")
+    got = C.conduit_refresh_attn(C.KvCache(k, v, hq), batch, idx, off, off_dev, q_rows).double()
+    assert torch.isnan(got[:, 0]).all()
+    for i, p in ((1, 90), (2, 270), (3, 299)):
+        for h in range(hq):
+            x = k[0, h // 2, :p + 1].double() @ q_rows[0, i, h].double() / d ** 0.5
+            want = torch.softmax(x, 0) @ v[0, h // 2, :p + 1].double()
+            bar = 1e-6 + 1e-5 * want.abs() if dtype == torch.float32 else 2e-2 + 2.0 ** -8 * want.abs()
+            assert torch.all((got[0, i, h] - want).abs() <= bar), (p, h)
